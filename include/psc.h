@@ -125,8 +125,8 @@ typedef struct {
     int32_t blocks_per_sm;    /* resident blocks per SM for grid sizing (8)     */
     int32_t collect_stats;    /* 1 = count attempts/hops/... (default 0), -1 off */
     int32_t graph_events;     /* >= 2: runs of this many events that take
-                                 per-event launches (species with reactions,
-                                 or persistent = -1) are captured in a CUDA
+                                 per-event launches (species with reactions
+                                 and long lists, or persistent = -1) are captured in a CUDA
                                  graph the second time their pattern (species
                                  in order, claim-table state, re-sort
                                  counters) comes up and replayed from then
@@ -142,9 +142,14 @@ typedef struct {
                                  2 = hash table of claims, 0/-1 = by size (a
                                  word per voxel up to 2^22 voxels, or where
                                  the two tables would be as large)             */
-    int32_t persistent;       /* 1 = run stretches of events of a species without
-                                 reactions in one cooperative launch (default),
-                                 -1 = one claim + commit launch per event       */
+    int32_t persistent;       /* 1 = run stretches of events in one launch
+                                 (default): of a species without reactions, and
+                                 of any species, in scheduler order, where the
+                                 lists are short (up to 131,072 molecules, with
+                                 reactions 300,000, partners included; not while
+                                 time_kernels is on for those with reactions)
+                                 and claims have a word per voxel;
+                                 -1 = claim and commit launches per event       */
     int32_t slot_map;         /* home slot of a claim in the hash table:
                                  1 = hashed voxel index (default), 2 = Morton
                                  order, 3 = Morton with permuted low bits      */

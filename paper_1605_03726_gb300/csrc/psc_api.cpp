@@ -252,6 +252,7 @@ void span_close(psc_lattice* L, cudaEvent_t a, int kind, int64_t events = 1)
 
 int resort(psc_lattice* L, int s)
 {
+    L->small.map_holds = false;
     const int blocks = list_blocks(L, s);
     const SpeciesList& list = L->model_h.lists[s];
     const int32_t* count = &L->sc->counts[s];
@@ -291,6 +292,7 @@ ReconcileArgs reconcile_args(const psc_lattice* L, int x)
 
 int enqueue_event(psc_lattice* L, int s)
 {
+    L->small.map_holds = false;
     const EventArgs a = event_args(L, s);
     const int threads = L->opt.block_threads;
     const int blocks = list_blocks(L, s);
@@ -656,6 +658,167 @@ int enqueue_subvol(psc_lattice* L, int s, int64_t n_events)
     return PSC_OK;
 }
 
+// What a stretch of k_small_run may take on the lattice's device: asked of the
+// device once (it does not change).
+static void small_shapes(psc_lattice* L)
+{
+    static std::mutex mu;
+    static int cluster[64], grid[64];
+    static bool known[64];
+    std::lock_guard<std::mutex> lk(mu);
+    auto& B = L->small;
+    const int d = L->device;
+    if (d < 64 && known[d]) {
+        B.cluster = cluster[d];
+        B.grid = grid[d];
+    } else {
+        small_limits(L->sm_count, &B.cluster, &B.grid);
+        if (d < 64) {
+            cluster[d] = B.cluster;
+            grid[d] = B.grid;
+            known[d] = true;
+        }
+    }
+    B.asked = true;
+}
+
+// Set-up of the first stretch: which species react, have partners, make what;
+// the argument templates.
+static int small_setup(psc_lattice* L)
+{
+    auto& B = L->small;
+    for (int s = 0; s < L->nsp; ++s) {
+        if (L->general[s]) B.general |= 1u << s;
+        if (L->fo2[s]) B.fo2 |= 1u << s;
+        auto products = [&](const Reaction& R) {
+            for (int q = 0; q < R.np; ++q) B.products[s] |= 1u << R.p[q];
+        };
+        for (int x = 0; x < L->nsp; ++x) {
+            if (L->pair[s][x] < 0) continue;
+            B.mapped |= 1u << s;
+            products(L->rx[L->pair[s][x]]);
+        }
+        for (int u = 0; u < L->sp[s].n_fo; ++u) products(L->rx[L->sp[s].fo[u]]);
+    }
+    std::vector<EventArgs> ev((size_t)L->nsp);
+    for (int s = 0; s < L->nsp; ++s) ev[(size_t)s] = event_args(L, s);
+    EventArgs* d = (EventArgs*)dev_alloc(L, sizeof(EventArgs) * ev.size());
+    if (!d) return PSC_E_NOMEM;
+    // (from pageable memory: the copy has left it when the call returns)
+    const int rc = cuda_fail(L, cudaMemcpyAsync(d, ev.data(), sizeof(EventArgs) * ev.size(), cudaMemcpyHostToDevice,
+                                                L->stream));
+    if (rc) return rc;
+    L->h2d += sizeof(EventArgs) * ev.size();
+    B.ev = d;
+    return PSC_OK;
+}
+
+// Can an event of species s run in a stretch of k_small_run?  Its own list and
+// its partners' hold at most kSmallList entries (by the estimates: a list that
+// has grown past it in the meantime only takes longer).
+static bool small_fits(psc_lattice* L, int s)
+{
+    if (!L->claim || L->opt.persistent <= 0 || L->opt.barrier_phantom > 0) return false;
+    if (!L->small.asked) small_shapes(L);
+    if (L->small.cluster <= 0 || L->small.grid <= 0) return false;
+    if (L->general[s]) {
+        // kernel timing keeps the phases of a reaction event apart; without the background
+        // copies of the list lengths nothing is known of them
+        if (L->opt.time_kernels > 0 || !L->counts_h) return false;
+        for (int x : L->reconcile[s])
+            if (L->est[x] > kSmallList) return false;
+        return true;
+    }
+    if (L->opt.run_per_thread > 0) return false;     // the caller picks the molecule-list kernel's shape
+    if (L->est[s] > kSmallWalk) return false;
+    TilePlan P{};
+    return !(L->opt.tiles > 0 && tile_plan(L, s, &P));
+}
+
+// A stretch of consecutive events, starting with species s at time t: one
+// launch.  *n = events queued.
+static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
+{
+    auto& B = L->small;
+    if (!B.ev) {
+        const int rc = small_setup(L);
+        if (rc) return rc;
+    }
+    bool lists = false;                              // a species with reactions may come up
+    for (int x = 0; x < L->nsp && !lists; ++x) lists = L->general[x] && L->sp[x].D > 0.0 && small_fits(L, x);
+    if (lists && B.mapped && !B.slot) {
+        B.slot = (uint32_t*)dev_alloc(L, (size_t)L->V * 4);
+        if (!B.slot) return PSC_E_NOMEM;
+    }
+    bool lists_long = false;                         // a stretch may take a grid
+    for (int x = 0; lists && x < L->nsp && !lists_long; ++x)
+        lists_long = L->sp[x].D > 0.0 && L->est[x] > kSmallCluster && small_fits(L, x);
+    if (lists_long && !B.scratch) {                  // closing lists up in a grid
+        int64_t most = 0;
+        for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, L->model_h.lists[x].cap);
+        B.scratch_n = (int32_t)std::min<int64_t>(4 * kSmallList, 4 * most + 4096);
+        B.scratch = (int32_t*)dev_alloc(L, (size_t)B.scratch_n * 8);
+        if (!B.scratch) return PSC_E_NOMEM;
+    }
+    SmallArgs A{};
+    A.ev = B.ev;
+    A.model = L->model_d;
+    A.sc = L->sc;
+    A.slot = B.slot;
+    A.holes = B.scratch;
+    A.surv = B.scratch + B.scratch_n;
+    A.scratch_n = B.scratch_n;
+    A.barrier = L->barrier;
+    A.barrier_timeout_ns = (uint64_t)L->opt.barrier_timeout_us * 1000ull;
+    A.g = L->g;
+    A.nsp = L->nsp;
+    A.collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
+    const int64_t limit = std::min<int64_t>(std::min<int64_t>(max_events, kSmallEvents),
+                                            (int64_t)UINT32_MAX - L->g);
+    int8_t fits[kMaxSpecies] = {};                   // 0 not asked yet, 1 yes, -1 no
+    fits[s] = 1;
+    int64_t longest = 0;
+    bool reacts = false;
+    for (;;) {
+        A.seq[A.n_events++] = (uint8_t)s;
+        longest = std::max(longest, L->est[s]);
+        reacts = reacts || L->general[s];
+        L->sp[s].done++;
+        L->g++;
+        L->clock = t;
+        if (A.n_events >= limit || !next_event(L, &s, &t) || t > t_end) break;
+        if (fits[s] == 0) fits[s] = small_fits(L, s) ? 1 : -1;
+        if (fits[s] < 0) break;
+    }
+    if (reacts) {
+        A.general = B.general;
+        A.fo2 = B.fo2;
+        A.mapped = B.mapped;
+        std::memcpy(A.products, B.products, sizeof(A.products));
+        A.build_map = B.map_holds ? 0 : 1;
+        B.map_holds = true;
+    }
+    // the shape: a cluster of 16 blocks up to kSmallCluster entries (with fewer
+    // blocks, or 128 threads in each, short lists got slower: 2621 walkers 3.9 us
+    // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM,
+    // of half the threads while they suffice (45,000 molecules 7.8 us per event
+    // against 8.2), and two per SM for the longest
+    const bool cluster = longest <= kSmallCluster;
+    const int threads = !cluster && longest <= 65536 ? kSmallThreads / 2 : kSmallThreads;
+    const int blocks = cluster ? B.cluster : std::min(B.grid, longest <= 131072 ? L->sm_count : 2 * L->sm_count);
+    int rc = PSC_OK;
+    if (!cluster) rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream));
+    if (rc) return rc;
+    cudaEvent_t sp = span_open(L);
+    rc = cuda_fail(L, launch_small(A, blocks, threads, cluster, L->stream));
+    span_close(L, sp, kSpanRun, A.n_events);
+    if (rc) return rc;
+    L->launches += 1;
+    L->events += (uint64_t)A.n_events;
+    *n = A.n_events;
+    return PSC_OK;
+}
+
 // Sec. 2.2: the next event belongs to the mobile species whose next diffusion
 // time (events done + 1) * tau is earliest; ties go to the lower index.
 bool next_event(const psc_lattice* L, int* s_out, double* t_out)
@@ -967,6 +1130,9 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         max_cap = std::max(max_cap, c);
         if (L->sp[s].D > 0.0) max_mobile = std::max(max_mobile, c);
     }
+    // lists of products that are not sized for the lattice keep room for the
+    // tombstones of k_small_run
+    L->list_slack = growth || !L->stretches ? 0 : std::min<int64_t>(2 * N, 262144);
     bool any_fo2 = false;
     for (int s = 0; s < L->nsp; ++s) any_fo2 = any_fo2 || L->fo2[s];
 
@@ -1027,7 +1193,7 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         M.comp[s] = (uint8_t)(comps ? L->sp[s].comp : 0);
         M.mirror[s] = L->bits + (size_t)M.comp[s] * nwords;
         SpeciesList& l = M.lists[s];
-        l.cap = L->cap[s];
+        l.cap = L->cap[s] + (is_product[s] ? (int32_t)L->list_slack : 0);
         l.vox = (int32_t*)dev_alloc(L, (size_t)l.cap * 4);
         l.ids = (uint32_t*)dev_alloc(L, (size_t)l.cap * 4);
         l.img = (uint64_t*)dev_alloc(L, (size_t)l.cap * 8);
@@ -1282,6 +1448,7 @@ static int single_event(psc_lattice* L, int s, double t)
     for (const auto& G : L->graphs1) {
         if (G.key != key) continue;
         set_index();
+        L->small.map_holds = false;
         int rc = cuda_fail(L, cudaGraphLaunch(G.exec, L->stream));
         if (rc) return rc;
         L->table_used[0] = G.table_used[0];
@@ -1413,6 +1580,7 @@ static int graph_run(psc_lattice* L, double t_end, int64_t room, int64_t* done)
         if (G.key != key) continue;
         launch_fill_u32(&L->sc->g_base, L->g, 1, 1, L->stream);
         L->g_dev = (int64_t)L->g;
+        L->small.map_holds = false;
         int rc = cuda_fail(L, cudaGraphLaunch(G.exec, L->stream));
         if (rc) return rc;
         for (int e = 0; e < K; ++e) advance(e);
@@ -1529,6 +1697,13 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             L->g = g0;
             int rc = enqueue_subvol(L, s, e);
             L->g = g0 + (uint32_t)e;
+            if (rc) return rc;
+            queued += e;
+            continue;
+        }
+        if (small_fits(L, s)) {
+            int64_t e = 0;
+            int rc = small_stretch(L, s, t, t_end, max_events - queued, &e);
             if (rc) return rc;
             queued += e;
             continue;
@@ -1946,6 +2121,9 @@ int psc_device_bytes(const psc_lattice* L, int64_t* bytes)
     const int64_t mwords = (int64_t)mirror_words(L->ni, L->nj, L->nk);
     int64_t b = L->V * 2 + mwords * 4 * mirrors + 2 * ((mwords + 31) / 32) * 4 + (int64_t)sizeof(Scalars) +
                 (int64_t)sizeof(ModelDev);
+    if (L->small.ev) b += (int64_t)L->nsp * (int64_t)sizeof(EventArgs);
+    if (L->small.slot) b += L->V * 4;
+    b += (int64_t)L->small.scratch_n * 8;
     if (L->claim) b += L->V * 4;
     b += 2 * L->table_slots * 8;
     int64_t N = 0;
@@ -1953,7 +2131,7 @@ int psc_device_bytes(const psc_lattice* L, int64_t* bytes)
     if (L->populated) {
         int64_t mx = 1, mm = 1;
         for (int s = 0; s < L->nsp; ++s) {
-            b += (int64_t)L->cap[s] * 16;
+            b += (int64_t)L->model_h.lists[s].cap * 16;
             mx = std::max<int64_t>(mx, L->cap[s]);
             if (L->sp[s].D > 0.0) mm = std::max<int64_t>(mm, L->cap[s]);
         }

@@ -162,6 +162,7 @@ int batch_event(psc_batch* B, double t_cap, int* rc_out)
     }
     for (int a = 0; a < na; ++a) {
         psc_lattice* L = B->slot[acts[a].slot].L;
+        L->small.map_holds = false;
         L->sp[acts[a].s].done++;
         L->g++;
         L->clock = acts[a].t;
@@ -437,6 +438,7 @@ int build_lattice(const Request& q, int device, cudaStream_t stream, psc_lattice
     o.claim_table = 1;
     o.resort_period = -1;
     psc_set_options(L, &o);
+    L->stretches = false;                            // the batch runs its events
     for (int s = 0; s < r.n_species && !rc; ++s) rc = psc_add_species(L, q.D[s], q.n0[s], nullptr);
     for (int x = 0; x < r.n_reactions && !rc; ++x)
         rc = psc_add_reaction(L, &q.re[2 * x], q.nre[x], &q.pr[2 * x], q.npr[x], q.k[x], nullptr);

@@ -109,6 +109,8 @@ struct Scalars {
     int32_t births;                  // births queued in the current event
     int32_t err;                     // kErr* bits
     uint32_t g_base;                 // index of the first event of a replayed graph
+    uint32_t touched[2];             // by event parity, in k_small_run: the event had births
+    int32_t hole_n[kMaxSpecies], surv_n[kMaxSpecies];   // while k_small_run closes its lists up
     unsigned long long stats[kNumStats];
 };
 
@@ -257,6 +259,42 @@ struct ReconcileArgs {
     uint32_t* g_bump;          // null, or the word the event's last launch sets to its index + 1
 };
 
+// A stretch of events, of any species in scheduler order, of a lattice with
+// per-voxel claim words (k_small_run).
+constexpr int kSmallEvents = 512;          // events of one launch
+constexpr int kSmallThreads = 512;         // threads of a block
+// The longest list of a stretch.  With reactions (30 % crowding): 205,000
+// molecules take 16.5 us per event against 24.9 in per-event launches, 400,000
+// 26 to 29 against 30, and 839,000 57 against 42 (twice the threads in flight
+// there, and Morton re-sorts).  Without (128^3): 63,000 walkers 8.4 against
+// 10.8 in the molecule-list kernel, 210,000 14.4 against 13.0.
+constexpr int64_t kSmallList = 300000;     // of a species with reactions, or a partner
+constexpr int64_t kSmallWalk = 131072;     // of one without
+// The longest list that runs in one cluster of 16 blocks: 16,000 molecules take
+// 3.6 us per event there and 4.8 in a grid, 30,000 13.1 and 7.8.
+constexpr int64_t kSmallCluster = 16384;
+struct SmallArgs {
+    const EventArgs* ev;       // [nsp] templates on the device (event_args with g unset)
+    const ModelDev* model;
+    Scalars* sc;
+    uint32_t* slot;            // per voxel: the list slot of its molecule, for species in `mapped`
+    int32_t* holes;            // [scratch_n] slots of tombstones and of the entries that take them
+    int32_t* surv;
+    int32_t scratch_n;
+    BarrierState* barrier;
+    uint64_t barrier_timeout_ns;
+    uint32_t g;                // index of the first event
+    int32_t n_events;
+    int32_t nsp;
+    int32_t collect_stats;
+    int32_t build_map;         // the map has to be built first
+    uint32_t general;          // bit s: species s has reactions
+    uint32_t fo2;              // bit s: a first-order reaction of s has two products
+    uint32_t mapped;           // bit s: s can be a second-order partner
+    uint32_t products[kMaxSpecies];        // bit y: an event of s may append to list y
+    uint8_t seq[kSmallEvents]; // species of each event
+};
+
 // ---- launchers (psc_kernels.cu) ----
 void upload_stencil(cudaStream_t st);
 void launch_claim(const EventArgs& a, bool general, int blocks, int threads, cudaStream_t st);
@@ -347,6 +385,10 @@ struct ListFill {
 };
 void launch_fill(const ListFill& f, cudaStream_t st);
 void launch_births(const EventArgs& a, cudaStream_t st);
+// Most blocks of a stretch on the current device: as one cluster, as a
+// cooperative grid (0: not at all).  Sets the kernels' attributes there.
+void small_limits(int sm_count, int* cluster, int* grid);
+cudaError_t launch_small(const SmallArgs& A, int blocks, int threads, bool cluster, cudaStream_t st);
 void launch_fill_u32(uint32_t* p, uint32_t value, size_t n, int blocks, cudaStream_t st);
 // molecule r (ids in species order, species s owning [offsets[s],
 // offsets[s+1])) takes sorted_vox[starts[s] + r - offsets[s]]; its bit goes

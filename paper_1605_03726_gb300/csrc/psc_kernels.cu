@@ -1165,7 +1165,7 @@ void launch_event_one(const EventArgs& a, cudaStream_t st)
 // ---------------------------------------------------------------------------
 constexpr int kBirthSortMax = 8192;
 
-__device__ __forceinline__ void births_body(const EventArgs& a)
+__device__ __forceinline__ void births_body(const EventArgs& a, uint32_t* slot_map = nullptr, uint32_t mapped = 0u)
 {
     extern __shared__ unsigned long long keys[];
     int nb = a.sc->births;
@@ -1201,6 +1201,7 @@ __device__ __forceinline__ void births_body(const EventArgs& a)
             dst.vox[slot] = b.t;
             dst.ids[slot] = base_id + (uint32_t)x;
             dst.img[slot] = b.img;
+            if ((mapped >> b.species) & 1u) slot_map[b.t] = (uint32_t)slot;
         } else {
             atomicOr(&a.sc->err, kErrListOverflow);
         }
@@ -1622,6 +1623,7 @@ void launch_births_batch(const EventArgs* tmpl, const BatchLaunch& bl, cudaStrea
     k_births_batch<<<bl.n, 1024, smem, st>>>(tmpl, bl);
 }
 
+#include "psc_small.cuh"
 #include "psc_tiles.cuh"
 #include "psc_slab.cuh"
 #include "psc_subvol.cuh"

@@ -105,6 +105,23 @@ struct psc_lattice {
     int sticky = PSC_OK;
     std::vector<void*> allocs;
 
+    // stretches of events in one launch (k_small_run): per-species argument
+    // templates on the device, the voxel -> slot map and the scratch of closing
+    // lists up
+    struct SmallBuffers {
+        EventArgs* ev = nullptr;       // written at the first stretch
+        uint32_t* slot = nullptr;      // allocated with the first stretch that may react
+        int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
+        int32_t scratch_n = 0;
+        bool map_holds = false;        // the map agrees with the lists (nothing else has changed them since)
+        bool asked = false;            // the device was asked for the next two
+        int cluster = 0, grid = 0;     // most blocks of a stretch: one cluster, a cooperative grid
+        uint32_t general = 0, fo2 = 0, mapped = 0;
+        uint32_t products[kMaxSpecies] = {};
+    } small;
+    bool stretches = true;             // false: made for a batch, no room for tombstones is kept
+    int64_t list_slack = 0;            // entries of room for tombstones in the lists of reaction products
+
     // per-event runs replayed from CUDA graphs (psc_options.graph_events):
     // graphs by run pattern, patterns seen once, and the first event index
     // of a run being captured (-1: none)

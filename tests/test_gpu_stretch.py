@@ -1,0 +1,96 @@
+"""Stretches of events of any species in one launch (short lists): one cluster
+of blocks up to 16,384 molecules, a cooperative grid above.
+
+Compared bit for bit with the oracle where such a stretch can go wrong: lists
+on either side of the cluster's limit and crossing it, calls that end a stretch
+after 1, 2, 511 and 513 events, per-event launches in between (they change the
+lists behind the voxel -> slot map), reactions fast enough that tombstones fill
+the lists' room several times within a stretch, births, immobile partners,
+compartments, and walkers between species with reactions.
+"""
+import pytest
+
+import models
+import paper_1605_03726_gb300 as psc
+from test_gpu_parity import assert_same, build_both
+
+pytestmark = pytest.mark.gpu
+
+TAU = 6.666666666666667e-05             # hop interval at D = 1 um^2/s, r_v = 10 nm
+
+
+def flipping(L, n):
+    """A and B turn into each other, 8 % of them per event, and meet an immobile X."""
+    a = L.add_species(1e-12, n)
+    b = L.add_species(0.9e-12, n // 3)
+    x = L.add_species(0.0, n // 4)
+    L.add_reaction([a], [b], 0.08 / TAU)
+    L.add_reaction([b], [a], 0.08 / TAU)
+    L.add_reaction([a, x], [x, b], 1e-19)
+    L.add_reaction([b, x], [a, x], 1e-19)
+
+
+def splitting(L, n):
+    """A splits and recombines; C takes A away; walkers in between."""
+    a = L.add_species(1e-12, n)
+    c = L.add_species(0.7e-12, n // 2)
+    w = L.add_species(0.8e-12, n // 2)
+    L.add_reaction([a], [a, c], 0.02 / TAU)
+    L.add_reaction([a, c], [a], 5e-20)
+    assert w == 2
+
+
+CASES = [
+    ("ab_16383", (64, 64, 64), 7, lambda L: models.reaction_diffusion_ab(L, 16383, 9000), (1, 2, 511)),
+    ("ab_16385", (64, 64, 64), 7, lambda L: models.reaction_diffusion_ab(L, 16385, 16384), (1, 513)),
+    ("flip_cluster", (40, 36, 44), 7, lambda L: flipping(L, 5000), (513, 2)),
+    ("flip_grid", (72, 64, 60), 0, lambda L: flipping(L, 20000), (511, 1)),
+    ("split_cluster", (37, 41, 29), 0, lambda L: splitting(L, 700), (2, 150)),
+    ("split_grid", (60, 58, 64), 7, lambda L: splitting(L, 18000), (40, 1)),
+    ("walkers", (48, 44, 52), 6, lambda L: [L.add_species(d, n) for d, n in ((1e-12, 17000), (1e-12, 3), (0.6e-12, 900))],
+     (1, 513)),
+]
+
+
+@pytest.mark.parametrize("name,shape,boundary,recipe,calls", CASES, ids=[c[0] for c in CASES])
+def test_stretches_match_oracle(name, shape, boundary, recipe, calls):
+    g, o = build_both(shape, recipe, 11, boundary=boundary)
+    for n in calls:
+        g.run_events(n)
+        o.run_events(n)
+        assert_same(g, o, (name, n))
+    # per-event launches, then a stretch again
+    for persistent in (-1, 1):
+        g.set_options(persistent=persistent)
+        g.run_events(7)
+        o.run_events(7)
+        assert_same(g, o, (name, persistent))
+    before = g.stats()["launches"]
+    g.run_events(64)
+    assert g.stats()["launches"] - before <= 2            # one stretch, not per-event launches
+
+
+def test_stretches_count_events_as_launches_do():
+    stats = {}
+    for persistent in (1, -1):
+        L = psc.Lattice(40, 36, 44, voxel_radius=1e-8)
+        L.set_options(collect_stats=1, persistent=persistent)
+        flipping(L, 3000)
+        L.populate(5)
+        L.run_events(300)
+        stats[persistent] = L.stats()
+        L.close()
+    for k in ("attempts", "hops", "collisions", "accepted", "reactions2", "fires", "reactions1", "births", "events"):
+        assert stats[1][k] == stats[-1][k], k
+    assert stats[1]["launches"] < stats[-1]["launches"] // 10
+
+
+def test_stretch_in_a_cell_with_compartments():
+    shape = (40, 36, 32)
+    lab = models.cell_labels(*shape, radius=28.0)
+    g, o = build_both(shape, lambda L: models.receptor_binding(L, lab, 1500, 500, n_x=300, n_outside=900, koff=2e3), 4,
+                      boundary=0)
+    for n in (3, 400):
+        g.run_events(n)
+        o.run_events(n)
+        assert_same(g, o, n)
