@@ -137,18 +137,25 @@ typedef struct {
                                  lattice's stream meanwhile: a stream that
                                  other threads also feed needs -1              */
     int32_t time_kernels;     /* 1 = record CUDA events around the kernels of
-                                 every event (psc_kernel_times_get), -1 off     */
+                                 every event (psc_kernel_times_get), -1 off;
+                                 while on, events run in the kernels it tells
+                                 apart (no graphs, no stretches of lattices
+                                 without reactions or of reaction events)       */
     int32_t claim_table;      /* before populate: 1 = one claim word per voxel,
                                  2 = hash table of claims, 0/-1 = by size (a
-                                 word per voxel up to 2^22 voxels, or where
-                                 the two tables would be as large)             */
+                                 word per voxel up to 2^22 voxels, where the
+                                 two tables would be as large, or up to 28
+                                 million voxels where there are no reactions
+                                 and the molecules fit in shared memory)       */
     int32_t persistent;       /* 1 = run stretches of events in one launch
-                                 (default): of a species without reactions, and
-                                 of any species, in scheduler order, where the
-                                 lists are short (up to 131,072 molecules, with
-                                 reactions 300,000, partners included; not while
-                                 time_kernels is on for those with reactions)
-                                 and claims have a word per voxel;
+                                 (default): of a lattice without reactions and
+                                 compartments whose molecules fit in shared
+                                 memory (up to 2.8 million, 28 million voxels),
+                                 all its species in turn; of any species, in
+                                 scheduler order, where the lists are short (up
+                                 to 131,072 molecules, with reactions 300,000,
+                                 partners included) and claims have a word per
+                                 voxel; of a species without reactions otherwise;
                                  -1 = claim and commit launches per event       */
     int32_t slot_map;         /* home slot of a claim in the hash table:
                                  1 = hashed voxel index (default), 2 = Morton
@@ -170,7 +177,9 @@ typedef struct {
     int32_t tiles;            /* persistent stretches of a species without
                                  reactions: 1 = owner-computes tile kernel
                                  wherever it applies, -1 = never, 0 = default
-                                 (when the species has >= 2^18 molecules on a
+                                 (when the lattice does not run in stretches
+                                 of all its species, see persistent, and
+                                 the species has >= 2^18 molecules on a
                                  lattice of more than 2^22 voxels and,
                                  at its first stretch, the fullest box holds
                                  at most 1.4 x the mean: molecules confined

@@ -73,6 +73,7 @@ int batch_event(psc_batch* B, double t_cap, int* rc_out)
         double t;
         if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
         acts[na++] = {i, s, t};
+        if ((*rc_out = claims_free(L))) return 1;
         BatchItem& it = bl.item[bl.n++];
         it.rep = i;
         it.sel = s;

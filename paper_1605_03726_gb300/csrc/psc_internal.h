@@ -295,6 +295,44 @@ struct SmallArgs {
     uint8_t seq[kSmallEvents]; // species of each event
 };
 
+// A stretch of events of a lattice without reactions (k_walk_run): every
+// mobile species' molecules in shared memory, claim words that tell vacancy.
+constexpr int kWalkEvents = 512;           // events of one launch
+constexpr int kWalkThreads = 1024;         // threads of a block: one per SM, a cooperative grid
+constexpr int kWalkClusterThreads = 512;   // or one cluster
+constexpr int64_t kWalkCluster = 16384;    // molecules a cluster takes
+// Shorter lists run as fast in any order: 168,000 walkers on 256^3 8.4 us per
+// event either way, 629,000 on 128^3 13.7 sorted every 64 events, 15.1 unsorted.
+constexpr int64_t kWalkSorted = 200000;
+constexpr int kWalkClusterSmem = 36 * 1024;        // shared memory of its blocks, at most
+constexpr int64_t kWalkVoxels = 28000000;  // largest lattice that gets claim words for it (112 MB)
+constexpr int64_t kWalkSmem = 225 * 1024;  // shared memory of its blocks
+struct WalkArgs {
+    Geometry geo;
+    FastDiv div_nbi, div_nbij; // by the mirror's words along i, and along i and j
+    uint32_t* word;            // per voxel, in the mirror's order (word << 5 | bit): all ones vacant, else the
+                               // last claim that won it (0: occupied since the words were made)
+    uint32_t epoch;            // of the first event; claims are epoch << id_bits | id - id_lo
+    int32_t id_bits;
+    uint32_t id_lo[kMaxSpecies];
+    uint32_t* bits;            // vacancy mirror
+    Scalars* sc;
+    BarrierState* barrier;
+    uint64_t barrier_timeout_ns;
+    uint32_t barrier_phantom;
+    uint32_t key0, key1;
+    uint32_t g;                // index of the first event
+    int32_t n_events;
+    int32_t collect_stats;
+    int32_t n_species;         // mobile species with molecules
+    int32_t slots;             // molecules a thread holds at most, over all species
+    int32_t n[kMaxSpecies];    // per species: molecules, first slot, index, list
+    int32_t slot0[kMaxSpecies];
+    uint8_t species[kMaxSpecies];
+    SpeciesList list[kMaxSpecies];
+    uint8_t seq[kWalkEvents];  // species of each event (place in the arrays above)
+};
+
 // ---- launchers (psc_kernels.cu) ----
 void upload_stencil(cudaStream_t st);
 void launch_claim(const EventArgs& a, bool general, int blocks, int threads, cudaStream_t st);
@@ -303,6 +341,11 @@ void launch_commit(const EventArgs& a, bool general, int blocks, int threads, cu
 // reactions in a single block (lists of a few hundred molecules)
 constexpr int kEventOneThreads = 512;
 void launch_event_one(const EventArgs& a, cudaStream_t st);
+void launch_walk_words(uint32_t* word, const uint32_t* bits, uint64_t words, int blocks, cudaStream_t st);
+// blocks of the largest cluster, shared memory of a block on the current
+// device (0: none); sets the kernels' attributes there
+void walk_limits(int* cluster, int* smem);
+cudaError_t launch_walk(const WalkArgs& A, int blocks, bool cluster, cudaStream_t st);
 void launch_fill_u64(uint64_t* p, uint64_t value, size_t n, int blocks, cudaStream_t st);
 // Molecules per thread the persistent kernel holds in registers (0 = the
 // stretch does not fit); threads = its launch width.
@@ -397,12 +440,22 @@ void launch_populate_scatter(const uint32_t* sorted_vox, int64_t n_total, const 
                              const int64_t* starts, int n_species, uint16_t* occ, const Geometry& geo,
                              const ModelDev* model, int blocks, cudaStream_t st);
 // The Morton re-sort of a list's first min(*count, limit) entries (the rest,
-// if any, keep their places: list order never changes results).
+// if any, keep their places: list order never changes results): by the whole
+// code (keys and values for the radix sort, then a permutation), or by cells, the
+// top `cell_bits` bits of the Morton code: the entries per cell are counted
+// (cells zeroed before), and after an exclusive scan of the counts every entry
+// takes the next place of its cell in dst.
+constexpr int32_t kCellSortMax = 1 << 22;  // longer lists sort by the whole code: with cells, 10.7M walkers on 1024^3
+                                           // took 920 us per event against 843
 void launch_morton_keys(const SpeciesList& list, const int32_t* count, int32_t limit, const Geometry& geo,
                         uint32_t* keys, uint32_t* vals, int blocks, cudaStream_t st);
 uint32_t morton_sort_bits(const Geometry& geo);
 void launch_permute(const SpeciesList& src, const SpeciesList& dst, const uint32_t* perm,
                     const int32_t* count, int32_t limit, int blocks, cudaStream_t st);
+void launch_cell_count(const SpeciesList& list, const int32_t* count, int32_t limit, const Geometry& geo,
+                       uint32_t cell_bits, uint32_t* cells, int blocks, cudaStream_t st);
+void launch_cell_scatter(const SpeciesList& src, const SpeciesList& dst, const int32_t* count, int32_t limit,
+                         const Geometry& geo, uint32_t cell_bits, uint32_t* cells, int blocks, cudaStream_t st);
 void launch_copy_list(const SpeciesList& src, const SpeciesList& dst, const int32_t* count, int32_t limit,
                       int blocks, cudaStream_t st);
 // set the vacancy-mirror bit of every molecule of a list (mirror cleared before)
@@ -485,6 +538,8 @@ struct SortScratch {
 };
 size_t sort_scratch_bytes(int64_t max_n);
 void sort_scratch_bind(SortScratch& s, void* base, int64_t max_n);
+// exclusive scan of data[len] in place; sums: a word per 4096 of them
+void exclusive_scan(uint32_t* data, int64_t len, uint32_t* sums, cudaStream_t st, int64_t* launches);
 // After the call the sorted data is in (keys, vals) again.
 int radix_sort_pairs(uint32_t* keys, uint32_t* vals, const int32_t* n_dev, int64_t n_host,
                      int64_t max_n, int bits, SortScratch& scratch, cudaStream_t st,

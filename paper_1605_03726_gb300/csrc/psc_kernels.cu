@@ -1441,6 +1441,64 @@ void launch_populate_scatter(const uint32_t* sorted_vox, int64_t n_total, const 
     k_populate_scatter<<<blocks, 256, 0, st>>>(sorted_vox, n_total, o, b, n_species, occ, geo, model);
 }
 
+// Re-sort of a list by Morton cells, a counting sort: the order within a cell
+// is as it comes.  Seven short launches in all; a radix sort by the whole code
+// took 25 (1.23M entries: 178 us against 58, 2621 entries: 124 against 20).
+// Lanes in the same cell, most of a warp of a list sorted not long ago, count
+// together.
+__device__ __forceinline__ uint32_t cell_of(const Geometry& G, uint32_t v, uint32_t cell_bits)
+{
+    int32_t i, j, k;
+    decode(G, v, i, j, k);
+    return morton(G, i, j, k) >> (G.mort_bits - cell_bits);
+}
+
+__global__ void __launch_bounds__(256) k_cell_count(const SpeciesList L, const int32_t* count, int32_t limit,
+                                                    Geometry G, uint32_t cell_bits, uint32_t* cells)
+{
+    const int32_t n = min(*count, limit);
+    for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
+        const int idx = base + threadIdx.x;
+        const uint32_t c = idx < n ? cell_of(G, (uint32_t)L.vox[idx], cell_bits) : 0xFFFFFFFFu;
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, c);
+        if (idx < n && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&cells[c], (uint32_t)__popc(peers));
+    }
+}
+
+__global__ void __launch_bounds__(256) k_cell_scatter(const SpeciesList src, const SpeciesList dst,
+                                                      const int32_t* count, int32_t limit, Geometry G,
+                                                      uint32_t cell_bits, uint32_t* cells)
+{
+    const int32_t n = min(*count, limit);
+    const int lane = threadIdx.x & 31;
+    for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
+        const int idx = base + threadIdx.x;
+        const uint32_t v = idx < n ? (uint32_t)src.vox[idx] : 0u;
+        const uint32_t c = idx < n ? cell_of(G, v, cell_bits) : 0xFFFFFFFFu;
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, c);
+        const int leader = __ffs(peers) - 1;
+        uint32_t at = 0u;
+        if (idx < n && lane == leader) at = atomicAdd(&cells[c], (uint32_t)__popc(peers));
+        at = __shfl_sync(0xFFFFFFFFu, at, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        if (idx >= n) continue;
+        dst.vox[at] = (int32_t)v;
+        dst.ids[at] = src.ids[idx];
+        dst.img[at] = src.img[idx];
+    }
+}
+
+void launch_cell_count(const SpeciesList& list, const int32_t* count, int32_t limit, const Geometry& geo,
+                       uint32_t cell_bits, uint32_t* cells, int blocks, cudaStream_t st)
+{
+    k_cell_count<<<blocks, 256, 0, st>>>(list, count, limit, geo, cell_bits, cells);
+}
+
+void launch_cell_scatter(const SpeciesList& src, const SpeciesList& dst, const int32_t* count, int32_t limit,
+                         const Geometry& geo, uint32_t cell_bits, uint32_t* cells, int blocks, cudaStream_t st)
+{
+    k_cell_scatter<<<blocks, 256, 0, st>>>(src, dst, count, limit, geo, cell_bits, cells);
+}
+
 // Morton (Z-order) key of the voxel of each list entry (compact code)
 __global__ void k_morton_keys(const SpeciesList L, const int32_t* count, int32_t limit, Geometry G, uint32_t* keys,
                               uint32_t* vals)
@@ -1624,6 +1682,7 @@ void launch_births_batch(const EventArgs* tmpl, const BatchLaunch& bl, cudaStrea
 }
 
 #include "psc_small.cuh"
+#include "psc_walk.cuh"
 #include "psc_tiles.cuh"
 #include "psc_slab.cuh"
 #include "psc_subvol.cuh"

@@ -67,6 +67,7 @@ struct psc_lattice {
     int32_t ncomp = 1;                 // compartments (Sec. 2)
     std::vector<uint8_t> labels;       // compartment of every voxel (empty: all 0)
     uint32_t* claim = nullptr;         // per-voxel claim words (small lattices)
+    int64_t claim_n = 0;               // their number
     uint64_t* tables[2] = {nullptr, nullptr};   // claim hash tables (large lattices)
     uint32_t table_used[2] = {0, 0};   // slots written by the event that used it
     int64_t table_slots = 0;
@@ -92,6 +93,7 @@ struct psc_lattice {
     bool fo2[kMaxSpecies] = {};
     std::vector<int> reconcile[kMaxSpecies];
     uint64_t since_resort[kMaxSpecies] = {};
+    bool placed_order[kMaxSpecies] = {};       // the list is as the placement left it, in no order
 
     psc_options opt{64, 256, 8, 0, 32, 0, 0, 1, 1, 3, 0, 1000000, 0, 0, 0, -1, 1};
     int64_t launches = 0;
@@ -114,11 +116,16 @@ struct psc_lattice {
         int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
         int32_t scratch_n = 0;
         bool map_holds = false;        // the map agrees with the lists (nothing else has changed them since)
-        bool asked = false;            // the device was asked for the next two
         int cluster = 0, grid = 0;     // most blocks of a stretch: one cluster, a cooperative grid
         uint32_t general = 0, fo2 = 0, mapped = 0;
         uint32_t products[kMaxSpecies] = {};
     } small;
+    // lattices without reactions (k_walk_run)
+    bool walk_only = false;            // no reactions, no compartments
+    bool claim_vacancy = false;        // the claim words tell vacancy (else all free between events)
+    uint32_t walk_epoch = 0;           // of the last event that claimed in them
+    int walk_cluster = 0, walk_smem = 0;       // blocks of a cluster, shared memory of a block (0: none)
+    bool shapes_known = false;         // the device was asked for these and for small.cluster, small.grid
     bool stretches = true;             // false: made for a batch, no room for tombstones is kept
     int64_t list_slack = 0;            // entries of room for tombstones in the lists of reaction products
 
@@ -205,12 +212,15 @@ EventArgs event_args(const psc_lattice* L, int s);
 ReconcileArgs reconcile_args(const psc_lattice* L, int x);
 bool next_event(const psc_lattice* L, int* s_out, double* t_out);
 int check_device(psc_lattice* L);
+// every claim word free again (after stretches of k_walk_run), as the other kernels want them
+int claims_free(psc_lattice* L);
 // queue events in scheduler order until max_events or the next event lies after t_end
 int drive(psc_lattice* L, double t_end, int64_t max_events);
 // drop every captured graph (launch options changed)
 void graph_cache_clear(psc_lattice* L);
 // Morton re-sort of species s's list (queued on the lattice's stream)
 int resort(psc_lattice* L, int s);
+int sort_first(psc_lattice* L, int s);
 void dev_free_one(psc_lattice* L, void* p);
 // Can stretches of species s run under the tile kernel?  Fills the plan.
 bool tile_plan(psc_lattice* L, int s, TilePlan* P);

@@ -44,17 +44,22 @@ __device__ __forceinline__ void small_copy(void* dst, const void* src, size_t by
     for (uint32_t x = threadIdx.x; x < bytes / 4; x += blockDim.x) d[x] = s[x];
 }
 
+// Barrier of a cluster's blocks.  One fence per block, made cumulative over
+// the block by the block barrier: a release by every warp took 500 cycles longer.
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncthreads();
+    if (threadIdx.x == 0) __threadfence();
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <bool CLUSTER>
 __device__ __forceinline__ bool small_barrier(const SmallArgs& A)
 {
     if (CLUSTER) {
-        // one fence per block, made cumulative over the block by the block
-        // barrier: a release by every warp took 500 cycles longer
-        __syncthreads();
-        if (threadIdx.x == 0) __threadfence();
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.relaxed.aligned;\n"
-                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        cluster_barrier();
         return true;
     }
     return grid_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, 0u);

@@ -1,8 +1,9 @@
 // psc_sort.cu -- stable LSD radix sort of (uint32 key, uint32 value) pairs.
 //
 // Used for the placement of molecules (voxels ordered by their Philox key; a
-// stable sort of keys in voxel order gives the (key, voxel) order) and for the
-// periodic Morton re-sort of the molecule lists.  Each 8-bit pass is
+// stable sort of keys in voxel order gives the (key, voxel) order) and for
+// read-outs in id order; its scan also serves the re-sort of the molecule
+// lists by cells.  Each 8-bit pass is
 //   hist     per-tile digit counts, stored digit-major;
 //   scan     exclusive scan of the counts (three kernels);
 //   scatter  per tile, stable ranks from warp match + per-warp prefix counts.
@@ -186,6 +187,20 @@ k_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, 
         }
         __syncthreads();
     }
+}
+
+void exclusive_scan(uint32_t* data, int64_t len, uint32_t* sums, cudaStream_t st, int64_t* launches)
+{
+    const int blocks = (int)ceil_div(len, kScanTile);
+    if (blocks <= 4) {                  // a few tiles: one block, tile after tile
+        k_scan_sums<<<1, kScanThreads, 0, st>>>(data, len);
+        if (launches) *launches += 1;
+        return;
+    }
+    k_scan_reduce<<<blocks, kScanThreads, 0, st>>>(data, len, sums);
+    k_scan_sums<<<1, kScanThreads, 0, st>>>(sums, blocks);
+    k_scan_down<<<blocks, kScanThreads, 0, st>>>(data, len, sums);
+    if (launches) *launches += 3;
 }
 
 int radix_sort_pairs(uint32_t* keys, uint32_t* vals, const int32_t* n_dev, int64_t n_host,

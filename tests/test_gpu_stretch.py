@@ -65,6 +65,7 @@ def test_stretches_match_oracle(name, shape, boundary, recipe, calls):
         g.run_events(7)
         o.run_events(7)
         assert_same(g, o, (name, persistent))
+    g.set_options(resort_period=-1)
     before = g.stats()["launches"]
     g.run_events(64)
     assert g.stats()["launches"] - before <= 2            # one stretch, not per-event launches
