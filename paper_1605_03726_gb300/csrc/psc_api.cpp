@@ -2039,14 +2039,17 @@ static void order_by_id(const std::vector<uint32_t>& ids, std::vector<int64_t>& 
     std::sort(order.begin(), order.end(), [&](int64_t x, int64_t y) { return ids[x] < ids[y]; });
 }
 
-// The n molecules of list s in id order, built on the device (ids sorted with
-// their slots, then one gather) and copied to the caller's host buffers in
-// one piece each.  Used when the list fits the re-sort scratch; returns
-// PSC_OK, an error, or 1 when the caller should build the answer on the host.
+// The n molecules of list s in id order, built on the device and copied to the
+// caller's host buffers in one piece each: entries of a species without
+// reactions go straight to their places, its ids being the ones placement gave
+// it; else the ids are sorted with their slots, where the list fits the
+// re-sort scratch.  Returns PSC_OK, an error, or 1 when the caller should build
+// the answer on the host.
 static int device_positions(psc_lattice* L, int32_t s, int64_t n, bool unwrapped, int32_t* out,
                             uint32_t* ids_out)
 {
-    if (n <= 0 || n > L->rs_max) return 1;
+    const bool by_id = !L->live[s] && n == L->sp[s].n0;
+    if (n <= 0 || (n > L->rs_max && !by_id)) return 1;
     if (n > L->readout_cap) {
         if (L->readout) dev_free_one(L, L->readout);
         L->readout = (int32_t*)dev_alloc(L, (size_t)n * 16);
@@ -2056,7 +2059,13 @@ static int device_positions(psc_lattice* L, int32_t s, int64_t n, bool unwrapped
     int32_t* pos = L->readout;
     uint32_t* ids = reinterpret_cast<uint32_t*>(L->readout + 3 * n);
     const int blocks = event_blocks(L, n);
-    if (readout_positions(L->model_h.lists[s], (int32_t)n, L->ni, L->nj, L->nk, unwrapped,
+    if (by_id) {
+        uint32_t id_lo = 0;
+        for (int x = 0; x < s; ++x) id_lo += (uint32_t)L->sp[x].n0;
+        if (readout_by_id(L->model_h.lists[s], (int32_t)n, id_lo, L->ni, L->nj, L->nk, unwrapped,
+                          (L->bflags & PSC_FCC) != 0, pos, ids, &L->sc->err, blocks, L->stream, &L->launches) != 0)
+            return cuda_fail(L, cudaErrorUnknown);
+    } else if (readout_positions(L->model_h.lists[s], (int32_t)n, L->ni, L->nj, L->nk, unwrapped,
                           (L->bflags & PSC_FCC) != 0, L->rs_keys, L->rs_vals, L->rs_scratch, pos, ids, blocks,
                           L->stream, &L->launches) != 0)
         return cuda_fail(L, cudaErrorUnknown);
