@@ -144,9 +144,11 @@ typedef struct {
     int32_t claim_table;      /* before populate: 1 = one claim word per voxel,
                                  2 = hash table of claims, 0/-1 = by size (a
                                  word per voxel up to 2^22 voxels, where the
-                                 two tables would be as large, or up to 28
-                                 million voxels where there are no reactions
-                                 and the molecules fit in shared memory)       */
+                                 two tables would be as large, or without
+                                 reactions: up to 28 million voxels where the
+                                 molecules fit in shared memory, above that
+                                 from 262,144 molecules of a species on, if
+                                 the memory is there)                          */
     int32_t persistent;       /* 1 = run stretches of events in one launch
                                  (default): of a lattice without reactions and
                                  compartments whose molecules fit in shared
@@ -180,7 +182,10 @@ typedef struct {
                                  (when the lattice does not run in stretches
                                  of all its species, see persistent, and
                                  the species has >= 2^18 molecules on a
-                                 lattice of more than 2^22 voxels and,
+                                 lattice of more than 2^22 voxels -- above 28
+                                 million voxels its lean variant, below 2.6
+                                 million molecules; else claim and commit
+                                 launches -- and,
                                  at its first stretch, the fullest box holds
                                  at most 1.4 x the mean: molecules confined
                                  to part of the lattice take the molecule-

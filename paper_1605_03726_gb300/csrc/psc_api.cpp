@@ -137,10 +137,13 @@ int32_t sort_limit(const psc_lattice* L, int x)
 // Does Morton order pay for list x?  Only if the list holds at least 1/256 of
 // the voxels (by its estimate): sparser lists share too few cache lines
 // between neighbours in any order, and their re-sorts cost more than they
-// save.  A skipped re-sort changes no result.
+// save.  (Long lists on large lattices always: their claim launches read a
+// mirror that does not fit in L2; 2.1M walkers on 1024^3 118 us per event, 140
+// unsorted.)  A skipped re-sort changes no result.
 bool sorted_order_pays(const psc_lattice* L, int x)
 {
-    return !L->counts_h || L->est[x] * 256 >= L->V;
+    return !L->counts_h || L->est[x] * 256 >= L->V ||
+           (L->open_claims && L->est[x] >= kOpenList);
 }
 
 // Lists come from the placement in no order: the first sort of list s is due
@@ -341,6 +344,13 @@ int enqueue_event(psc_lattice* L, int s)
         launch_event_one(a1, L->stream);
         span_close(L, sp, kSpanClaim);
         L->launches += 1;
+    } else if (!L->general[s] && L->est[s] >= kOpenList) {
+        launch_open_claim(a, L->est[s], L->sm_count, L->stream);
+        span_close(L, sp, kSpanClaim);
+        sp = span_open(L);
+        launch_open_commit(a, L->est[s], L->sm_count, L->stream);
+        span_close(L, sp, kSpanCommit);
+        L->launches += 2;
     } else {
         launch_claim(a, L->general[s], blocks, threads, L->stream);
         span_close(L, sp, kSpanClaim);
@@ -543,6 +553,7 @@ bool tile_plan(psc_lattice* L, int s, TilePlan* P)
                      lean_smem_bytes(best) <= L->tile_smem) ? 1 : 0;
     }
     if (L->opt.tiles == 0) {
+        if (L->open_claims && (!best.lean || L->sp[s].n0 >= kOpenOverLean)) return false;
         if (L->tile_auto[s] == 0) L->tile_auto[s] = tile_balanced(L, s, best) ? 1 : -1;
         if (L->tile_auto[s] < 0) return false;
     }
@@ -600,6 +611,19 @@ static int tile_buffers(psc_lattice* L, const TilePlan& P, int64_t ids)
         if (!T.img_id) return PSC_E_NOMEM;
     }
     return PSC_OK;
+}
+
+// Do events of species s take claim and commit launches (psc_open.cuh)
+// although stretches are on?  Long lists of large lattices without reactions,
+// unless the tile kernel takes them.  Decided once (options reset it).
+static bool open_route(psc_lattice* L, int s)
+{
+    if (!L->open_claims || L->opt.persistent <= 0 || L->opt.run_per_thread > 0 || L->sp[s].n0 < kOpenList) return false;
+    if (L->open_auto[s] == 0) {
+        TilePlan P{};
+        L->open_auto[s] = tile_plan(L, s, &P) ? -1 : 1;
+    }
+    return L->open_auto[s] > 0;
 }
 
 int enqueue_tiles(psc_lattice* L, int s, int64_t n_events, const TilePlan& P)
@@ -1321,6 +1345,10 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         if (L->sp[s].D > 0.0 && hb > hb_max) hb_max = hb;
     }
     bool direct = L->V <= (1ll << 22) || hb_max == 0;
+    // (batches take the lattices that have claim words by these rules)
+    L->batchable = direct || 2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V;
+    if (L->opt.claim_table == 1) L->batchable = true;
+    if (L->opt.claim_table == 2 && hb_max > 0) L->batchable = false;
     // lattices without reactions whose claim words fit in the L2 cache take
     // k_walk_run while their molecules fit in shared memory
     L->walk_only = L->nrx == 0 && !comps && L->opt.subvolume <= 0;
@@ -1331,14 +1359,27 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     // per-event kernels empty the previous table in full every event (species
     // that are reaction products get lists sized for the lattice)
     if (2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V) direct = true;
+    // larger ones with long lists and no reactions skip most claims: words need
+    // no table to be emptied (and the tile kernel wants them too)
+    bool open = false;
+    for (int s = 0; s < L->nsp; ++s)
+        open = open || (L->nrx == 0 && L->V > kWalkVoxels && L->sp[s].D > 0.0 && L->sp[s].n0 >= kOpenList &&
+                        L->opt.subvolume <= 0);
     if (L->opt.claim_table == 1) direct = true;
-    if (L->opt.claim_table == 2 && hb_max > 0) direct = false;
-    if (direct) {
+    if (L->opt.claim_table == 2 && hb_max > 0) direct = open = false;
+    if (open && !direct) {
+        L->claim_n = L->V;
+        L->claim = (uint32_t*)dev_alloc(L, V * sizeof(uint32_t));
+        direct = L->claim != nullptr;                // no room: tables
+        if (!direct) cudaGetLastError();
+    }
+    L->open_claims = open && direct;
+    if (direct && !L->claim) {
         // (k_walk_run orders them as the mirror's bits, whole bricks)
         L->claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
         L->claim = (uint32_t*)dev_alloc(L, (size_t)L->claim_n * sizeof(uint32_t));
         if (!L->claim) return PSC_E_NOMEM;
-    } else {
+    } else if (!direct) {
         L->table_slots = (int64_t)1 << hb_max;
         for (int t = 0; t < 2; ++t) {
             L->tables[t] = (uint64_t*)dev_alloc(L, ((size_t)1 << hb_max) * sizeof(uint64_t));
@@ -1707,7 +1748,7 @@ static int graph_run(psc_lattice* L, double t_end, int64_t room, int64_t* done)
             if (best < 0 || t < tb) { best = s; tb = t; }
         }
         if (best < 0 || tb > t_end) return PSC_OK;
-        if (!L->general[best] && L->opt.persistent > 0) return PSC_OK;   // a stretch comes first
+        if (!L->general[best] && L->opt.persistent > 0 && !open_route(L, best)) return PSC_OK;   // a stretch comes first
         seq[(size_t)e] = best;
         at[(size_t)e] = tb;
         next[best]++;
@@ -1874,11 +1915,12 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             continue;
         }
         int threads = 0, blocks = 0;
-        const int per = run_width(L, s, &threads, &blocks);
+        const bool open = open_route(L, s);
+        const int per = open ? 0 : run_width(L, s, &threads, &blocks);
         TilePlan plan{};
         // the tile kernel needs no molecule slots per thread: it also takes
         // species above the molecule-list kernel's capacity
-        const bool tiles = L->opt.persistent > 0 && !L->general[s] && tile_plan(L, s, &plan);
+        const bool tiles = !open && L->opt.persistent > 0 && !L->general[s] && tile_plan(L, s, &plan);
         if (!tiles)
             if (int rc = sort_first(L, s)) return rc;
         if (per > 0 || tiles) {
@@ -2223,6 +2265,7 @@ int psc_set_options(psc_lattice* L, const psc_options* o)
         return PSC_E_ARG;
     if (o->blocks_per_sm < 0) return PSC_E_ARG;
     graph_cache_clear(L);                            // captured launches follow the options
+    std::memset(L->open_auto, 0, sizeof(L->open_auto));
     if (o->resort_period) L->opt.resort_period = o->resort_period;
     if (o->block_threads) L->opt.block_threads = o->block_threads;
     if (o->blocks_per_sm) L->opt.blocks_per_sm = o->blocks_per_sm;

@@ -205,7 +205,7 @@ int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop)
 {
     if (!B || !L) return PSC_E_ARG;
     if (!L->populated) return PSC_E_ORDER;
-    if (L->device != B->device || L->stream != B->stream || !L->claim || L->tables[0]) return PSC_E_UNSUPPORTED;
+    if (L->device != B->device || L->stream != B->stream || !L->claim || !L->batchable) return PSC_E_UNSUPPORTED;
     int free_slot = -1;
     for (int i = 0; i < kBatchMax; ++i) {
         if (B->slot[i].L == L) return PSC_E_ARG;

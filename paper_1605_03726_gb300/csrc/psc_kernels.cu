@@ -1684,6 +1684,7 @@ void launch_births_batch(const EventArgs* tmpl, const BatchLaunch& bl, cudaStrea
 #include "psc_small.cuh"
 #include "psc_walk.cuh"
 #include "psc_tiles.cuh"
+#include "psc_open.cuh"
 #include "psc_slab.cuh"
 #include "psc_subvol.cuh"
 

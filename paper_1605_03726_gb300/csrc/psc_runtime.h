@@ -122,6 +122,9 @@ struct psc_lattice {
     } small;
     // lattices without reactions (k_walk_run)
     bool walk_only = false;            // no reactions, no compartments
+    bool batchable = false;            // may join a batch
+    int8_t open_auto[kMaxSpecies] = {};        // 0 not decided, 1 those launches, -1 another kernel
+    bool open_claims = false;          // no reactions, too large for k_walk_run, a claim word per voxel
     bool claim_vacancy = false;        // the claim words tell vacancy (else all free between events)
     uint32_t walk_epoch = 0;           // of the last event that claimed in them
     int walk_cluster = 0, walk_smem = 0;       // blocks of a cluster, shared memory of a block (0: none)

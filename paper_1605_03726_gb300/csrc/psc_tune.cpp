@@ -28,6 +28,7 @@ struct Trial {
 void apply(psc_lattice* L, const Trial& t)
 {
     graph_cache_clear(L);
+    std::memset(L->open_auto, 0, sizeof(L->open_auto));
     L->opt.persistent = t.persistent;
     L->opt.run_per_thread = t.run_per_thread;
     L->opt.block_threads = t.block_threads;

@@ -114,10 +114,10 @@ __device__ __forceinline__ uint32_t walk_target(const WalkArgs& A, const uint8_t
     return small_place(G, nb.i, nb.j, nb.k) | kWalkWrap;
 }
 
-__device__ __forceinline__ uint32_t walk_draw(const WalkArgs& A, uint32_t id, uint32_t g, uint32_t c2)
+__device__ __forceinline__ uint32_t walk_draw(uint32_t key0, uint32_t key1, uint32_t id, uint32_t g, uint32_t c2)
 {
     uint32_t u[4];
-    philox(id, g, c2, 0u, A.key0, A.key1, u);
+    philox(id, g, c2, 0u, key0, key1, u);
     return __umulhi(u[0], 12u);
 }
 
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(CLUSTER ? kWalkClusterThreads : kWalkThreads, 
     auto draw = [&](int e) {
         const int q = A.seq[e], mine = count(q);
         for (int m = A.slot0[q]; m < A.slot0[q] + mine; ++m)
-            s_t[m * NT] = walk_draw(A, s_id[m * NT], A.g + (uint32_t)e, ((uint32_t)A.species[q] << 4) | kTagEvent);
+            s_t[m * NT] = walk_draw(A.key0, A.key1, s_id[m * NT], A.g + (uint32_t)e, ((uint32_t)A.species[q] << 4) | kTagEvent);
     };
     draw(0);
     for (int e = 0; e < A.n_events; ++e) {
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(CLUSTER ? kWalkClusterThreads : kWalkThreads, 
             if (again) {
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (m + u < mine) d[u] = walk_draw(A, id[u], A.g + (uint32_t)e + 1u, ((uint32_t)A.species[q] << 4) | kTagEvent);
+                    if (m + u < mine) d[u] = walk_draw(A.key0, A.key1, id[u], A.g + (uint32_t)e + 1u, ((uint32_t)A.species[q] << 4) | kTagEvent);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
