@@ -791,44 +791,90 @@ static bool small_fits(psc_lattice* L, int s)
     return !(L->opt.tiles > 0 && tile_plan(L, s, &P));
 }
 
-// A stretch of consecutive events, starting with species s at time t: one
-// launch.  *n = events queued.
-static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
+// Bytes of the buffers a lattice's stretches of k_small_run still lack, and
+// their allocation; scratch: lists are closed up in a grid or a group of blocks.
+static int32_t small_scratch(const psc_lattice* L)
+{
+    int64_t most = 0;
+    for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, L->model_h.lists[x].cap);
+    return (int32_t)std::min<int64_t>(4 * kSmallList, 4 * most + 4096);
+}
+
+int64_t small_lacks(const psc_lattice* L, bool scratch)
+{
+    const auto& B = L->small;
+    bool pairs = false, general = false;
+    for (int s = 0; s < L->nsp; ++s) {
+        general = general || L->general[s];
+        for (int x = 0; x < L->nsp; ++x) pairs = pairs || L->pair[s][x] >= 0;
+    }
+    int64_t b = B.ev ? 0 : (int64_t)L->nsp * (int64_t)sizeof(EventArgs);
+    if (pairs && !B.slot) b += L->V * 4;
+    if (scratch && general && !B.scratch) b += (int64_t)small_scratch(L) * 8;
+    return b;
+}
+
+int small_buffers(psc_lattice* L, bool lists, bool scratch)
 {
     auto& B = L->small;
     if (!B.ev) {
         const int rc = small_setup(L);
         if (rc) return rc;
     }
-    bool lists = false;                              // a species with reactions may come up
-    for (int x = 0; x < L->nsp && !lists; ++x) lists = L->general[x] && L->sp[x].D > 0.0 && small_fits(L, x);
     if (lists && B.mapped && !B.slot) {
         B.slot = (uint32_t*)dev_alloc(L, (size_t)L->V * 4);
         if (!B.slot) return PSC_E_NOMEM;
     }
-    bool lists_long = false;                         // a stretch may take a grid
-    for (int x = 0; lists && x < L->nsp && !lists_long; ++x)
-        lists_long = L->sp[x].D > 0.0 && L->est[x] > kSmallCluster && small_fits(L, x);
-    if (lists_long && !B.scratch) {                  // closing lists up in a grid
-        int64_t most = 0;
-        for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, L->model_h.lists[x].cap);
-        B.scratch_n = (int32_t)std::min<int64_t>(4 * kSmallList, 4 * most + 4096);
+    if (lists && scratch && B.general && !B.scratch) {
+        B.scratch_n = small_scratch(L);
         B.scratch = (int32_t*)dev_alloc(L, (size_t)B.scratch_n * 8);
-        if (!B.scratch) return PSC_E_NOMEM;
+        if (!B.scratch) {
+            B.scratch_n = 0;
+            return PSC_E_NOMEM;
+        }
     }
+    return PSC_OK;
+}
+
+// The arguments of a stretch but its events; reacts: they include reactions.
+void small_args(psc_lattice* L, bool reacts, SmallArgs* A)
+{
+    auto& B = L->small;
+    A->ev = B.ev;
+    A->model = L->model_d;
+    A->sc = L->sc;
+    A->slot = B.slot;
+    A->holes = B.scratch;
+    A->surv = B.scratch + B.scratch_n;
+    A->scratch_n = B.scratch_n;
+    A->barrier = L->barrier;
+    A->barrier_timeout_ns = (uint64_t)L->opt.barrier_timeout_us * 1000ull;
+    A->nsp = L->nsp;
+    A->collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
+    if (!reacts) return;
+    A->general = B.general;
+    A->fo2 = B.fo2;
+    A->mapped = B.mapped;
+    std::memcpy(A->products, B.products, sizeof(A->products));
+    A->build_map = B.map_holds ? 0 : 1;
+    B.map_holds = true;
+}
+
+// A stretch of consecutive events, starting with species s at time t: one
+// launch.  *n = events queued.
+static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
+{
+    auto& B = L->small;
+    bool lists = false, grid = false;                // a species with reactions may come up; a grid may
+    for (int x = 0; x < L->nsp; ++x) {
+        if (!(L->sp[x].D > 0.0) || !small_fits(L, x)) continue;
+        lists = lists || L->general[x];
+        grid = grid || L->est[x] > kSmallCluster;
+    }
+    int rc = small_buffers(L, lists, grid);
+    if (rc) return rc;
     SmallArgs A{};
-    A.ev = B.ev;
-    A.model = L->model_d;
-    A.sc = L->sc;
-    A.slot = B.slot;
-    A.holes = B.scratch;
-    A.surv = B.scratch + B.scratch_n;
-    A.scratch_n = B.scratch_n;
-    A.barrier = L->barrier;
-    A.barrier_timeout_ns = (uint64_t)L->opt.barrier_timeout_us * 1000ull;
     A.g = L->g;
-    A.nsp = L->nsp;
-    A.collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
     const int64_t limit = std::min<int64_t>(std::min<int64_t>(max_events, kSmallEvents),
                                             (int64_t)UINT32_MAX - L->g);
     int8_t fits[kMaxSpecies] = {};                   // 0 not asked yet, 1 yes, -1 no
@@ -846,14 +892,7 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
         if (fits[s] == 0) fits[s] = small_fits(L, s) ? 1 : -1;
         if (fits[s] < 0) break;
     }
-    if (reacts) {
-        A.general = B.general;
-        A.fo2 = B.fo2;
-        A.mapped = B.mapped;
-        std::memcpy(A.products, B.products, sizeof(A.products));
-        A.build_map = B.map_holds ? 0 : 1;
-        B.map_holds = true;
-    }
+    small_args(L, reacts, &A);
     // the shape: a cluster of 16 blocks up to kSmallCluster entries (with fewer
     // blocks, or 128 threads in each, short lists got slower: 2621 walkers 3.9 us
     // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM,
@@ -862,7 +901,6 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
     const bool cluster = longest <= kSmallCluster;
     const int threads = !cluster && longest <= 65536 ? kSmallThreads / 2 : kSmallThreads;
     const int blocks = cluster ? B.cluster : std::min(B.grid, longest <= 131072 ? L->sm_count : 2 * L->sm_count);
-    int rc = PSC_OK;
     if (!cluster) rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream));
     if (rc) return rc;
     cudaEvent_t sp = span_open(L);

@@ -26,6 +26,7 @@ constexpr int kItemThreadsDefault = 256;   // threads per block of the batched l
 struct Member {
     psc_lattice* L = nullptr;
     double t_stop = INFINITY;             // run events up to this time
+    bool stretch = false;                 // runs in stretches (else in batched launches per event phase)
 };
 
 }  // namespace
@@ -42,6 +43,16 @@ struct psc_batch {
     int threads = kItemThreadsDefault;
     int item_blocks_max = kItemBlocksMaxDefault;
     int32_t resort_period = -1;           // events of a member's species between Morton re-sorts (-1 never)
+    // stretches of the members' events, one launch for many members
+    int stretch_blocks = -1;              // most blocks of a launch (-1: not asked, 0: no stretches)
+    bool use_stretches = true;
+    SmallArgs* args_d = nullptr;          // [kBatchMax], device: one for each member that takes part
+    int2* group_d = nullptr;              // [stretch_blocks]
+    int32_t* counts_d = nullptr;          // [kBatchMax][kMaxSpecies] list lengths after a stretch
+    int32_t* counts_h = nullptr;          // pinned copy, for the next stretch's groups
+    cudaEvent_t counts_ev = nullptr;
+    bool counts_pending = false;
+    std::vector<psc_lattice*> counts_of;  // whose lengths counts_h holds
 };
 
 namespace {
@@ -54,7 +65,8 @@ int item_blocks(const psc_batch* B, int64_t work)
 
 // Queue the next event of every member whose next event time is <= its
 // t_stop (and <= t_cap); returns how many members had one.
-int batch_event(psc_batch* B, double t_cap, int* rc_out)
+// (all: members that could run in stretches too.)
+int batch_event(psc_batch* B, double t_cap, bool all, int* rc_out)
 {
     *rc_out = PSC_OK;
     struct Act {
@@ -68,7 +80,7 @@ int batch_event(psc_batch* B, double t_cap, int* rc_out)
     int total = 0;
     for (int i = 0; i < kBatchMax; ++i) {
         psc_lattice* L = B->slot[i].L;
-        if (!L || L->sticky) continue;
+        if (!L || L->sticky || (!all && B->slot[i].stretch)) continue;
         int s;
         double t;
         if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
@@ -183,6 +195,155 @@ int batch_event(psc_batch* B, double t_cap, int* rc_out)
     return na;
 }
 
+// ---------------------------------------------------------------------------
+// stretches: every member's events in a group of blocks of its own, at its own
+// pace, one launch for as many members as there are blocks on the device
+// ---------------------------------------------------------------------------
+int stretch_buffers(psc_batch* B, psc_lattice* L)
+{
+    if (B->stretch_blocks < 0) B->stretch_blocks = small_batch_blocks(L->sm_count);
+    if (B->stretch_blocks == 0 || B->args_d) return PSC_OK;
+    if (cudaMalloc(&B->args_d, sizeof(SmallArgs) * kBatchMax) != cudaSuccess ||
+        cudaMalloc(&B->group_d, sizeof(int2) * (size_t)B->stretch_blocks) != cudaSuccess ||
+        cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kMaxSpecies) != cudaSuccess ||
+        cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kMaxSpecies) != cudaSuccess ||
+        cudaEventCreateWithFlags(&B->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        B->stretch_blocks = 0;            // what was allocated goes with the batch
+    }
+    return PSC_OK;
+}
+
+// May L run in stretches?  extra: bytes of its buffers for that, at most `room`.
+bool member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra)
+{
+    *extra = 0;
+    if (L->opt.persistent <= 0 || L->opt.time_kernels > 0 || L->opt.subvolume > 0 || L->opt.barrier_phantom > 0)
+        return false;
+    stretch_buffers(B, L);
+    if (B->stretch_blocks <= 0) return false;
+    const int64_t lacks = small_lacks(L, true);
+    if (lacks > room) return false;
+    if (small_buffers(L, true, true) != PSC_OK) {
+        cudaGetLastError();
+        L->sticky = PSC_OK;               // no room on the device: batched launches
+        return false;
+    }
+    // a group's barrier goes on from whatever complete barriers left there
+    if (cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), B->stream) != cudaSuccess) return false;
+    *extra = lacks;
+    return true;
+}
+
+// Up to n_events next events of every member that runs in stretches, up to
+// its t_stop and t_cap; the number of members that had any.
+int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
+{
+    *rc_out = PSC_OK;
+    if (!B->use_stretches || B->stretch_blocks <= 0) return 0;
+    // the list lengths after the last stretch: groups follow them
+    if (B->counts_pending) {
+        if (cudaEventSynchronize(B->counts_ev) != cudaSuccess) {
+            *rc_out = PSC_E_CUDA;
+            return 1;
+        }
+        B->counts_pending = false;
+        for (size_t r = 0; r < B->counts_of.size(); ++r) {
+            psc_lattice* L = B->counts_of[r];
+            bool member = false;
+            for (int i = 0; i < kBatchMax && !member; ++i) member = B->slot[i].L == L;
+            for (int s = 0; member && s < L->nsp; ++s) {
+                const int32_t c = B->counts_h[r * kMaxSpecies + (size_t)s];
+                if (c >= 0) L->est[s] = c;
+            }
+        }
+    }
+    std::vector<SmallArgs> args;
+    std::vector<double> work;             // molecules per event
+    B->counts_of.clear();
+    bool births = false;
+    for (int i = 0; i < kBatchMax; ++i) {
+        psc_lattice* L = B->slot[i].L;
+        if (!L || L->sticky || !B->slot[i].stretch) continue;
+        int s;
+        double t;
+        if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
+        if ((*rc_out = claims_free(L))) return 1;
+        SmallArgs A{};
+        small_args(L, true, &A);
+        A.g = L->g;
+        const int64_t limit = std::min<int64_t>(std::min<int64_t>(n_events, kSmallEvents), (int64_t)UINT32_MAX - L->g);
+        double molecules = 0.0;
+        do {
+            A.seq[A.n_events++] = (uint8_t)s;
+            molecules += (double)L->est[s];
+            L->sp[s].done++;
+            L->g++;
+            L->clock = t;
+        } while (A.n_events < limit && next_event(L, &s, &t) && t <= B->slot[i].t_stop && t <= t_cap);
+        births = births || A.fo2 != 0u;
+        L->events += (uint64_t)A.n_events;
+        L->launches += 1;
+        work.push_back(molecules / A.n_events);
+        args.push_back(A);
+        B->counts_of.push_back(L);
+    }
+    if (args.empty()) return 0;
+    const int total = (int)args.size();
+    const int launches = (total + B->stretch_blocks - 1) / B->stretch_blocks;
+    std::vector<int2> group;
+    for (int l = 0; l < launches; ++l) {
+        const int lo = (int)((int64_t)total * l / launches), hi = (int)((int64_t)total * (l + 1) / launches);
+        // blocks by work; an event takes about as long with no molecules as
+        // with 600 per block
+        double sum = 0.0;
+        for (int r = lo; r < hi; ++r) sum += work[(size_t)r] + 600.0;
+        const int spare = B->stretch_blocks - (hi - lo);
+        group.clear();
+        for (int r = lo; r < hi; ++r) {
+            const int more = (int)(spare * (work[(size_t)r] + 600.0) / sum);
+            const int most = (int)(work[(size_t)r] / kSmallThreads);           // with it, a molecule per thread
+            const int blocks = 1 + std::min(more, most);
+            args[(size_t)r].blocks = blocks;
+            group.insert(group.end(), (size_t)blocks, make_int2(r, (int)group.size()));
+        }
+        if (cudaMemcpyAsync(B->args_d + lo, args.data() + lo, sizeof(SmallArgs) * (size_t)(hi - lo),
+                            cudaMemcpyHostToDevice, B->stream) != cudaSuccess ||
+            cudaMemcpyAsync(B->group_d, group.data(), sizeof(int2) * group.size(), cudaMemcpyHostToDevice, B->stream) !=
+                cudaSuccess ||
+            (l == 0 && cudaMemsetAsync(B->counts_d, 0xFF, sizeof(int32_t) * kMaxSpecies * (size_t)total, B->stream) !=
+                           cudaSuccess) ||
+            launch_small_batch(B->args_d, B->group_d, B->counts_d, (int)group.size(), births, B->stream) !=
+                cudaSuccess) {
+            *rc_out = PSC_E_CUDA;
+            return total;
+        }
+        B->launches += 1;
+    }
+    if (cudaMemcpyAsync(B->counts_h, B->counts_d, sizeof(int32_t) * kMaxSpecies * (size_t)total,
+                        cudaMemcpyDeviceToHost, B->stream) != cudaSuccess ||
+        cudaEventRecord(B->counts_ev, B->stream) != cudaSuccess)
+        *rc_out = PSC_E_CUDA;
+    else
+        B->counts_pending = true;
+    return total;
+}
+
+// Up to n_events next events of every member, up to t_cap; false when none had
+// any left.
+bool batch_advance(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
+{
+    const int64_t e = std::min<int64_t>(n_events, kSmallEvents);
+    bool any = batch_stretch(B, t_cap, e, rc_out) > 0;
+    if (*rc_out) return true;
+    for (int64_t x = 0; x < e; ++x) {
+        if (batch_event(B, t_cap, !B->use_stretches, rc_out) == 0) break;
+        any = true;
+        if (*rc_out) return true;
+    }
+    return any;
+}
+
 int upload_templates(psc_batch* B, int slot, psc_lattice* L)
 {
     std::vector<EventArgs> ev(kMaxSpecies);
@@ -201,7 +362,7 @@ int upload_templates(psc_batch* B, int slot, psc_lattice* L)
     return PSC_OK;
 }
 
-int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop)
+int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop, int64_t room, int64_t* extra)
 {
     if (!B || !L) return PSC_E_ARG;
     if (!L->populated) return PSC_E_ORDER;
@@ -217,6 +378,7 @@ int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop)
     if (rc) return rc;
     B->slot[free_slot].L = L;
     B->slot[free_slot].t_stop = t_stop;
+    B->slot[free_slot].stretch = member_stretches(B, L, room, extra);
     B->size++;
     return PSC_OK;
 }
@@ -252,7 +414,11 @@ int psc_batch_create(psc_batch** out, int device, void* cuda_stream)
     return PSC_OK;
 }
 
-int psc_batch_add(psc_batch* B, psc_lattice* L) { return batch_add_until(B, L, INFINITY); }
+int psc_batch_add(psc_batch* B, psc_lattice* L)
+{
+    int64_t extra = 0;
+    return batch_add_until(B, L, INFINITY, INT64_MAX, &extra);
+}
 
 int psc_batch_remove(psc_batch* B, psc_lattice* L)
 {
@@ -280,10 +446,10 @@ int psc_batch_run_events(psc_batch* B, int64_t n_events)
 {
     if (!B || n_events < 0) return PSC_E_ARG;
     DevGuard dg(B->device);
-    // every member with events left takes part in each batched event
-    for (int64_t e = 0; e < n_events; ++e) {
+    // every member with events left takes part
+    for (int64_t e = 0; e < n_events; e += kSmallEvents) {
         int rc;
-        if (batch_event(B, INFINITY, &rc) == 0) break;
+        if (!batch_advance(B, INFINITY, n_events - e, &rc)) break;
         if (rc) return rc;
     }
     return PSC_OK;
@@ -295,7 +461,7 @@ int psc_batch_run(psc_batch* B, double t_end)
     DevGuard dg(B->device);
     for (;;) {
         int rc;
-        if (batch_event(B, t_end, &rc) == 0) break;
+        if (!batch_advance(B, t_end, kSmallEvents, &rc)) break;
         if (rc) return rc;
     }
     for (int i = 0; i < kBatchMax; ++i) {
@@ -328,7 +494,7 @@ int psc_batch_autotune(psc_batch* B, int64_t max_rounds, psc_batch_tune_result* 
         if (time_it && cudaEventRecord(a, B->stream) != cudaSuccess) return PSC_E_CUDA;
         for (; done < n; ++done) {
             int r;
-            if (batch_event(B, INFINITY, &r) == 0) break;
+            if (batch_event(B, INFINITY, true, &r) == 0) break;
             if (r) return r;
         }
         budget -= done;
@@ -373,6 +539,31 @@ int psc_batch_autotune(psc_batch* B, int64_t max_rounds, psc_batch_tune_result* 
         if (!(rc = rounds(span, true, &us)) && us < best_us) { best_us = us; best_r = period; }
     }
     B->resort_period = best_r;
+    // the members' stretches against the best of these launches
+    B->use_stretches = true;
+    if (!rc && budget >= W) {
+        auto stretch = [&](bool time_it, double* us) -> int {
+            if (time_it && cudaEventRecord(a, B->stream) != cudaSuccess) return PSC_E_CUDA;
+            int r;
+            const bool any = batch_advance(B, INFINITY, W, &r);
+            if (r || !any) return r;
+            budget -= W;
+            out->rounds += W;
+            if (!time_it) return PSC_OK;
+            if (cudaEventRecord(b, B->stream) != cudaSuccess || cudaEventSynchronize(b) != cudaSuccess)
+                return PSC_E_CUDA;
+            float ms = 0.f;
+            if (cudaEventElapsedTime(&ms, a, b) != cudaSuccess) return PSC_E_CUDA;
+            out->trials++;
+            *us = 1e3 * (double)ms / (double)W;
+            return PSC_OK;
+        };
+        double us = INFINITY;
+        if (budget >= 2 * W) rc = stretch(false, nullptr);
+        if (!rc) rc = stretch(true, &us);
+        if (!rc && us < best_us) best_us = us;
+        else B->use_stretches = false;
+    }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     out->threads = best_t;
@@ -390,6 +581,11 @@ void psc_batch_destroy(psc_batch* B)
         cudaStreamSynchronize(B->stream);
         cudaFree(B->tmpl_ev);
         cudaFree(B->tmpl_rc);
+        cudaFree(B->args_d);
+        cudaFree(B->group_d);
+        cudaFree(B->counts_d);
+        if (B->counts_h) cudaFreeHost(B->counts_h);
+        if (B->counts_ev) cudaEventDestroy(B->counts_ev);
         if (B->own_stream) cudaStreamDestroy(B->stream);
     }
     delete B;
@@ -568,7 +764,9 @@ int psc_server_step(psc_server* S, int32_t n_events, int32_t* n_active, int32_t*
             continue;
         }
         psc_device_bytes(L, &bytes);
-        rc = batch_add_until(S->batch, L, q.r.t_end);
+        int64_t extra = 0;
+        rc = batch_add_until(S->batch, L, q.r.t_end, S->max_bytes - S->used - bytes, &extra);
+        bytes += extra;
         if (rc) {
             psc_lattice_destroy(L);
             Outcome& o = S->done[q.ticket];
@@ -589,9 +787,9 @@ int psc_server_step(psc_server* S, int32_t n_events, int32_t* n_active, int32_t*
         S->queue.pop_front();
     }
     // advance every running simulation by up to n_events of its events
-    for (int32_t e = 0; e < n_events; ++e) {
+    for (int64_t e = 0; e < n_events; e += kSmallEvents) {
         int rc;
-        if (batch_event(S->batch, INFINITY, &rc) == 0) break;
+        if (!batch_advance(S->batch, INFINITY, n_events - e, &rc)) break;
         if (rc) return rc;
     }
     // retire the finished ones

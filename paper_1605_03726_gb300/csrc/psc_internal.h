@@ -288,6 +288,7 @@ struct SmallArgs {
     int32_t nsp;
     int32_t collect_stats;
     int32_t build_map;         // the map has to be built first
+    int32_t blocks;            // blocks of the lattice's group (batched launches)
     uint32_t general;          // bit s: species s has reactions
     uint32_t fo2;              // bit s: a first-order reaction of s has two products
     uint32_t mapped;           // bit s: s can be a second-order partner
@@ -440,6 +441,11 @@ void launch_births(const EventArgs& a, cudaStream_t st);
 // Most blocks of a stretch on the current device: as one cluster, as a
 // cooperative grid (0: not at all).  Sets the kernels' attributes there.
 void small_limits(int sm_count, int* cluster, int* grid);
+// stretches of many lattices in one launch of `blocks` blocks: args on the
+// device per lattice, group[block] = (lattice, first block of its group)
+int small_batch_blocks(int sm_count);       // most blocks on the current device (0: not at all)
+cudaError_t launch_small_batch(const SmallArgs* args, const int2* group, int32_t* counts, int blocks, bool births,
+                               cudaStream_t st);
 cudaError_t launch_small(const SmallArgs& A, int blocks, int threads, bool cluster, cudaStream_t st);
 void launch_fill_u32(uint32_t* p, uint32_t value, size_t n, int blocks, cudaStream_t st);
 // molecule r (ids in species order, species s owning [offsets[s],

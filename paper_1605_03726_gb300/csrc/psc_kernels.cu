@@ -679,20 +679,20 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
-// Grid barrier: block 0 adds 2^31 - (blocks - 1), every other block adds 1,
+// Barrier of nblk blocks: block 0 adds 2^31 - (blocks - 1), every other adds 1,
 // so the top bit of the arrival word flips exactly when all have arrived.
 // The wait is bounded by timeout_ns of wall time (one second unless the
 // caller sets it) and by a spin count: on time-out the block raises
 // kErrBarrierTimeout and every thread of it returns false.  `phantom` counts
 // arrivals awaited from blocks that do not exist (0 outside tests): with
 // phantom > 0 the bit never flips and every block waits out its bound.
-__device__ __forceinline__ bool grid_barrier(BarrierState* bs, int32_t* err, uint64_t timeout_ns,
-                                             uint32_t phantom)
+__device__ __forceinline__ bool block_barrier(BarrierState* bs, int32_t* err, uint64_t timeout_ns,
+                                              uint32_t phantom, int blk, int nblk)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned int inc = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u + phantom) : 1u;
+        const unsigned int inc = blk == 0 ? 0x80000000u - ((unsigned)nblk - 1u + phantom) : 1u;
         __threadfence();
         const unsigned int old = atomicAdd(&bs->arrive, inc);
         volatile unsigned int* word = &bs->arrive;
@@ -715,6 +715,12 @@ __device__ __forceinline__ bool grid_barrier(BarrierState* bs, int32_t* err, uin
     }
     __syncthreads();
     return ok != 0;
+}
+
+// the same for all blocks of the launch
+__device__ __forceinline__ bool grid_barrier(BarrierState* bs, int32_t* err, uint64_t timeout_ns, uint32_t phantom)
+{
+    return block_barrier(bs, err, timeout_ns, phantom, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // packed claim state of one molecule: bit 31 claimed, bits 27-30 direction,

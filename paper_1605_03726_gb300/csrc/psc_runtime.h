@@ -215,6 +215,11 @@ EventArgs event_args(const psc_lattice* L, int s);
 ReconcileArgs reconcile_args(const psc_lattice* L, int x);
 bool next_event(const psc_lattice* L, int* s_out, double* t_out);
 int check_device(psc_lattice* L);
+// stretches of k_small_run (and of batches): buffers still lacking, their
+// allocation, the arguments but the events
+int64_t small_lacks(const psc_lattice* L, bool scratch);
+int small_buffers(psc_lattice* L, bool lists, bool scratch);
+void small_args(psc_lattice* L, bool reacts, SmallArgs* A);
 // every claim word free again (after stretches of k_walk_run), as the other kernels want them
 int claims_free(psc_lattice* L);
 // queue events in scheduler order until max_events or the next event lies after t_end

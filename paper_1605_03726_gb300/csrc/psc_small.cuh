@@ -55,14 +55,25 @@ __device__ __forceinline__ void cluster_barrier()
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <bool CLUSTER>
-__device__ __forceinline__ bool small_barrier(const SmallArgs& A)
+// The blocks of a stretch: all of the launch, as one cluster or a cooperative
+// grid, or a group of the blocks of a batched launch.
+enum SmallMode { kSmallInCluster, kSmallInGrid, kSmallInGroup };
+struct SmallBlocks {
+    int blk, nblk;
+};
+
+template <SmallMode MODE>
+__device__ __forceinline__ bool small_barrier(const SmallArgs& A, const SmallBlocks& B)
 {
-    if (CLUSTER) {
+    if (MODE == kSmallInCluster) {
         cluster_barrier();
         return true;
     }
-    return grid_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, 0u);
+    if (MODE == kSmallInGroup && B.nblk == 1) {
+        __syncthreads();                                        // what a block wrote, the block sees
+        return true;
+    }
+    return block_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, 0u, B.blk, B.nblk);
 }
 
 // molecule (id, img) on voxel v joins list y
@@ -301,8 +312,8 @@ __device__ __forceinline__ void small_commit(const SmallArgs& A, const EventArgs
 // all (lists that grew far past their estimates) the blocks pack there too.
 // The caller has a barrier before, if counts were read, and one after, if the
 // stretch goes on.
-template <bool CLUSTER>
-__device__ bool small_close(const SmallArgs& A, SmallShared& S, int t0, int stride)
+template <SmallMode MODE>
+__device__ bool small_close(const SmallArgs& A, SmallShared& S, const SmallBlocks& B, int t0, int stride)
 {
     __shared__ int32_t s_warp[32];
     const ModelDev& M = S.model;
@@ -314,7 +325,7 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, int t0, int stri
     int64_t total = 0;
     for (int x = 0; x < A.nsp; ++x) total += S.k[x];
     if (total == 0) return true;
-    const bool fits = !CLUSTER && total <= A.scratch_n;
+    const bool fits = MODE != kSmallInCluster && total <= A.scratch_n;
     int32_t base = 0;
     for (int x = 0; fits && x < A.nsp; ++x) {
         if (S.k[x] <= 0) continue;
@@ -329,7 +340,7 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, int t0, int stri
         }
         base += S.k[x];
     }
-    if (!CLUSTER && !small_barrier<CLUSTER>(A)) return false;
+    if (MODE != kSmallInCluster && !small_barrier<MODE>(A, B)) return false;
     base = 0;
     for (int x = 0; fits && x < A.nsp; ++x) {
         if (S.k[x] <= 0) continue;
@@ -350,7 +361,7 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, int t0, int stri
         }
         base += S.k[x];
     }
-    for (int x = blockIdx.x; !fits && x < A.nsp; x += gridDim.x) {
+    for (int x = B.blk; !fits && x < A.nsp; x += B.nblk) {
         if (S.k[x] <= 0) continue;
         const SpeciesList list = M.lists[x];
         const int32_t n = S.n[x];
@@ -391,9 +402,9 @@ constexpr int kSmallCarry = 2;              // molecules a thread carries in reg
 // molecules (idx = t0 + c * stride), loaded by the caller; n: the list's
 // length.  `next`: null, or the arguments of the next event, whose entries of
 // this thread nobody else changes: they are loaded before the barrier.
-template <bool GENERAL, bool CLUSTER>
-__device__ __forceinline__ bool small_event(const SmallArgs& A, const EventArgs& a, const ModelDev& M, uint32_t g,
-                                            int t0, int stride, int n, SmallMol (&m)[kSmallCarry],
+template <bool GENERAL, SmallMode MODE>
+__device__ __forceinline__ bool small_event(const SmallArgs& A, const SmallBlocks& B, const EventArgs& a,
+                                            const ModelDev& M, uint32_t g, int t0, int stride, int n, SmallMol (&m)[kSmallCarry],
                                             const EventArgs* next)
 {
     unsigned n_att = 0, n_col = 0, n_acc = 0, n_fire = 0, n_hop = 0, n_r2 = 0, n_r1 = 0;
@@ -417,7 +428,7 @@ __device__ __forceinline__ bool small_event(const SmallArgs& A, const EventArgs&
         }
         a.dec[idx] = (uint8_t)w.dec;                            // read back by this thread
     }
-    if (!small_barrier<CLUSTER>(A)) return false;
+    if (!small_barrier<MODE>(A, B)) return false;
 #pragma unroll
     for (int c = 0; c < kSmallCarry; ++c)
         if (m[c].dec != kDecNone) small_commit<GENERAL>(A, a, M, g, t0 + c * stride, m[c], n_hop, n_r2, n_r1);
@@ -455,16 +466,15 @@ __device__ __forceinline__ bool small_event(const SmallArgs& A, const EventArgs&
             flush_stat(&A.sc->stats[kStatReactions1], n_r1);
         }
     }
-    return small_barrier<CLUSTER>(A);
+    return small_barrier<MODE>(A, B);
 }
 
-template <bool CLUSTER>
-__global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(const SmallArgs A)
+template <SmallMode MODE>
+__device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, const SmallBlocks& B)
 {
-    __shared__ SmallShared S;
     // a list is dealt out warp by warp over the blocks, so that a short one
     // keeps every SM of the launch busy
-    const int blk = blockIdx.x, nblk = gridDim.x;               // one cluster, or the grid
+    const int blk = B.blk, nblk = B.nblk;
     const int lane = (int)threadIdx.x & 31;
     const int t0 = (((int)threadIdx.x >> 5) * nblk + blk) * 32 + lane;
     const int stride = nblk * (int)blockDim.x;
@@ -492,7 +502,7 @@ __global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(co
         S.n[threadIdx.x] = A.sc->counts[threadIdx.x];
     }
     __syncthreads();
-    if (!small_barrier<CLUSTER>(A)) return;
+    if (!small_barrier<MODE>(A, B)) return;
     const ModelDev& M = S.model;
     bool prev_fo2 = false, loaded = false;
     SmallMol m[kSmallCarry];
@@ -529,36 +539,82 @@ __global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(co
             if (born) {
                 if (blk == 0) births_body(S.ev[S.seq[e - 1]], A.slot, A.mapped);
                 prev_fo2 = false;
-                if (!small_barrier<CLUSTER>(A)) return;
+                if (!small_barrier<MODE>(A, B)) return;
                 continue;
             }
             if (last) break;
-            const bool tight = __any_sync(0xFFFFFFFFu, holes > 0) &&
-                               (__any_sync(0xFFFFFFFFu, room < 2 * (int64_t)n) ||
-                                (!CLUSTER && (int64_t)__reduce_add_sync(0xFFFFFFFFu, holes) + 2 * (int64_t)n >
-                                                 (int64_t)A.scratch_n));
+            // (a list without tombstones has room for what the event can add)
+            const bool tight = __any_sync(0xFFFFFFFFu, holes > 0 && room < 2 * (int64_t)n) ||
+                               (A.scratch_n > 0 && __any_sync(0xFFFFFFFFu, holes > 0) &&
+                                (int64_t)__reduce_add_sync(0xFFFFFFFFu, holes) + 2 * (int64_t)n >
+                                    (int64_t)A.scratch_n);
             if (!tight) break;
-            if (!small_barrier<CLUSTER>(A)) return;             // the counts are read
-            if (!small_close<CLUSTER>(A, S, t0, stride)) return;
-            if (!small_barrier<CLUSTER>(A)) return;
+            if (!small_barrier<MODE>(A, B)) return;             // the counts are read
+            if (!small_close<MODE>(A, S, B, t0, stride)) return;
+            if (!small_barrier<MODE>(A, B)) return;
             if (t0 < kMaxSpecies) A.sc->hole_n[t0] = A.sc->surv_n[t0] = 0;
         }
         if (last) {
-            if (A.general) small_close<CLUSTER>(A, S, t0, stride);
+            if (A.general) small_close<MODE>(A, S, B, t0, stride);
             return;
         }
         n = min(n, a.list.cap);
         if ((A.general >> s) & 1u) {
             // word g & 1 was last read an event ago
             if (t0 == 0) A.sc->touched[g & 1u] = 0u;
-            if (!small_event<true, CLUSTER>(A, a, M, g, t0, stride, n, m, nullptr)) return;
+            if (!small_event<true, MODE>(A, B, a, M, g, t0, stride, n, m, nullptr)) return;
         } else {
             const EventArgs* next = (A.general || e + 1 == A.n_events) ? nullptr : &S.ev[S.seq[e + 1]];
-            if (!small_event<false, CLUSTER>(A, a, M, g, t0, stride, n, m, next)) return;
+            if (!small_event<false, MODE>(A, B, a, M, g, t0, stride, n, m, next)) return;
             loaded = next != nullptr;
         }
         prev_fo2 = (A.fo2 >> s) & 1u;
     }
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(const SmallArgs A)
+{
+    __shared__ SmallShared S;
+    small_run<CLUSTER ? kSmallInCluster : kSmallInGrid>(A, S, SmallBlocks{(int)blockIdx.x, (int)gridDim.x});
+}
+
+// Stretches of many lattices in one cooperative launch, each with a group of
+// consecutive blocks and at its own pace: no lattice waits for another.
+// counts: list lengths afterwards, [lattice][kMaxSpecies], for the next
+// launch's groups.
+__global__ void __launch_bounds__(kSmallThreads, 2) k_small_batch(const SmallArgs* args, const int2* group,
+                                                                  int32_t* counts)
+{
+    __shared__ SmallShared S;
+    __shared__ SmallArgs A;
+    const int2 mine = group[blockIdx.x];                        // lattice, first block of its group
+    small_copy(&A, args + mine.x, sizeof(SmallArgs));
+    __syncthreads();
+    const SmallBlocks B{(int)blockIdx.x - mine.y, A.blocks};
+    small_run<kSmallInGroup>(A, S, B);
+    if (A.general && B.blk == 0 && (int)threadIdx.x < A.nsp)
+        counts[mine.x * kMaxSpecies + threadIdx.x] = S.n[threadIdx.x] - S.k[threadIdx.x];
+}
+
+int small_batch_blocks(int sm_count)
+{
+    const void* f = (const void*)k_small_batch;
+    const int smem = kBirthSortMax * (int)sizeof(unsigned long long);
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kSmallThreads, smem) != cudaSuccess)
+        per_sm = 0;
+    cudaGetLastError();
+    return per_sm * sm_count;
+}
+
+cudaError_t launch_small_batch(const SmallArgs* args, const int2* group, int32_t* counts, int blocks, bool births,
+                               cudaStream_t st)
+{
+    void* p[] = {&args, &group, &counts};
+    return cudaLaunchCooperativeKernel((const void*)k_small_batch, dim3(blocks), dim3(kSmallThreads), p,
+                                       births ? (size_t)kBirthSortMax * sizeof(unsigned long long) : 0, st);
 }
 
 static void small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int blocks, int threads, bool cluster, bool births)

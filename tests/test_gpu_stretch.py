@@ -8,6 +8,7 @@ lists behind the voxel -> slot map), reactions fast enough that tombstones fill
 the lists' room several times within a stretch, births, immobile partners,
 compartments, and walkers between species with reactions.
 """
+import numpy as np
 import pytest
 
 import models
@@ -95,3 +96,38 @@ def test_stretch_in_a_cell_with_compartments():
         g.run_events(n)
         o.run_events(n)
         assert_same(g, o, n)
+
+
+def test_members_in_stretches_and_in_launches_together():
+    # batches: a member that keeps per-event launches (persistent = -1) beside members
+    # that run in stretches, calls longer than a stretch, a member without
+    # reactions, and a batch larger than one launch has blocks for
+    import torch
+    stream = torch.cuda.Stream()
+    B = psc.Batch(stream=stream.cuda_stream)
+    pairs = []
+    for r in range(310):
+        e = 8 + 2 * (r % 5) if r >= 6 else (24, 30, 40, 26, 28, 34)[r]
+        both = []
+        for st in (stream.cuda_stream, None):
+            L = psc.Lattice(e, e, e, voxel_radius=1e-8, stream=st)
+            L.set_options(claim_table=1, resort_period=-1, persistent=-1 if r == 1 else 1)
+            if r == 2:
+                L.add_species(1e-12, 3000)
+            else:
+                models.reaction_diffusion_ab(L, int(0.06 * e ** 3), int(0.04 * e ** 3))
+            L.populate(40 + r)
+            both.append(L)
+        B.add(both[0])
+        pairs.append(both)
+    for n in (3, 530):
+        B.run_events(n)
+        for r, (m, solo) in enumerate(pairs):
+            if r > 8 and r % 29:
+                continue
+            solo.run_events(n)
+            assert np.array_equal(m.grid(), solo.grid()) and m.time() == solo.time()
+            for s in range(m.n_species):
+                a, b = m.coords(s), solo.coords(s)
+                assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    B.close()
