@@ -144,20 +144,21 @@ typedef struct {
     int32_t claim_table;      /* before populate: 1 = one claim word per voxel,
                                  2 = hash table of claims, 0/-1 = by size (a
                                  word per voxel up to 2^22 voxels, where the
-                                 two tables would be as large, or without
-                                 reactions: up to 28 million voxels where the
-                                 molecules fit in shared memory, above that
-                                 from 262,144 molecules of a species on, if
-                                 the memory is there)                          */
+                                 two tables would be as large; where the events
+                                 run in stretches, see persistent; without
+                                 reactions also from 262,144 molecules of a
+                                 species on; the last two if the memory is
+                                 there)                                        */
     int32_t persistent;       /* 1 = run stretches of events in one launch
                                  (default): of a lattice without reactions and
                                  compartments whose molecules fit in shared
                                  memory (up to 2.8 million, 28 million voxels),
-                                 all its species in turn; of any species, in
-                                 scheduler order, where the lists are short (up
-                                 to 131,072 molecules, with reactions 300,000,
-                                 partners included) and claims have a word per
-                                 voxel; of a species without reactions otherwise;
+                                 all its species in turn; of any lattice of up
+                                 to 2^26 voxels with a claim word per voxel, its
+                                 species in scheduler order, while no mobile
+                                 species has more than 2^22 molecules (without
+                                 reactions 131,072); of a species without
+                                 reactions otherwise;
                                  -1 = claim and commit launches per event       */
     int32_t slot_map;         /* home slot of a claim in the hash table:
                                  1 = hashed voxel index (default), 2 = Morton

@@ -162,6 +162,8 @@ int sort_first(psc_lattice* L, int s)
 // start the next one every 64 events.  The host queues events far faster than
 // the device runs them; once a copy is 256 events old the host waits for it,
 // so the estimates stay recent (the device still has that many queued).
+constexpr size_t kCountsBytes = offsetof(Scalars, next_id) + sizeof(uint32_t);   // counts to next_id
+
 void refresh_estimates(psc_lattice* L)
 {
     if (!L->counts_h) return;
@@ -177,14 +179,15 @@ void refresh_estimates(psc_lattice* L)
             L->est[s] = L->counts_h[s];
             L->grid_class[s] = grid_class_for(L, s, L->est[s], L->grid_class[s]);
         }
+        L->next_id_known = (uint32_t)L->counts_h[offsetof(Scalars, next_id) / 4];
+        L->next_id_g = L->counts_g;
         L->counts_pending = false;
     }
     if (L->g - L->counts_g < 64u) return;
-    if (cudaMemcpyAsync(L->counts_h, L->sc->counts, sizeof(int32_t) * (size_t)L->nsp, cudaMemcpyDeviceToHost,
-                        L->stream) != cudaSuccess ||
+    if (cudaMemcpyAsync(L->counts_h, L->sc, kCountsBytes, cudaMemcpyDeviceToHost, L->stream) != cudaSuccess ||
         cudaEventRecord(L->counts_ev, L->stream) != cudaSuccess)
         return;
-    L->d2h += sizeof(int32_t) * (size_t)L->nsp;
+    L->d2h += kCountsBytes;
     L->counts_pending = true;
     L->counts_g = L->g;
 }
@@ -271,7 +274,7 @@ void span_close(psc_lattice* L, cudaEvent_t a, int kind, int64_t events = 1)
 int resort(psc_lattice* L, int s)
 {
     L->placed_order[s] = false;
-    L->small.map_holds = false;
+    if (int rc = grid_current(L, true)) return rc;
     const int blocks = list_blocks(L, s);
     const SpeciesList& list = L->model_h.lists[s];
     const int32_t* count = &L->sc->counts[s];
@@ -326,7 +329,6 @@ ReconcileArgs reconcile_args(const psc_lattice* L, int x)
 
 int enqueue_event(psc_lattice* L, int s)
 {
-    L->small.map_holds = false;
     const EventArgs a = event_args(L, s);
     const int threads = L->opt.block_threads;
     const int blocks = list_blocks(L, s);
@@ -751,7 +753,6 @@ static int small_setup(psc_lattice* L)
         };
         for (int x = 0; x < L->nsp; ++x) {
             if (L->pair[s][x] < 0) continue;
-            B.mapped |= 1u << s;
             products(L->rx[L->pair[s][x]]);
         }
         for (int u = 0; u < L->sp[s].n_fo; ++u) products(L->rx[L->sp[s].fo[u]]);
@@ -769,63 +770,81 @@ static int small_setup(psc_lattice* L)
     return PSC_OK;
 }
 
-// Can an event of species s run in a stretch of k_small_run?  Its own list and
-// its partners' hold at most kSmallList entries (by the estimates: a list that
-// has grown past it in the meantime only takes longer).
-static bool small_fits(psc_lattice* L, int s)
+// No id is at or above this: an event makes at most births_cap of them.
+int64_t ids_bound(const psc_lattice* L)
 {
-    if (!L->claim || L->opt.persistent <= 0 || L->opt.barrier_phantom > 0) return false;
+    return L->next_id_known + (L->births_cap > 1 ? (int64_t)(L->g - L->next_id_g) * L->births_cap : 0);
+}
+
+// Do the lattice's events run in stretches of k_small_run?  Every mobile
+// species' list holds at most kSmallList molecules, in lattices without
+// reactions kSmallWalk (by the estimates: a list that has grown past it in the
+// meantime only takes longer).  All of them or none: the other kernels want
+// mirrors and codes, which these stretches bring up to date by a pass over the
+// lattice.
+static bool small_fits(psc_lattice* L)
+{
+    if (!L->claim || L->opt.persistent <= 0 || L->opt.barrier_phantom > 0 || L->V > kCellVoxels ||
+        ids_bound(L) > kCellIds)
+        return false;
+    for (int s = 0; s < L->nsp; ++s)
+        if (L->model_h.lists[s].cap > kCellVoxels) return false;
     if (!L->shapes_known) device_shapes(L);
     if (L->small.cluster <= 0 || L->small.grid <= 0) return false;
-    if (L->general[s]) {
+    const int64_t most = L->nrx > 0 ? kSmallList : kSmallWalk;
+    for (int s = 0; s < L->nsp; ++s) {
+        if (!(L->sp[s].D > 0.0)) continue;
+        if (L->est[s] > most) return false;
         // kernel timing keeps the phases of a reaction event apart; without the background
         // copies of the list lengths nothing is known of them
-        if (L->opt.time_kernels > 0 || !L->counts_h) return false;
-        for (int x : L->reconcile[s])
-            if (L->est[x] > kSmallList) return false;
-        return true;
+        if (L->general[s] && (L->opt.time_kernels > 0 || !L->counts_h)) return false;
+        if (L->general[s]) continue;
+        if (L->opt.run_per_thread > 0) return false; // the caller picks the molecule-list kernel's shape
+        TilePlan P{};
+        if (L->opt.tiles > 0 && tile_plan(L, s, &P)) return false;
     }
-    if (L->opt.run_per_thread > 0) return false;     // the caller picks the molecule-list kernel's shape
-    if (L->est[s] > kSmallWalk) return false;
-    TilePlan P{};
-    return !(L->opt.tiles > 0 && tile_plan(L, s, &P));
+    return true;
 }
 
 // Bytes of the buffers a lattice's stretches of k_small_run still lack, and
 // their allocation; scratch: lists are closed up in a grid or a group of blocks.
 static int32_t small_scratch(const psc_lattice* L)
 {
-    int64_t most = 0;
-    for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, L->model_h.lists[x].cap);
-    return (int32_t)std::min<int64_t>(4 * kSmallList, 4 * most + 4096);
+    // two tombstones per molecule of the due species and event, and as many
+    // again from the events before; lists may have grown by half
+    int64_t cap = 0, est = 0;
+    for (int x = 0; x < L->nsp; ++x) {
+        cap = std::max<int64_t>(cap, L->model_h.lists[x].cap);
+        if (L->sp[x].D > 0.0) est = std::max<int64_t>(est, L->est[x]);
+    }
+    return (int32_t)std::min<int64_t>(std::max<int64_t>(6 * est, 1200000), 4 * cap + 4096);
 }
 
 int64_t small_lacks(const psc_lattice* L, bool scratch)
 {
     const auto& B = L->small;
-    bool pairs = false, general = false;
-    for (int s = 0; s < L->nsp; ++s) {
-        general = general || L->general[s];
-        for (int x = 0; x < L->nsp; ++x) pairs = pairs || L->pair[s][x] >= 0;
-    }
+    bool general = false;
+    for (int s = 0; s < L->nsp; ++s) general = general || L->general[s];
     int64_t b = B.ev ? 0 : (int64_t)L->nsp * (int64_t)sizeof(EventArgs);
-    if (pairs && !B.slot) b += L->V * 4;
+    if (!B.cell) b += (int64_t)L->mirror_n * 128;
     if (scratch && general && !B.scratch) b += (int64_t)small_scratch(L) * 8;
     return b;
 }
 
-int small_buffers(psc_lattice* L, bool lists, bool scratch)
+int small_buffers(psc_lattice* L, bool scratch)
 {
     auto& B = L->small;
     if (!B.ev) {
         const int rc = small_setup(L);
         if (rc) return rc;
     }
-    if (lists && B.mapped && !B.slot) {
-        B.slot = (uint32_t*)dev_alloc(L, (size_t)L->V * 4);
-        if (!B.slot) return PSC_E_NOMEM;
+    if (!B.cell) {
+        B.cell = (uint32_t*)dev_alloc(L, (size_t)L->mirror_n * 128);
+        if (!B.cell) return PSC_E_NOMEM;
     }
-    if (lists && scratch && B.general && !B.scratch) {
+    // (a list that has doubled since wants more)
+    if (scratch && B.general && (!B.scratch || (int64_t)small_scratch(L) > 2 * (int64_t)B.scratch_n)) {
+        if (B.scratch) dev_free_one(L, B.scratch);
         B.scratch_n = small_scratch(L);
         B.scratch = (int32_t*)dev_alloc(L, (size_t)B.scratch_n * 8);
         if (!B.scratch) {
@@ -836,14 +855,22 @@ int small_buffers(psc_lattice* L, bool lists, bool scratch)
     return PSC_OK;
 }
 
-// The arguments of a stretch but its events; reacts: they include reactions.
-void small_args(psc_lattice* L, bool reacts, SmallArgs* A)
+// The arguments of a stretch but its events; the cells are built if need be.
+int small_args(psc_lattice* L, SmallArgs* A)
 {
     auto& B = L->small;
+    if (!B.cells_hold) {
+        launch_cells_build(B.cell, L->bits, L->mirror_n, L->labels.empty() ? 1 : L->ncomp, L->model_d, L->sc->counts,
+                           L->nsp, L->geo, L->sm_count * 8, L->stream);
+        L->launches += 2;
+        if (int rc = cuda_fail(L, cudaPeekAtLastError())) return rc;
+        B.cells_hold = true;
+    }
+    B.grid_stale = true;
     A->ev = B.ev;
     A->model = L->model_d;
     A->sc = L->sc;
-    A->slot = B.slot;
+    A->cell = B.cell;
     A->holes = B.scratch;
     A->surv = B.scratch + B.scratch_n;
     A->scratch_n = B.scratch_n;
@@ -851,13 +878,24 @@ void small_args(psc_lattice* L, bool reacts, SmallArgs* A)
     A->barrier_timeout_ns = (uint64_t)L->opt.barrier_timeout_us * 1000ull;
     A->nsp = L->nsp;
     A->collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
-    if (!reacts) return;
     A->general = B.general;
     A->fo2 = B.fo2;
-    A->mapped = B.mapped;
     std::memcpy(A->products, B.products, sizeof(A->products));
-    A->build_map = B.map_holds ? 0 : 1;
-    B.map_holds = true;
+    return PSC_OK;
+}
+
+int grid_current(psc_lattice* L, bool leave)
+{
+    auto& B = L->small;
+    if (B.grid_stale) {
+        launch_cells_grid(B.cell, L->bits, L->mirror_n, L->labels.empty() ? 1 : L->ncomp, L->occ, L->geo,
+                          L->sm_count * 8, L->stream);
+        L->launches += 1;
+        B.grid_stale = false;
+        if (int rc = cuda_fail(L, cudaPeekAtLastError())) return rc;
+    }
+    if (leave) B.cells_hold = false;
+    return PSC_OK;
 }
 
 // A stretch of consecutive events, starting with species s at time t: one
@@ -865,42 +903,30 @@ void small_args(psc_lattice* L, bool reacts, SmallArgs* A)
 static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
 {
     auto& B = L->small;
-    bool lists = false, grid = false;                // a species with reactions may come up; a grid may
-    for (int x = 0; x < L->nsp; ++x) {
-        if (!(L->sp[x].D > 0.0) || !small_fits(L, x)) continue;
-        lists = lists || L->general[x];
-        grid = grid || L->est[x] > kSmallCluster;
-    }
-    int rc = small_buffers(L, lists, grid);
+    bool grid = false;                               // a stretch may take a grid
+    for (int x = 0; x < L->nsp; ++x) grid = grid || (L->sp[x].D > 0.0 && L->est[x] > kSmallCluster);
+    int rc = small_buffers(L, grid);
     if (rc) return rc;
     SmallArgs A{};
+    if ((rc = small_args(L, &A))) return rc;
     A.g = L->g;
     const int64_t limit = std::min<int64_t>(std::min<int64_t>(max_events, kSmallEvents),
                                             (int64_t)UINT32_MAX - L->g);
-    int8_t fits[kMaxSpecies] = {};                   // 0 not asked yet, 1 yes, -1 no
-    fits[s] = 1;
     int64_t longest = 0;
-    bool reacts = false;
-    for (;;) {
+    do {
         A.seq[A.n_events++] = (uint8_t)s;
         longest = std::max(longest, L->est[s]);
-        reacts = reacts || L->general[s];
         L->sp[s].done++;
         L->g++;
         L->clock = t;
-        if (A.n_events >= limit || !next_event(L, &s, &t) || t > t_end) break;
-        if (fits[s] == 0) fits[s] = small_fits(L, s) ? 1 : -1;
-        if (fits[s] < 0) break;
-    }
-    small_args(L, reacts, &A);
+    } while (A.n_events < limit && next_event(L, &s, &t) && t <= t_end);
     // the shape: a cluster of 16 blocks up to kSmallCluster entries (with fewer
     // blocks, or 128 threads in each, short lists got slower: 2621 walkers 3.9 us
-    // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM,
-    // of half the threads while they suffice (45,000 molecules 7.8 us per event
-    // against 8.2), and two per SM for the longest
+    // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM, of
+    // half the threads while they suffice
     const bool cluster = longest <= kSmallCluster;
     const int threads = !cluster && longest <= 65536 ? kSmallThreads / 2 : kSmallThreads;
-    const int blocks = cluster ? B.cluster : std::min(B.grid, longest <= 131072 ? L->sm_count : 2 * L->sm_count);
+    const int blocks = cluster ? B.cluster : B.grid;
     if (!cluster) rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream));
     if (rc) return rc;
     cudaEvent_t sp = span_open(L);
@@ -1403,9 +1429,16 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     for (int s = 0; s < L->nsp; ++s)
         open = open || (L->nrx == 0 && L->V > kWalkVoxels && L->sp[s].D > 0.0 && L->sp[s].n0 >= kOpenList &&
                         L->opt.subvolume <= 0);
+    // the rest, as far as their events run in stretches of k_small_run (tables and
+    // a launch per phase before: A + B <-> C of 2000 + 1000 molecules on 200^3 9.9 ->
+    // 3.9 us per event, 200,000 + 100,000 on 256^3 27.5 -> 15.8, 100,000 + 50,000 on
+    // 400^3 24.6 -> 12.9; 60,000 walkers on 400^3 15.9 -> 6.0)
+    bool stretch = L->stretches && L->V <= kCellVoxels && L->opt.subvolume <= 0;
+    for (int s = 0; s < L->nsp; ++s)
+        stretch = stretch && (!(L->sp[s].D > 0.0) || L->sp[s].n0 <= (L->nrx > 0 ? kSmallList : kSmallWalk));
     if (L->opt.claim_table == 1) direct = true;
-    if (L->opt.claim_table == 2 && hb_max > 0) direct = open = false;
-    if (open && !direct) {
+    if (L->opt.claim_table == 2 && hb_max > 0) direct = open = stretch = false;
+    if ((open || stretch) && !direct) {
         L->claim_n = L->V;
         L->claim = (uint32_t*)dev_alloc(L, V * sizeof(uint32_t));
         direct = L->claim != nullptr;                // no room: tables
@@ -1595,7 +1628,9 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         L->placed_order[s] = true;
     }
     L->counts_g = 0;
-    if (!L->counts_h && cudaMallocHost(&L->counts_h, sizeof(int32_t) * kMaxSpecies) != cudaSuccess) {
+    L->next_id_known = N;
+    L->next_id_g = 0;
+    if (!L->counts_h && cudaMallocHost(&L->counts_h, kCountsBytes) != cudaSuccess) {
         L->counts_h = nullptr;
         cudaGetLastError();
     }
@@ -1684,7 +1719,6 @@ static int single_event(psc_lattice* L, int s, double t)
     for (const auto& G : L->graphs1) {
         if (G.key != key) continue;
         set_index();
-        L->small.map_holds = false;
         int rc = cuda_fail(L, cudaGraphLaunch(G.exec, L->stream));
         if (rc) return rc;
         L->table_used[0] = G.table_used[0];
@@ -1816,7 +1850,6 @@ static int graph_run(psc_lattice* L, double t_end, int64_t room, int64_t* done)
         if (G.key != key) continue;
         launch_fill_u32(&L->sc->g_base, L->g, 1, 1, L->stream);
         L->g_dev = (int64_t)L->g;
-        L->small.map_holds = false;
         int rc = cuda_fail(L, cudaGraphLaunch(G.exec, L->stream));
         if (rc) return rc;
         for (int e = 0; e < K; ++e) advance(e);
@@ -1939,19 +1972,21 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
         }
         if (walk_fits(L, s)) {
             int64_t e = 0;
+            if (int rc = grid_current(L, true)) return rc;
             int rc = walk_stretch(L, s, t, t_end, max_events - queued, &e);
             if (rc) return rc;
             queued += e;
             continue;
         }
         if (int rc = claims_free(L)) return rc;
-        if (small_fits(L, s)) {
+        if (small_fits(L)) {
             int64_t e = 0;
             int rc = small_stretch(L, s, t, t_end, max_events - queued, &e);
             if (rc) return rc;
             queued += e;
             continue;
         }
+        if (int rc = grid_current(L, true)) return rc;
         int threads = 0, blocks = 0;
         const bool open = open_route(L, s);
         const int per = open ? 0 : run_width(L, s, &threads, &blocks);
@@ -2237,6 +2272,7 @@ int psc_grid(psc_lattice* L, uint16_t* occ)
     DevGuard dg(L->device);
     int rc = check_device(L);
     if (rc) return rc;
+    if ((rc = grid_current(L, false))) return rc;
     // exact codes: mirror-masked codes of species with reactions, then the
     // species without reactions from their lists
     uint16_t* tmp = (uint16_t*)dev_alloc(L, (size_t)L->V * 2);
@@ -2379,7 +2415,7 @@ int psc_device_bytes(const psc_lattice* L, int64_t* bytes)
     int64_t b = L->V * 2 + mwords * 4 * mirrors + 2 * ((mwords + 31) / 32) * 4 + (int64_t)sizeof(Scalars) +
                 (int64_t)sizeof(ModelDev);
     if (L->small.ev) b += (int64_t)L->nsp * (int64_t)sizeof(EventArgs);
-    if (L->small.slot) b += L->V * 4;
+    if (L->small.cell) b += mwords * 128;
     b += (int64_t)L->small.scratch_n * 8;
     if (L->claim) b += L->claim_n * 4;
     b += 2 * L->table_slots * 8;

@@ -48,11 +48,11 @@ struct psc_batch {
     bool use_stretches = true;
     SmallArgs* args_d = nullptr;          // [kBatchMax], device: one for each member that takes part
     int2* group_d = nullptr;              // [stretch_blocks]
-    int32_t* counts_d = nullptr;          // [kBatchMax][kMaxSpecies] list lengths after a stretch
+    int32_t* counts_d = nullptr;          // [kBatchMax][kSmallCounts] list lengths after a stretch
     int32_t* counts_h = nullptr;          // pinned copy, for the next stretch's groups
     cudaEvent_t counts_ev = nullptr;
     bool counts_pending = false;
-    std::vector<psc_lattice*> counts_of;  // whose lengths counts_h holds
+    std::vector<std::pair<psc_lattice*, uint32_t>> counts_of;  // whose lengths counts_h holds, after which event
 };
 
 namespace {
@@ -85,7 +85,7 @@ int batch_event(psc_batch* B, double t_cap, bool all, int* rc_out)
         double t;
         if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
         acts[na++] = {i, s, t};
-        if ((*rc_out = claims_free(L))) return 1;
+        if ((*rc_out = claims_free(L)) || (*rc_out = grid_current(L, true))) return 1;
         BatchItem& it = bl.item[bl.n++];
         it.rep = i;
         it.sel = s;
@@ -175,7 +175,6 @@ int batch_event(psc_batch* B, double t_cap, bool all, int* rc_out)
     }
     for (int a = 0; a < na; ++a) {
         psc_lattice* L = B->slot[acts[a].slot].L;
-        L->small.map_holds = false;
         L->sp[acts[a].s].done++;
         L->g++;
         L->clock = acts[a].t;
@@ -205,8 +204,8 @@ int stretch_buffers(psc_batch* B, psc_lattice* L)
     if (B->stretch_blocks == 0 || B->args_d) return PSC_OK;
     if (cudaMalloc(&B->args_d, sizeof(SmallArgs) * kBatchMax) != cudaSuccess ||
         cudaMalloc(&B->group_d, sizeof(int2) * (size_t)B->stretch_blocks) != cudaSuccess ||
-        cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kMaxSpecies) != cudaSuccess ||
-        cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kMaxSpecies) != cudaSuccess ||
+        cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
+        cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         B->stretch_blocks = 0;            // what was allocated goes with the batch
@@ -222,9 +221,12 @@ bool member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra
         return false;
     stretch_buffers(B, L);
     if (B->stretch_blocks <= 0) return false;
+    if (L->V > kCellVoxels) return false;
+    for (int s = 0; s < L->nsp; ++s)
+        if (L->model_h.lists[s].cap > kCellVoxels) return false;
     const int64_t lacks = small_lacks(L, true);
     if (lacks > room) return false;
-    if (small_buffers(L, true, true) != PSC_OK) {
+    if (small_buffers(L, true) != PSC_OK) {
         cudaGetLastError();
         L->sticky = PSC_OK;               // no room on the device: batched launches
         return false;
@@ -249,12 +251,15 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         }
         B->counts_pending = false;
         for (size_t r = 0; r < B->counts_of.size(); ++r) {
-            psc_lattice* L = B->counts_of[r];
+            psc_lattice* L = B->counts_of[r].first;
             bool member = false;
             for (int i = 0; i < kBatchMax && !member; ++i) member = B->slot[i].L == L;
-            for (int s = 0; member && s < L->nsp; ++s) {
-                const int32_t c = B->counts_h[r * kMaxSpecies + (size_t)s];
-                if (c >= 0) L->est[s] = c;
+            const int32_t* h = B->counts_h + r * kSmallCounts;
+            for (int s = 0; member && s < L->nsp; ++s)
+                if (h[s] >= 0) L->est[s] = h[s];
+            if (member && h[kMaxSpecies] > 0) {
+                L->next_id_known = h[kMaxSpecies];
+                L->next_id_g = B->counts_of[r].second;
             }
         }
     }
@@ -265,12 +270,16 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
     for (int i = 0; i < kBatchMax; ++i) {
         psc_lattice* L = B->slot[i].L;
         if (!L || L->sticky || !B->slot[i].stretch) continue;
+        if (ids_bound(L) > kCellIds) {    // no more ids for the cells' claims
+            B->slot[i].stretch = false;
+            continue;
+        }
         int s;
         double t;
         if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
         if ((*rc_out = claims_free(L))) return 1;
         SmallArgs A{};
-        small_args(L, true, &A);
+        if ((*rc_out = small_args(L, &A))) return 1;
         A.g = L->g;
         const int64_t limit = std::min<int64_t>(std::min<int64_t>(n_events, kSmallEvents), (int64_t)UINT32_MAX - L->g);
         double molecules = 0.0;
@@ -286,7 +295,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         L->launches += 1;
         work.push_back(molecules / A.n_events);
         args.push_back(A);
-        B->counts_of.push_back(L);
+        B->counts_of.emplace_back(L, L->g);
     }
     if (args.empty()) return 0;
     const int total = (int)args.size();
@@ -311,7 +320,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
                             cudaMemcpyHostToDevice, B->stream) != cudaSuccess ||
             cudaMemcpyAsync(B->group_d, group.data(), sizeof(int2) * group.size(), cudaMemcpyHostToDevice, B->stream) !=
                 cudaSuccess ||
-            (l == 0 && cudaMemsetAsync(B->counts_d, 0xFF, sizeof(int32_t) * kMaxSpecies * (size_t)total, B->stream) !=
+            (l == 0 && cudaMemsetAsync(B->counts_d, 0xFF, sizeof(int32_t) * kSmallCounts * (size_t)total, B->stream) !=
                            cudaSuccess) ||
             launch_small_batch(B->args_d, B->group_d, B->counts_d, (int)group.size(), births, B->stream) !=
                 cudaSuccess) {
@@ -320,7 +329,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         }
         B->launches += 1;
     }
-    if (cudaMemcpyAsync(B->counts_h, B->counts_d, sizeof(int32_t) * kMaxSpecies * (size_t)total,
+    if (cudaMemcpyAsync(B->counts_h, B->counts_d, sizeof(int32_t) * kSmallCounts * (size_t)total,
                         cudaMemcpyDeviceToHost, B->stream) != cudaSuccess ||
         cudaEventRecord(B->counts_ev, B->stream) != cudaSuccess)
         *rc_out = PSC_E_CUDA;

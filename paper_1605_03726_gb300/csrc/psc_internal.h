@@ -263,21 +263,25 @@ struct ReconcileArgs {
 // per-voxel claim words (k_small_run).
 constexpr int kSmallEvents = 512;          // events of one launch
 constexpr int kSmallThreads = 512;         // threads of a block
-// The longest list of a stretch.  With reactions (30 % crowding): 205,000
-// molecules take 16.5 us per event against 24.9 in per-event launches, 400,000
-// 26 to 29 against 30, and 839,000 57 against 42 (twice the threads in flight
-// there, and Morton re-sorts).  Without (128^3): 63,000 walkers 8.4 against
-// 10.8 in the molecule-list kernel, 210,000 14.4 against 13.0.
-constexpr int64_t kSmallList = 300000;     // of a species with reactions, or a partner
-constexpr int64_t kSmallWalk = 131072;     // of one without
+constexpr int kSmallCounts = kMaxSpecies + 1;      // list lengths and next id, per lattice of a batch
+// limits of a cell's fields
+constexpr int64_t kCellVoxels = 1ll << 26; // (list slots)
+constexpr int64_t kCellIds = (1ll << 27) - (1ll << 23);    // next id when a stretch starts; a stretch makes at
+                                                           // most 512 x 8192 (births_cap) of them
+// The longest list of a mobile species of a lattice that runs in stretches:
+// with reactions as far as was measured (3.2M molecules 126 us per event, 180 in
+// per-event launches), else where the molecule-list and tile kernels take over
+// (128^3: 63,000 walkers 6.0 us per event against 10.8, 210,000 14.4 against 13.0).
+constexpr int64_t kSmallList = 1 << 22;
+constexpr int64_t kSmallWalk = 131072;
 // The longest list that runs in one cluster of 16 blocks: 16,000 molecules take
-// 3.6 us per event there and 4.8 in a grid, 30,000 13.1 and 7.8.
+// 3.1 us per event there and 4.8 in a grid, 30,000 13.1 and 6.8.
 constexpr int64_t kSmallCluster = 16384;
 struct SmallArgs {
     const EventArgs* ev;       // [nsp] templates on the device (event_args with g unset)
     const ModelDev* model;
     Scalars* sc;
-    uint32_t* slot;            // per voxel: the list slot of its molecule, for species in `mapped`
+    uint32_t* cell;            // a word per voxel (psc_small.cuh)
     int32_t* holes;            // [scratch_n] slots of tombstones and of the entries that take them
     int32_t* surv;
     int32_t scratch_n;
@@ -287,11 +291,9 @@ struct SmallArgs {
     int32_t n_events;
     int32_t nsp;
     int32_t collect_stats;
-    int32_t build_map;         // the map has to be built first
     int32_t blocks;            // blocks of the lattice's group (batched launches)
     uint32_t general;          // bit s: species s has reactions
     uint32_t fo2;              // bit s: a first-order reaction of s has two products
-    uint32_t mapped;           // bit s: s can be a second-order partner
     uint32_t products[kMaxSpecies];        // bit y: an event of s may append to list y
     uint8_t seq[kSmallEvents]; // species of each event
 };
@@ -441,6 +443,11 @@ void launch_births(const EventArgs& a, cudaStream_t st);
 // Most blocks of a stretch on the current device: as one cluster, as a
 // cooperative grid (0: not at all).  Sets the kernels' attributes there.
 void small_limits(int sm_count, int* cluster, int* grid);
+// cells from mirrors and lists; mirrors and codes from cells
+void launch_cells_build(uint32_t* cell, const uint32_t* bits0, uint64_t words, int n_mirrors, const ModelDev* model,
+                        const int32_t* counts, int nsp, const Geometry& geo, int blocks, cudaStream_t st);
+void launch_cells_grid(const uint32_t* cell, uint32_t* bits0, uint64_t words, int n_mirrors, uint16_t* occ,
+                       const Geometry& geo, int blocks, cudaStream_t st);
 // stretches of many lattices in one launch of `blocks` blocks: args on the
 // device per lattice, group[block] = (lattice, first block of its group)
 int small_batch_blocks(int sm_count);       // most blocks on the current device (0: not at all)

@@ -1171,7 +1171,7 @@ void launch_event_one(const EventArgs& a, cudaStream_t st)
 // ---------------------------------------------------------------------------
 constexpr int kBirthSortMax = 8192;
 
-__device__ __forceinline__ void births_body(const EventArgs& a, uint32_t* slot_map = nullptr, uint32_t mapped = 0u)
+__device__ __forceinline__ void births_body(const EventArgs& a, uint32_t* cell = nullptr)
 {
     extern __shared__ unsigned long long keys[];
     int nb = a.sc->births;
@@ -1207,7 +1207,12 @@ __device__ __forceinline__ void births_body(const EventArgs& a, uint32_t* slot_m
             dst.vox[slot] = b.t;
             dst.ids[slot] = base_id + (uint32_t)x;
             dst.img[slot] = b.img;
-            if ((mapped >> b.species) & 1u) slot_map[b.t] = (uint32_t)slot;
+            if (cell) {                                         // (psc_small.cuh)
+                int32_t i, j, k;
+                decode(a.geo, (uint32_t)b.t, i, j, k);
+                const BitPos p = bitpos(a.geo, i, j, k);
+                cell[p.word * 32u + (uint32_t)(__ffs(p.mask) - 1)] = ((uint32_t)b.species << 26) | (uint32_t)slot;
+            }
         } else {
             atomicOr(&a.sc->err, kErrListOverflow);
         }
@@ -1685,6 +1690,13 @@ void launch_births_batch(const EventArgs* tmpl, const BatchLaunch& bl, cudaStrea
         configured = true;
     }
     k_births_batch<<<bl.n, 1024, smem, st>>>(tmpl, bl);
+}
+
+// *p = min(*p, x) without the old value (atomicMin compiled to a returning
+// atomic in the walkers' kernel)
+__device__ __forceinline__ void red_min(uint32_t* p, uint32_t x)
+{
+    asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
 
 #include "psc_small.cuh"

@@ -108,16 +108,16 @@ struct psc_lattice {
     std::vector<void*> allocs;
 
     // stretches of events in one launch (k_small_run): per-species argument
-    // templates on the device, the voxel -> slot map and the scratch of closing
-    // lists up
+    // templates on the device, a cell per voxel and the scratch of closing lists up
     struct SmallBuffers {
         EventArgs* ev = nullptr;       // written at the first stretch
-        uint32_t* slot = nullptr;      // allocated with the first stretch that may react
+        uint32_t* cell = nullptr;      // the cells, allocated with the first stretch
         int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
         int32_t scratch_n = 0;
-        bool map_holds = false;        // the map agrees with the lists (nothing else has changed them since)
+        bool cells_hold = false;       // the cells agree with the lists
+        bool grid_stale = false;       // mirrors and codes are behind the cells
         int cluster = 0, grid = 0;     // most blocks of a stretch: one cluster, a cooperative grid
-        uint32_t general = 0, fo2 = 0, mapped = 0;
+        uint32_t general = 0, fo2 = 0;
         uint32_t products[kMaxSpecies] = {};
     } small;
     // lattices without reactions (k_walk_run)
@@ -154,6 +154,8 @@ struct psc_lattice {
     // estimate costs time, never results): a pinned copy of Scalars::counts
     // refreshed in the background every few events.
     int64_t est[kMaxSpecies] = {};
+    int64_t next_id_known = 0;             // Scalars::next_id after event next_id_g
+    uint32_t next_id_g = 0;
     int32_t grid_class[kMaxSpecies] = {};  // per-event grid limit of each list (INT32_MAX: none)
     int32_t* counts_h = nullptr;
     cudaEvent_t counts_ev = nullptr;
@@ -218,10 +220,14 @@ int check_device(psc_lattice* L);
 // stretches of k_small_run (and of batches): buffers still lacking, their
 // allocation, the arguments but the events
 int64_t small_lacks(const psc_lattice* L, bool scratch);
-int small_buffers(psc_lattice* L, bool lists, bool scratch);
-void small_args(psc_lattice* L, bool reacts, SmallArgs* A);
+int64_t ids_bound(const psc_lattice* L);
+int small_buffers(psc_lattice* L, bool scratch);
+int small_args(psc_lattice* L, SmallArgs* A);
 // every claim word free again (after stretches of k_walk_run), as the other kernels want them
 int claims_free(psc_lattice* L);
+// mirrors and codes in line with the cells of k_small_run; leave: the cells are
+// given up too, as another kernel goes on
+int grid_current(psc_lattice* L, bool leave);
 // queue events in scheduler order until max_events or the next event lies after t_end
 int drive(psc_lattice* L, double t_end, int64_t max_events);
 // drop every captured graph (launch options changed)

@@ -12,21 +12,33 @@
 //   - a thread carries its molecules from the claim to the commit phase in
 //     registers, and the counts, the list entries and what may be left to do
 //     from the last event are loaded together;
-//   - a map from voxel to list slot (of the species that can be a partner)
-//     tells a reacting molecule where its partner's entry is, so the commit
-//     itself takes both entries off their lists and appends the products: no
-//     list is checked against the grid;
+//   - one word per voxel, its cell, tells vacancy and compartment, takes the
+//     claims of a vacant voxel, and holds species and list slot of the molecule
+//     on an occupied one.  A hop reads its target's cell, claims in it, reads it
+//     back, and writes it and the one it leaves (with mirror, codes, claim words
+//     and slots apart there were about ten accesses).  A reacting molecule finds
+//     its partner's list entry there, so the commit itself takes both entries off
+//     their lists and appends the products: no list is checked against the grid.
+//     Mirror and codes are brought up to date when another kernel or a read-out
+//     wants them;
 //   - an entry that leaves stays behind as a tombstone (voxel -1); the lists
 //     are closed up at the end of the stretch, or when one could run out of
 //     room.
 // Births need a pass of their own (ids in parent order) in events that have
 // any.
 //
-// Measured (us per event; before: CUDA graphs of per-event launches, or the
-// molecule-list kernel for walkers): A + B -> C of 2000 + 2000 molecules on
-// 64^3 12.5 -> 4.9, a cascade of 22 species of up to 16,000 molecules on 200^3
-// 10.5 -> 3.6, 30,000 ligands and 5000 receptors in a cell on 128^3 19.8 -> 8.0,
-// 2621 walkers on 64^3 8.2 -> 3.9.
+// One block of 512 threads per SM: the events need about 110 registers (two
+// blocks per SM spilled: crowded 256^3 30.1 us per event against 25.3), and two
+// molecules in flight per thread (three 27.2, four 32.1).
+//
+// Measured (us per event; before: claim, commit, list check and fill launches
+// replayed from CUDA graphs, or the molecule-list kernel for walkers): A + B -> C
+// of 2000 + 2000 molecules on 64^3 12.5 -> 4.2, a cascade of 22 species of up to
+// 16,000 molecules on 200^3 10.5 -> 3.1, 30,000 ligands and 5000 receptors in a
+// cell on 128^3 19.8 -> 6.8, reversible A + B <-> C under 30 % crowding with 839,000
+// A on 256^3 40.0 -> 25.3, with 1.6M on 320^3 92 -> 52, with 3.2M on 400^3
+// 180 -> 126.  The order of a list makes no difference here (26.3 sorted on
+// 256^3), so these stretches have no re-sorts.
 
 // Event arguments and model of the lattice, copied to shared memory once per
 // launch: after a barrier a load of them from global memory would go to L2.
@@ -76,9 +88,94 @@ __device__ __forceinline__ bool small_barrier(const SmallArgs& A, const SmallBlo
     return block_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, 0u, B.blk, B.nblk);
 }
 
-// molecule (id, img) on voxel v joins list y
-__device__ __forceinline__ void small_append(const SmallArgs& A, const ModelDev& M, int y, uint32_t v, uint32_t id,
-                                             uint64_t img)
+// Cells, in the mirror's order (place = mirror word << 5 | bit).  Top bit set:
+// vacant, compartment in bits 27 to 30, in the low 27 the id of the lowest
+// claimant (all ones: none).  Clear: occupied, species in bits 26 to 30, list
+// slot below.
+constexpr uint32_t kCellVacant = 0x80000000u;
+constexpr uint32_t kCellNone = 0x07FFFFFFu;                    // no claimant
+__device__ __forceinline__ uint32_t cell_claim(uint32_t comp, uint32_t id) { return kCellVacant | (comp << 27) | id; }
+__device__ __forceinline__ uint32_t cell_free(uint32_t comp) { return cell_claim(comp, kCellNone); }
+__device__ __forceinline__ uint32_t cell_of_entry(int s, uint32_t slot) { return ((uint32_t)s << 26) | slot; }
+
+// vacant in compartment comp at the start of the event (claimed or not)
+__device__ __forceinline__ bool cell_open(uint32_t w, uint32_t comp)
+{
+    return (w & kCellVacant) && ((w >> 27) & 15u) == comp;
+}
+
+__device__ __forceinline__ uint32_t small_place(const Geometry& G, int32_t i, int32_t j, int32_t k)
+{
+    const uint32_t word = (((uint32_t)k >> 1) * G.nbj + ((uint32_t)j >> 2)) * G.nbi + ((uint32_t)i >> 2);
+    return (word << 5) | ((uint32_t)i & 3u) | (((uint32_t)j & 3u) << 2) | (((uint32_t)k & 1u) << 4);
+}
+__device__ __forceinline__ BitPos small_bit(uint32_t place) { return BitPos{place >> 5, 1u << (place & 31u)}; }
+
+// Cells of all voxels from the mirrors (occupied ones 0: their lists' entries
+// follow, k_cells_lists), a thread per voxel of a mirror word
+__global__ void k_cells_vacant(uint32_t* cell, const uint32_t* bits0, uint64_t words, int n_mirrors)
+{
+    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < words * 32;
+         x += (uint64_t)gridDim.x * blockDim.x) {
+        uint32_t w = 0u;
+        for (int c = 0; c < n_mirrors; ++c)
+            if (!((bits0[(uint64_t)c * words + (x >> 5)] >> (x & 31u)) & 1u)) w = cell_free((uint32_t)c);
+        cell[x] = w;
+    }
+}
+
+__global__ void k_cells_lists(uint32_t* cell, const ModelDev* model, const int32_t* counts, int nsp, Geometry G)
+{
+    for (int s = 0; s < nsp; ++s) {
+        const SpeciesList& list = model->lists[s];
+        const int n = counts[s];
+        for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
+            int32_t i, j, k;
+            decode(G, (uint32_t)list.vox[idx], i, j, k);
+            cell[small_place(G, i, j, k)] = cell_of_entry(s, (uint32_t)idx);
+        }
+    }
+}
+
+// Mirrors and codes from the cells: a warp per mirror word.  A voxel's bit is
+// set in every mirror if it is occupied, else in all but its compartment's.
+__global__ void k_cells_grid(const uint32_t* cell, uint32_t* bits0, uint64_t words, int n_mirrors, uint16_t* occ,
+                             Geometry G)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint64_t x = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; x < words;
+         x += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint32_t w = cell[x * 32 + lane];
+        const int32_t i = (int32_t)((uint32_t)(x % G.nbi) * 4u + (lane & 3u));
+        const int32_t j = (int32_t)((uint32_t)((x / G.nbi) % G.nbj) * 4u + ((lane >> 2) & 3u));
+        const int32_t k = (int32_t)((uint32_t)(x / ((uint64_t)G.nbi * G.nbj)) * 2u + (lane >> 4));
+        const bool inside = i < G.ni && j < G.nj && k < G.nk;   // else its bit stays clear
+        for (int c = 0; c < n_mirrors; ++c) {
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, inside && !cell_open(w, (uint32_t)c));
+            if (lane == 0) bits0[(uint64_t)c * words + x] = m;
+        }
+        if (inside)
+            occ[(uint64_t)i + (uint64_t)G.ni * ((uint64_t)j + (uint64_t)G.nj * (uint64_t)k)] =
+                (w & kCellVacant) ? (uint16_t)0 : (uint16_t)((w >> 26) + 1u);
+    }
+}
+
+void launch_cells_build(uint32_t* cell, const uint32_t* bits0, uint64_t words, int n_mirrors, const ModelDev* model,
+                        const int32_t* counts, int nsp, const Geometry& geo, int blocks, cudaStream_t st)
+{
+    k_cells_vacant<<<blocks, 256, 0, st>>>(cell, bits0, words, n_mirrors);
+    k_cells_lists<<<blocks, 256, 0, st>>>(cell, model, counts, nsp, geo);
+}
+
+void launch_cells_grid(const uint32_t* cell, uint32_t* bits0, uint64_t words, int n_mirrors, uint16_t* occ,
+                       const Geometry& geo, int blocks, cudaStream_t st)
+{
+    k_cells_grid<<<blocks, 256, 0, st>>>(cell, bits0, words, n_mirrors, occ, geo);
+}
+
+// molecule (id, img) on voxel v, place p, joins list y
+__device__ __forceinline__ void small_append(const SmallArgs& A, const ModelDev& M, int y, uint32_t v, uint32_t p,
+                                             uint32_t id, uint64_t img)
 {
     const SpeciesList dst = M.lists[y];
     const int slot = atomicAdd(&A.sc->counts[y], 1);
@@ -89,7 +186,7 @@ __device__ __forceinline__ void small_append(const SmallArgs& A, const ModelDev&
     dst.vox[slot] = (int32_t)v;
     dst.ids[slot] = id;
     dst.img[slot] = img;
-    if ((A.mapped >> y) & 1u) A.slot[v] = (uint32_t)slot;
+    A.cell[p] = cell_of_entry(y, (uint32_t)slot);
 }
 
 // the entry at `slot` of list x leaves it
@@ -100,21 +197,14 @@ __device__ __forceinline__ void small_leave(const SmallArgs& A, const ModelDev& 
 }
 
 // A molecule between its claim and its commit phase: its voxel, id, the
-// claim's outcome (kDec*, with kSmallWrap where the hop crosses a periodic
-// boundary), the target voxel, and the places of both in the vacancy mirror
-// (word << 5 | bit).
+// claim's outcome (kDec*; with a direction, kSmallWrap where the hop crosses a
+// periodic boundary and kSmallReact where it is an accepted collision), the
+// target voxel, the places of both, and the target's cell as it was.
 struct SmallMol {
     int32_t v;
-    uint32_t id, dec, t, wv, wt;
+    uint32_t id, dec, t, pv, pt, w;
 };
-constexpr uint32_t kSmallWrap = 0x80u;
-
-__device__ __forceinline__ uint32_t small_place(const Geometry& G, int32_t i, int32_t j, int32_t k)
-{
-    const uint32_t word = (((uint32_t)k >> 1) * G.nbj + ((uint32_t)j >> 2)) * G.nbi + ((uint32_t)i >> 2);
-    return (word << 5) | ((uint32_t)i & 3u) | (((uint32_t)j & 3u) << 2) | (((uint32_t)k & 1u) << 4);
-}
-__device__ __forceinline__ BitPos small_bit(uint32_t place) { return BitPos{place >> 5, 1u << (place & 31u)}; }
+constexpr uint32_t kSmallWrap = 0x80u, kSmallReact = 0x40u;
 
 // the target of direction d; false behind a reflective wall
 __device__ __forceinline__ bool small_target(const Geometry& G, SmallMol& m, int32_t i, int32_t j, int32_t k, int d,
@@ -123,16 +213,17 @@ __device__ __forceinline__ bool small_target(const Geometry& G, SmallMol& m, int
     Nb nb;
     if (!neighbor(G, i, j, k, d, nb)) return false;
     m.t = (uint32_t)nb.t;
-    m.wv = small_place(G, i, j, k);
-    m.wt = small_place(G, nb.i, nb.j, nb.k);
+    m.pv = small_place(G, i, j, k);
+    m.pt = small_place(G, nb.i, nb.j, nb.k);
     *wrap = nb.wrap;
     return true;
 }
 
-// Claim phase of molecule (m.v, m.id): the rest of m.
+// Claim phase of molecule (m.v, m.id) up to its target: m.dec is kDecFire (its
+// claim, if it has one, is made), kDecNone or the direction; returns u1.
 template <bool GENERAL>
-__device__ __forceinline__ void small_claim(const EventArgs& a, const ModelDev& M, uint32_t g, SmallMol& m,
-                                            unsigned& n_col, unsigned& n_acc, unsigned& n_fire)
+__device__ __forceinline__ uint32_t small_aim(const SmallArgs& A, const EventArgs& a, const ModelDev& M, uint32_t g,
+                                              SmallMol& m, unsigned& n_fire)
 {
     int32_t i, j, k;
     decode(a.geo, (uint32_t)m.v, i, j, k);
@@ -143,81 +234,92 @@ __device__ __forceinline__ void small_claim(const EventArgs& a, const ModelDev& 
         ++n_fire;
         m.dec = kDecFire;
         const int r = pick_first_order(&M, a.s, u[3]);
-        if (M.rx[r].np != 2) return;
+        if (M.rx[r].np != 2) return 0u;
         // second product: uniform pick among the neighbours vacant now in its compartment
-        const uint32_t* pb = M.mirror[M.rx[r].p1];
+        const uint32_t comp = M.comp[M.rx[r].p1];
         uint32_t open = 0u;
         for (int d = 0; d < 12; ++d) {
             Nb nb;
-            if (neighbor(a.geo, i, j, k, d, nb) && !occupied(pb, bitpos(a.geo, nb.i, nb.j, nb.k))) open |= 1u << d;
+            if (neighbor(a.geo, i, j, k, d, nb) &&
+                cell_open(__ldcg(&A.cell[small_place(a.geo, nb.i, nb.j, nb.k)]), comp))
+                open |= 1u << d;
         }
-        if (!open) return;
+        if (!open) return 0u;
         for (int want = (int)__umulhi(u[0], (uint32_t)__popc(open)); want > 0; --want) open &= open - 1u;
         Nb nb;
         neighbor(a.geo, i, j, k, __ffs(open) - 1, nb);
-        claim<false>(a, nb, m.id);
-        return;
+        red_min(&A.cell[small_place(a.geo, nb.i, nb.j, nb.k)], cell_claim(comp, m.id));
+        return 0u;
     }
     const int d = (int)__umulhi(u[0], 12u);
     uint64_t wrap;
-    if (!small_target(a.geo, m, i, j, k, d, &wrap)) return;
-    bool go = !occupied(a.bits, small_bit(m.wt));
-    if (GENERAL && !go) {
-        const uint16_t o = __ldcg(&a.occ[m.t]);
-        if (o != 0 && o != kBlocked) {
-            const int r = M.pair[a.s][o - 1];
-            if (r >= 0) {
-                ++n_col;
-                go = (uint64_t)u[1] < M.rx[r].T;
-                if (go) ++n_acc;
+    if (small_target(a.geo, m, i, j, k, d, &wrap)) m.dec = (uint32_t)d | (wrap ? kSmallWrap : 0u);
+    return u[1];
+}
+
+// The rest of it, the target's cell being m.w: a claim or kDecNone.
+template <bool GENERAL>
+__device__ __forceinline__ void small_decide(const SmallArgs& A, const EventArgs& a, const ModelDev& M, SmallMol& m,
+                                             uint32_t u1, unsigned& n_col, unsigned& n_acc)
+{
+    const uint32_t comp = M.comp[a.s];
+    if (cell_open(m.w, comp)) {
+        red_min(&A.cell[m.pt], cell_claim(comp, m.id));
+        return;
+    }
+    bool go = false;
+    if (GENERAL && !(m.w & kCellVacant)) {
+        const int r = M.pair[a.s][m.w >> 26];
+        if (r >= 0) {
+            ++n_col;
+            go = (uint64_t)u1 < M.rx[r].T;
+            if (go) {
+                ++n_acc;
+                red_min(&a.ct.direct[m.t], m.id);               // its partner's voxel: a claim word
+                m.dec |= kSmallReact;
             }
         }
     }
-    if (!go) return;
-    atomicMin(&a.ct.direct[m.t], m.id);
-    m.dec = (uint32_t)d | (wrap ? kSmallWrap : 0u);
+    if (!go) m.dec = kDecNone;
 }
 
-// did molecule id win voxel t?  (the winner resets the word)
-__device__ __forceinline__ bool small_won(const EventArgs& a, uint32_t t, uint32_t id)
+// the word the commit phase reads back: the claim word of a collision, else
+// the target's cell
+__device__ __forceinline__ uint32_t small_readback(const SmallArgs& A, const EventArgs& a, const SmallMol& m)
 {
-    if (__ldcg(&a.ct.direct[t]) != id) return false;
-    a.ct.direct[t] = kNoClaim;
-    return true;
+    return __ldcg((m.dec & kSmallReact) ? &a.ct.direct[m.t] : &A.cell[m.pt]);
 }
 
 // Commit phase of the molecule at list slot idx whose claim phase did not end
-// with kDecNone; a hop sets m.v.
+// with kDecNone; `back` is the word read back (not used for kDecFire).  A hop
+// sets m.v.
 template <bool GENERAL>
 __device__ __forceinline__ void small_commit(const SmallArgs& A, const EventArgs& a, const ModelDev& M, uint32_t g,
-                                             int idx, SmallMol& m, unsigned& n_hop, unsigned& n_r2, unsigned& n_r1)
+                                             int idx, SmallMol& m, uint32_t back, unsigned& n_hop, unsigned& n_r2,
+                                             unsigned& n_r1)
 {
     const int s = a.s;
     const uint32_t v = (uint32_t)m.v, id = m.id;
     if (GENERAL && m.dec == kDecFire) {
         int32_t i, j, k;
         decode(a.geo, v, i, j, k);
-        const BitPos bv = bitpos(a.geo, i, j, k);
+        const uint32_t pv = small_place(a.geo, i, j, k);
         uint32_t u[4];
         philox(id, g, ((uint32_t)s << 4) | kTagEvent, 0u, a.key0, a.key1, u);
         const ReactionDev R = M.rx[pick_first_order(&M, s, u[3])];
         if (R.np == 2) {
-            // the neighbour this molecule claimed, if it won it; only its
-            // winner changes the bit of a claimed voxel
-            uint32_t* pb = M.mirror[R.p1];
+            // the neighbour this molecule claimed, if it won it
+            const uint32_t mine = cell_claim(M.comp[R.p1], id);
             for (int d = 0; d < 12; ++d) {
                 Nb nb;
                 if (!neighbor(a.geo, i, j, k, d, nb)) continue;
-                const BitPos bt = bitpos(a.geo, nb.i, nb.j, nb.k);
-                if (occupied(pb, bt) || !small_won(a, (uint32_t)nb.t, id)) continue;
-                a.occ[v] = (uint16_t)(R.p0 + 1);
-                a.occ[nb.t] = (uint16_t)(R.p1 + 1);
-                bit_set(pb, bt);
+                if (__ldcg(&A.cell[small_place(a.geo, nb.i, nb.j, nb.k)]) != mine) continue;
                 const uint64_t img = a.list.img[idx];
                 if (R.p0 != s) {
                     small_leave(A, M, s, (uint32_t)idx);
-                    small_append(A, M, R.p0, v, id, img);
+                    small_append(A, M, R.p0, v, pv, id, img);
                 }
+                // (its cell follows with its list entry, in the births' pass)
                 const int slot = atomicAdd(&A.sc->births, 1);
                 A.sc->touched[g & 1u] = 1u;
                 if (slot < a.births_cap) {
@@ -234,31 +336,18 @@ __device__ __forceinline__ void small_commit(const SmallArgs& A, const EventArgs
             return;
         }
         ++n_r1;
-        if (R.np == 0) {
-            a.occ[v] = 0;
-            bit_clear(a.bits, bv);
-        } else {
-            a.occ[v] = (uint16_t)(R.p0 + 1);
-            if (R.p0 == s) return;
-        }
+        if (R.np && R.p0 == s) return;
         const uint64_t img = a.list.img[idx];
         small_leave(A, M, s, (uint32_t)idx);
-        if (R.np) small_append(A, M, R.p0, v, id, img);
+        if (R.np) small_append(A, M, R.p0, v, pv, id, img);
+        else A.cell[pv] = cell_free(M.comp[s]);
         return;
     }
-    // the bit of a claimed voxel only changes through its winner, so it still
-    // tells a vacant target (hop) from a partner (reaction)
-    const BitPos bv = small_bit(m.wv), bt = small_bit(m.wt);
-    const uint32_t word = GENERAL ? __ldcg(&a.bits[bt.word]) : 0u;
-    if (!small_won(a, m.t, id)) return;
-    if (!GENERAL || !(word & bt.mask)) {
-        bit_move(a.bits, bv, bt);                               // move (Sec. 2.3)
-        if (a.live) {
-            a.occ[m.t] = (uint16_t)(s + 1);
-            a.occ[v] = 0;
-        }
+    if (!GENERAL || !(m.dec & kSmallReact)) {
+        if (back != cell_claim(M.comp[s], id)) return;
+        A.cell[m.pt] = cell_of_entry(s, (uint32_t)idx);         // move (Sec. 2.3)
+        A.cell[m.pv] = cell_free(M.comp[s]);
         a.list.vox[idx] = (int32_t)m.t;
-        if (GENERAL && ((A.mapped >> s) & 1u)) A.slot[m.t] = (uint32_t)idx;
         if (m.dec & kSmallWrap) {
             int32_t i, j, k;
             decode(a.geo, v, i, j, k);
@@ -270,14 +359,17 @@ __device__ __forceinline__ void small_commit(const SmallArgs& A, const EventArgs
         ++n_hop;
         return;
     }
-    // accepted collision with partner y (Sec. 2.4.2): first product on the
-    // partner's voxel, second on the mover's, unless that puts a product
-    // outside its compartment (then they trade places)
-    const int y = (int)__ldcg(&a.occ[m.t]) - 1;
+    // accepted collision with partner y (Sec. 2.4.2), if it won it: first
+    // product on the partner's voxel, second on the mover's, unless that puts a
+    // product outside its compartment (then they trade places)
+    if (back != id) return;
+    a.ct.direct[m.t] = kNoClaim;
+    const int y = (int)(m.w >> 26);
+    const uint32_t slot = m.w & 0x03FFFFFFu;
     const ReactionDev R = M.rx[M.pair[s][y]];
     const bool straight = R.np == 0 ||
                           (M.comp[R.p0] == M.comp[y] && (R.np < 2 || M.comp[R.p1] == M.comp[s]));
-    int at_t = 0, at_v = 0;                                     // codes afterwards
+    int at_t = 0, at_v = 0;                                     // species + 1 afterwards
     if (R.np == 1) {
         if (straight) at_t = R.p0 + 1;
         else at_v = R.p0 + 1;
@@ -285,23 +377,29 @@ __device__ __forceinline__ void small_commit(const SmallArgs& A, const EventArgs
         at_t = (straight ? R.p0 : R.p1) + 1;
         at_v = (straight ? R.p1 : R.p0) + 1;
     }
-    a.occ[m.t] = (uint16_t)at_t;
-    a.occ[v] = (uint16_t)at_v;
-    if (at_t == 0) bit_clear(M.mirror[y], bt);
-    if (at_v == 0) bit_clear(a.bits, bv);
     if (at_v != s + 1) {
         const uint64_t img = a.list.img[idx];
         small_leave(A, M, s, (uint32_t)idx);
-        if (at_v) small_append(A, M, at_v - 1, v, id, img);
+        if (at_v) small_append(A, M, at_v - 1, v, m.pv, id, img);
+        else A.cell[m.pv] = cell_free(M.comp[s]);
     }
     if (at_t != y + 1) {
-        const uint32_t slot = __ldcg(&A.slot[m.t]);            // the partner's entry
         const uint32_t pid = __ldcg(&M.lists[y].ids[slot]);
         const uint64_t pimg = __ldcg(&M.lists[y].img[slot]);
         small_leave(A, M, y, slot);
-        if (at_t) small_append(A, M, at_t - 1, m.t, pid, pimg);
+        if (at_t) small_append(A, M, at_t - 1, m.t, m.pt, pid, pimg);
+        else A.cell[m.pt] = cell_free(M.comp[y]);
     }
     ++n_r2;
+}
+
+// the entry of list x on voxel v is at slot h now
+__device__ __forceinline__ void small_entry(const SmallArgs& A, const SmallShared& S, int x, int32_t v, uint32_t h)
+{
+    const Geometry& G = S.ev[0].geo;
+    int32_t i, j, k;
+    decode(G, (uint32_t)v, i, j, k);
+    A.cell[small_place(G, i, j, k)] = cell_of_entry(x, h);
 }
 
 // The lists closed up.  In a cluster one block packs a list chunk by chunk
@@ -346,14 +444,13 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, const SmallBlock
         if (S.k[x] <= 0) continue;
         const SpeciesList list = M.lists[x];
         const int32_t moves = __ldcg(&A.sc->hole_n[x]);
-        const bool mapped = (A.mapped >> x) & 1u;
         for (int q = t0; q < moves; q += stride) {
             const int32_t h = __ldcg(A.holes + base + q), p = __ldcg(A.surv + base + q);
             const int32_t v = __ldcg(list.vox + p);
             list.vox[h] = v;
             list.ids[h] = __ldcg(list.ids + p);
             list.img[h] = __ldcg(list.img + p);
-            if (mapped) A.slot[v] = (uint32_t)h;
+            small_entry(A, S, x, v, (uint32_t)h);
         }
         if (t0 == 0) {
             A.sc->counts[x] = S.n[x] - S.k[x];
@@ -384,7 +481,7 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, const SmallBlock
                 list.vox[at] = v;
                 list.ids[at] = id;
                 list.img[at] = img;
-                if ((A.mapped >> x) & 1u) A.slot[v] = (uint32_t)at;
+                small_entry(A, S, x, v, (uint32_t)at);
             }
             __syncthreads();
         }
@@ -408,43 +505,74 @@ __device__ __forceinline__ bool small_event(const SmallArgs& A, const SmallBlock
                                             const EventArgs* next)
 {
     unsigned n_att = 0, n_col = 0, n_acc = 0, n_fire = 0, n_hop = 0, n_r2 = 0, n_r1 = 0;
+    // kSmallCarry molecules of the thread at a time, from slot t0 + c0 * stride:
+    // the cells' loads go out together
+    auto claims = [&](int c0, SmallMol (&q)[kSmallCarry]) {
+        uint32_t u1[kSmallCarry];
 #pragma unroll
-    for (int c = 0; c < kSmallCarry; ++c) {
-        if (t0 + c * stride < n && m[c].v >= 0) {
-            ++n_att;
-            small_claim<GENERAL>(a, M, g, m[c], n_col, n_acc, n_fire);
-        } else {
-            m[c].dec = kDecNone;
+        for (int c = 0; c < kSmallCarry; ++c) {
+            if (t0 + (c0 + c) * stride < n && q[c].v >= 0) {
+                ++n_att;
+                u1[c] = small_aim<GENERAL>(A, a, M, g, q[c], n_fire);
+            } else {
+                q[c].dec = kDecNone;
+            }
         }
-    }
-    for (int idx = t0 + kSmallCarry * stride; idx < n; idx += stride) {
-        SmallMol w;
-        w.v = __ldcg(&a.list.vox[idx]);
-        w.id = __ldcg(&a.list.ids[idx]);
-        w.dec = kDecNone;
-        if (w.v >= 0) {
-            ++n_att;
-            small_claim<GENERAL>(a, M, g, w, n_col, n_acc, n_fire);
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c)
+            if (q[c].dec != kDecNone && q[c].dec != kDecFire) q[c].w = __ldcg(&A.cell[q[c].pt]);
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c)
+            if (q[c].dec != kDecNone && q[c].dec != kDecFire)
+                small_decide<GENERAL>(A, a, M, q[c], u1[c], n_col, n_acc);
+    };
+    auto commits = [&](int c0, SmallMol (&q)[kSmallCarry]) {
+        uint32_t back[kSmallCarry];
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c)
+            if (q[c].dec != kDecNone && q[c].dec != kDecFire) back[c] = small_readback(A, a, q[c]);
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c)
+            if (q[c].dec != kDecNone)
+                small_commit<GENERAL>(A, a, M, g, t0 + (c0 + c) * stride, q[c], back[c], n_hop, n_r2, n_r1);
+    };
+    claims(0, m);
+    for (int c0 = kSmallCarry; t0 + c0 * stride < n; c0 += kSmallCarry) {
+        SmallMol q[kSmallCarry];
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c) {
+            const int idx = t0 + (c0 + c) * stride;
+            q[c].v = idx < n ? __ldcg(&a.list.vox[idx]) : -1;
+            q[c].id = idx < n ? __ldcg(&a.list.ids[idx]) : 0u;
         }
-        a.dec[idx] = (uint8_t)w.dec;                            // read back by this thread
+        claims(c0, q);
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c) {
+            const int idx = t0 + (c0 + c) * stride;
+            if (idx < n) a.dec[idx] = (uint8_t)q[c].dec;        // read back by this thread
+        }
     }
     if (!small_barrier<MODE>(A, B)) return false;
+    commits(0, m);
+    for (int c0 = kSmallCarry; t0 + c0 * stride < n; c0 += kSmallCarry) {
+        SmallMol q[kSmallCarry];
 #pragma unroll
-    for (int c = 0; c < kSmallCarry; ++c)
-        if (m[c].dec != kDecNone) small_commit<GENERAL>(A, a, M, g, t0 + c * stride, m[c], n_hop, n_r2, n_r1);
-    for (int idx = t0 + kSmallCarry * stride; idx < n; idx += stride) {
-        SmallMol w;
-        w.dec = a.dec[idx];
-        if (w.dec == kDecNone) continue;
-        w.v = __ldcg(&a.list.vox[idx]);
-        w.id = __ldcg(&a.list.ids[idx]);
-        if (w.dec != kDecFire) {
-            int32_t i, j, k;
-            decode(a.geo, (uint32_t)w.v, i, j, k);
-            uint64_t wrap;
-            small_target(a.geo, w, i, j, k, (int)(w.dec & 15u), &wrap);
+        for (int c = 0; c < kSmallCarry; ++c) {
+            const int idx = t0 + (c0 + c) * stride;
+            q[c].dec = idx < n ? a.dec[idx] : (uint32_t)kDecNone;
+            q[c].v = idx < n ? __ldcg(&a.list.vox[idx]) : -1;
+            q[c].id = idx < n ? __ldcg(&a.list.ids[idx]) : 0u;
         }
-        small_commit<GENERAL>(A, a, M, g, idx, w, n_hop, n_r2, n_r1);
+#pragma unroll
+        for (int c = 0; c < kSmallCarry; ++c) {
+            if (q[c].dec == kDecNone || q[c].dec == kDecFire) continue;
+            int32_t i, j, k;
+            decode(a.geo, (uint32_t)q[c].v, i, j, k);
+            uint64_t wrap;
+            small_target(a.geo, q[c], i, j, k, (int)(q[c].dec & 15u), &wrap);
+            if (q[c].dec & kSmallReact) q[c].w = __ldcg(&A.cell[q[c].pt]);
+        }
+        commits(c0, q);
     }
     if (next != nullptr && next != &a) {
 #pragma unroll
@@ -481,15 +609,6 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
     small_copy(S.ev, A.ev, sizeof(EventArgs) * A.nsp);
     small_copy(&S.model, A.model, sizeof(ModelDev));
     for (int e = threadIdx.x; e < A.n_events; e += blockDim.x) S.seq[e] = A.seq[e];
-    // the voxel -> slot map, where it does not hold from the last stretch
-    if (A.build_map) {
-        for (uint32_t m = A.mapped; m; m &= m - 1u) {
-            const int x = __ffs(m) - 1;
-            const SpeciesList& list = A.model->lists[x];
-            const int n = A.sc->counts[x];
-            for (int idx = t0; idx < n; idx += stride) A.slot[list.vox[idx]] = (uint32_t)idx;
-        }
-    }
     if (t0 < kMaxSpecies) {
         A.sc->tmp_count[t0] = 0;                                // tombstones per list
         A.sc->hole_n[t0] = 0;
@@ -537,7 +656,7 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
             // the same decision in every warp: nothing read here changes
             // between the last event's end and this event's commit phase
             if (born) {
-                if (blk == 0) births_body(S.ev[S.seq[e - 1]], A.slot, A.mapped);
+                if (blk == 0) births_body(S.ev[S.seq[e - 1]], A.cell);
                 prev_fo2 = false;
                 if (!small_barrier<MODE>(A, B)) return;
                 continue;
@@ -573,7 +692,7 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
 }
 
 template <bool CLUSTER>
-__global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(const SmallArgs A)
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(const SmallArgs A)
 {
     __shared__ SmallShared S;
     small_run<CLUSTER ? kSmallInCluster : kSmallInGrid>(A, S, SmallBlocks{(int)blockIdx.x, (int)gridDim.x});
@@ -581,9 +700,9 @@ __global__ void __launch_bounds__(kSmallThreads, CLUSTER ? 1 : 2) k_small_run(co
 
 // Stretches of many lattices in one cooperative launch, each with a group of
 // consecutive blocks and at its own pace: no lattice waits for another.
-// counts: list lengths afterwards, [lattice][kMaxSpecies], for the next
-// launch's groups.
-__global__ void __launch_bounds__(kSmallThreads, 2) k_small_batch(const SmallArgs* args, const int2* group,
+// counts: list lengths and next id afterwards, [lattice][kSmallCounts], for the
+// next launch's groups.
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArgs* args, const int2* group,
                                                                   int32_t* counts)
 {
     __shared__ SmallShared S;
@@ -593,8 +712,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small_batch(const SmallArg
     __syncthreads();
     const SmallBlocks B{(int)blockIdx.x - mine.y, A.blocks};
     small_run<kSmallInGroup>(A, S, B);
-    if (A.general && B.blk == 0 && (int)threadIdx.x < A.nsp)
-        counts[mine.x * kMaxSpecies + threadIdx.x] = S.n[threadIdx.x] - S.k[threadIdx.x];
+    int32_t* out = counts + mine.x * kSmallCounts;
+    if (A.general && B.blk == 0 && (int)threadIdx.x < A.nsp) out[threadIdx.x] = S.n[threadIdx.x] - S.k[threadIdx.x];
+    if (B.blk == 0 && threadIdx.x == 0) out[kMaxSpecies] = (int32_t)min(A.sc->next_id, 0x7FFFFFFFu);
 }
 
 int small_batch_blocks(int sm_count)

@@ -54,13 +54,6 @@ __device__ __forceinline__ bool walk_barrier(const WalkArgs& A)
     return grid_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, A.barrier_phantom);
 }
 
-// *p = min(*p, x) without the old value (atomicMin compiled to a returning
-// atomic here)
-__device__ __forceinline__ void red_min(uint32_t* p, uint32_t x)
-{
-    asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
-}
-
 // coordinates of place p = mirror word << 5 | bit
 __device__ __forceinline__ void walk_decode(const WalkArgs& A, uint32_t p, int32_t& i, int32_t& j, int32_t& k)
 {

@@ -3,8 +3,9 @@ of blocks up to 16,384 molecules, a cooperative grid above.
 
 Compared bit for bit with the oracle where such a stretch can go wrong: lists
 on either side of the cluster's limit and crossing it, calls that end a stretch
-after 1, 2, 511 and 513 events, per-event launches in between (they change the
-lists behind the voxel -> slot map), reactions fast enough that tombstones fill
+after 1, 2, 511 and 513 events, per-event launches in between (they want the
+occupancy bits and codes that stretches leave behind, and change the lists behind
+the cells), lists of more entries than threads carry, reactions fast enough that tombstones fill
 the lists' room several times within a stretch, births, immobile partners,
 compartments, and walkers between species with reactions.
 """
@@ -41,6 +42,17 @@ def splitting(L, n):
     assert w == 2
 
 
+def crowded(L, n):
+    """More molecules than a grid's threads carry, walkers among them, between crowders."""
+    L.add_species(0.0, n)
+    a = L.add_species(1e-12, n)
+    b = L.add_species(0.8e-12, n // 4)
+    c = L.add_species(0.9e-12, 0)
+    L.add_species(1e-12, 2 * n)
+    L.add_reaction([a, b], [c], 3e-20)
+    L.add_reaction([c], [a, b], 0.05 / TAU)
+
+
 CASES = [
     ("ab_16383", (64, 64, 64), 7, lambda L: models.reaction_diffusion_ab(L, 16383, 9000), (1, 2, 511)),
     ("ab_16385", (64, 64, 64), 7, lambda L: models.reaction_diffusion_ab(L, 16385, 16384), (1, 513)),
@@ -48,6 +60,7 @@ CASES = [
     ("flip_grid", (72, 64, 60), 0, lambda L: flipping(L, 20000), (511, 1)),
     ("split_cluster", (37, 41, 29), 0, lambda L: splitting(L, 700), (2, 150)),
     ("split_grid", (60, 58, 64), 7, lambda L: splitting(L, 18000), (40, 1)),
+    ("crowded", (96, 92, 100), 0, lambda L: crowded(L, 170000), (2, 60)),
     ("walkers", (48, 44, 52), 6, lambda L: [L.add_species(d, n) for d, n in ((1e-12, 17000), (1e-12, 3), (0.6e-12, 900))],
      (1, 513)),
 ]
