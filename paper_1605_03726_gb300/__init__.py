@@ -322,7 +322,7 @@ class Lattice:
 
     def grid(self):
         ni, nj, nk = self.shape
-        g = np.zeros(ni * nj * nk, dtype=np.uint16)
+        g = np.empty(ni * nj * nk, dtype=np.uint16)              # every entry is written
         _check("psc_grid", lib().psc_grid(self._h, _ptr(g)))
         return g
 

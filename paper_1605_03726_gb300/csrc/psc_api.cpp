@@ -17,7 +17,11 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <thread>
 #include <vector>
+
+#include <sys/mman.h>
+#include <unistd.h>
 
 using namespace psc;
 
@@ -69,6 +73,67 @@ void* dev_alloc(psc_lattice* L, size_t bytes)
     if (p) L->allocs.push_back(p);
     return p;
 }
+
+namespace {
+
+// Buffers carved from one allocation: a lattice of 64^3 voxels spent more on some
+// thirty allocations and their release than on its placement.
+struct Carve {
+    std::vector<std::pair<void*, size_t>> parts;     // address of the pointer, offset
+    size_t bytes = 0;
+    template <typename T>
+    void add(T** p, size_t n)
+    {
+        parts.emplace_back((void*)p, bytes);
+        bytes += (std::max<size_t>(n, 1) + 255) & ~(size_t)255;
+    }
+    char* commit(psc_lattice* L)
+    {
+        char* base = (char*)dev_alloc(L, bytes);
+        for (const auto& x : parts) {
+            char* q = base ? base + x.second : nullptr;
+            std::memcpy(x.first, &q, sizeof(q));
+        }
+        return base;
+    }
+};
+
+// Pages of a host buffer that a read-out is about to fill, made present by
+// several threads: a copy into fresh pages faults them in one after the other
+// (64 MB 2.49 ms; made present by one thread, and copied, 2.33, two 1.53, four
+// 1.22, eight 2.05).  Contents stay as they are; a buffer whose pages are there
+// already (its ends and middle say so), or a small one, is left alone.
+void make_present(void* buf, size_t bytes)
+{
+    const size_t kPart = (size_t)2 << 20;
+    if (bytes < 2 * kPart) return;
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+    const uintptr_t lo = ((uintptr_t)buf + page - 1) & ~(page - 1), hi = ((uintptr_t)buf + bytes) & ~(page - 1);
+    unsigned char there = 1;
+    const uintptr_t look[3] = {lo, (lo + (hi - lo) / 2) & ~(page - 1), hi - page};
+    for (int x = 0; x < 3 && (there & 1); ++x)
+        if (mincore((void*)look[x], page, &there) != 0) return;
+    if (there & 1) return;
+    const size_t want = std::min<size_t>({bytes / kPart, (size_t)4, (size_t)std::max(1u, std::thread::hardware_concurrency())});
+    const int parts = (int)std::max<size_t>(want, 1);
+    auto part = [=](int x) {
+        const uintptr_t step = ((hi - lo) / (uintptr_t)parts) & ~(page - 1);
+        const uintptr_t a = lo + step * (uintptr_t)x, b = x == parts - 1 ? hi : a + step;
+        (void)madvise((void*)a, b - a, MADV_POPULATE_WRITE);       // a kernel without it: the copy faults them in
+    };
+    std::vector<std::thread> helpers;
+    int mine = 1;
+    try {
+        helpers.reserve((size_t)parts);
+        for (; mine < parts; ++mine) helpers.emplace_back(part, mine);
+    } catch (...) {                                    // no more threads: the rest here
+    }
+    part(0);
+    for (; mine < parts; ++mine) part(mine);
+    for (auto& h : helpers) h.join();
+}
+
+}  // namespace
 
 void dev_free_all(psc_lattice* L)
 {
@@ -163,6 +228,17 @@ int sort_first(psc_lattice* L, int s)
 // the device runs them; once a copy is 256 events old the host waits for it,
 // so the estimates stay recent (the device still has that many queued).
 constexpr size_t kCountsBytes = offsetof(Scalars, next_id) + sizeof(uint32_t);   // counts to next_id
+constexpr size_t kStateBytes = offsetof(Scalars, err) + sizeof(int32_t);         // counts to err
+constexpr size_t kStateAt = 2048;           // of check_device's copy, in the same page
+static_assert(kCountsBytes <= kStateAt && kStateAt + kStateBytes <= 4096, "both fit a page");
+
+static void counts_free(psc_lattice* L)
+{
+    if (!L->counts_h) return;
+    cudaHostUnregister(L->counts_h);
+    std::free(L->counts_h);
+    L->counts_h = nullptr;
+}
 
 void refresh_estimates(psc_lattice* L)
 {
@@ -1073,13 +1149,18 @@ bool next_event(const psc_lattice* L, int* s_out, double* t_out)
 
 int check_device(psc_lattice* L)
 {
-    cudaError_t e = cudaStreamSynchronize(L->stream);
+    if (!L->populated) {
+        const cudaError_t e = cudaStreamSynchronize(L->stream);
+        return e != cudaSuccess ? cuda_fail(L, e) : L->sticky;
+    }
+    // list lengths and error bits come with the wait itself
+    int32_t* state = L->counts_h ? L->counts_h + kStateAt / 4 : L->state;
+    cudaError_t e = cudaMemcpyAsync(state, L->sc, kStateBytes, cudaMemcpyDeviceToHost, L->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(L->stream);
     if (e != cudaSuccess) return cuda_fail(L, e);
-    if (!L->populated) return L->sticky;
-    int32_t err = 0;
-    e = cudaMemcpy(&err, &L->sc->err, sizeof(err), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(L, e);
-    L->d2h += sizeof(err);
+    if (state != L->state) std::memcpy(L->state, state, kStateBytes);
+    L->d2h += kStateBytes;
+    const int32_t err = L->state[offsetof(Scalars, err) / 4];
     if (err & kErrBarrierTimeout) L->sticky = PSC_E_TIMEOUT;
     else if (err) L->sticky = PSC_E_CAPACITY;
     return L->sticky;
@@ -1377,28 +1458,16 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     const size_t nwords = (size_t)mirror_words(L->ni, L->nj, L->nk);
     const int nmirror = comps ? L->ncomp : 1;
     L->mirror_n = nwords;
-    L->occ = (uint16_t*)dev_alloc(L, V * sizeof(uint16_t));
-    L->bits = (uint32_t*)dev_alloc(L, nwords * nmirror * sizeof(uint32_t));
     L->dirty_words = (uint32_t)((nwords + 31) / 32);
-    for (int x = 0; x < 2; ++x) {
-        L->dirty[x] = (uint32_t*)dev_alloc(L, (size_t)L->dirty_words * 4);
-        if (!L->dirty[x]) return PSC_E_NOMEM;
-    }
-    L->sc = (Scalars*)dev_alloc(L, sizeof(Scalars));
-    L->model_d = (ModelDev*)dev_alloc(L, sizeof(ModelDev));
-    L->barrier = (BarrierState*)dev_alloc(L, sizeof(BarrierState));
-    uint32_t* mort = (uint32_t*)dev_alloc(L, (size_t)(L->ni + L->nj + L->nk) * sizeof(uint32_t));
-    if (!L->occ || !L->bits || !L->sc || !L->model_d || !L->barrier || !mort) return PSC_E_NOMEM;
-    {
-        std::vector<uint32_t> mt((size_t)(L->ni + L->nj + L->nk));
-        uint32_t mbits = 0;
-        build_morton_tables(L->ni, L->nj, L->nk, mt.data(), &mbits);
-        int rc0 = cuda_fail(L, cudaMemcpy(mort, mt.data(), mt.size() * 4, cudaMemcpyHostToDevice));
-        if (rc0) return rc0;
-        L->h2d += mt.size() * 4;
-        L->geo.mort = mort;
-        L->geo.mort_bits = mbits;
-    }
+    uint32_t* mort = nullptr;
+    Carve carve;
+    carve.add(&L->occ, V * sizeof(uint16_t));
+    carve.add(&L->bits, nwords * nmirror * sizeof(uint32_t));
+    for (int x = 0; x < 2; ++x) carve.add(&L->dirty[x], (size_t)L->dirty_words * 4);
+    carve.add(&L->sc, sizeof(Scalars));
+    carve.add(&L->model_d, sizeof(ModelDev));
+    carve.add(&L->barrier, sizeof(BarrierState));
+    carve.add(&mort, (size_t)(L->ni + L->nj + L->nk) * sizeof(uint32_t));
     // claims: a word per voxel on small lattices, else two hash tables with at
     // least two slots per molecule of the largest mobile species
     uint32_t hb_max = 0;
@@ -1448,40 +1517,52 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     if (direct && !L->claim) {
         // (k_walk_run orders them as the mirror's bits, whole bricks)
         L->claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
-        L->claim = (uint32_t*)dev_alloc(L, (size_t)L->claim_n * sizeof(uint32_t));
-        if (!L->claim) return PSC_E_NOMEM;
+        carve.add(&L->claim, (size_t)L->claim_n * sizeof(uint32_t));
     } else if (!direct) {
         L->table_slots = (int64_t)1 << hb_max;
-        for (int t = 0; t < 2; ++t) {
-            L->tables[t] = (uint64_t*)dev_alloc(L, ((size_t)1 << hb_max) * sizeof(uint64_t));
-            if (!L->tables[t]) return PSC_E_NOMEM;
-        }
+        for (int t = 0; t < 2; ++t) carve.add(&L->tables[t], ((size_t)1 << hb_max) * sizeof(uint64_t));
     }
     for (int s = 0; s < L->nsp; ++s) {
-        M.comp[s] = (uint8_t)(comps ? L->sp[s].comp : 0);
-        M.mirror[s] = L->bits + (size_t)M.comp[s] * nwords;
         SpeciesList& l = M.lists[s];
         l.cap = L->cap[s] + (is_product[s] ? (int32_t)L->list_slack : 0);
-        l.vox = (int32_t*)dev_alloc(L, (size_t)l.cap * 4);
-        l.ids = (uint32_t*)dev_alloc(L, (size_t)l.cap * 4);
-        l.img = (uint64_t*)dev_alloc(L, (size_t)l.cap * 8);
-        if (!l.vox || !l.ids || !l.img) return PSC_E_NOMEM;
+        carve.add(&l.vox, (size_t)l.cap * 4);
+        carve.add(&l.ids, (size_t)l.cap * 4);
+        carve.add(&l.img, (size_t)l.cap * 8);
     }
+    // from here to the end: scratch of events and re-sorts, and first of the placement
+    const size_t scratch_at = carve.bytes;
     // the list passes of an event note up to two leavers per reaction, at most
     // one reaction per molecule of the due species
     L->tmp.cap = (int32_t)max_cap;
-    L->tmp.vox = (int32_t*)dev_alloc(L, (size_t)max_cap * 8);
-    L->tmp.ids = (uint32_t*)dev_alloc(L, (size_t)max_cap * 8);
-    L->tmp.img = (uint64_t*)dev_alloc(L, (size_t)max_cap * 8);
-    if (!L->tmp.vox || !L->tmp.ids || !L->tmp.img) return PSC_E_NOMEM;
+    carve.add(&L->tmp.vox, (size_t)max_cap * 8);
+    carve.add(&L->tmp.ids, (size_t)max_cap * 8);
+    carve.add(&L->tmp.img, (size_t)max_cap * 8);
     L->births_cap = any_fo2 ? 8192 : 1;
-    L->births = (Birth*)dev_alloc(L, (size_t)L->births_cap * sizeof(Birth));
+    carve.add(&L->births, (size_t)L->births_cap * sizeof(Birth));
     L->rs_max = max_mobile;
-    L->rs_keys = (uint32_t*)dev_alloc(L, (size_t)max_mobile * 4);
-    L->rs_vals = (uint32_t*)dev_alloc(L, (size_t)max_mobile * 4);
-    void* rs = dev_alloc(L, sort_scratch_bytes(max_mobile));
-    if (!L->births || !L->rs_keys || !L->rs_vals || !rs) return PSC_E_NOMEM;
+    void* rs = nullptr;
+    carve.add(&L->rs_keys, (size_t)max_mobile * 4);
+    carve.add(&L->rs_vals, (size_t)max_mobile * 4);
+    carve.add(&rs, sort_scratch_bytes(max_mobile));
+    char* const carved = carve.commit(L);
+    if (!carved) return PSC_E_NOMEM;
+    char* const place_scratch = L->scratch = carved + scratch_at;
+    const size_t place_room = L->scratch_bytes = carve.bytes - scratch_at;
     sort_scratch_bind(L->rs_scratch, rs, max_mobile);
+    for (int s = 0; s < L->nsp; ++s) {
+        M.comp[s] = (uint8_t)(comps ? L->sp[s].comp : 0);
+        M.mirror[s] = L->bits + (size_t)M.comp[s] * nwords;
+    }
+    {
+        std::vector<uint32_t> mt((size_t)(L->ni + L->nj + L->nk));
+        uint32_t mbits = 0;
+        build_morton_tables(L->ni, L->nj, L->nk, mt.data(), &mbits);
+        int rc0 = cuda_fail(L, cudaMemcpy(mort, mt.data(), mt.size() * 4, cudaMemcpyHostToDevice));
+        if (rc0) return rc0;
+        L->h2d += mt.size() * 4;
+        L->geo.mort = mort;
+        L->geo.mort_bits = mbits;
+    }
 
     if (L->opt.subvolume > 0) {
         auto& SV = L->subvol;
@@ -1546,11 +1627,14 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         const int bins = 1 << kPlaceBits;
         int64_t need[kMaxCompartments] = {};
         for (int s = 0; s < L->nsp; ++s) need[comps ? L->sp[s].comp : 0] += L->sp[s].n0;
-        uint32_t* hist = (uint32_t*)dev_alloc(L, (size_t)nc * bins * 4);
-        int32_t* pick_n = (int32_t*)dev_alloc(L, 4);
-        if (!hist || !pick_n) return PSC_E_NOMEM;
-        if ((rc = cuda_fail(L, cudaMemsetAsync(hist, 0, (size_t)nc * bins * 4, st)))) return rc;
-        if ((rc = cuda_fail(L, cudaMemsetAsync(pick_n, 0, 4, st)))) return rc;
+        // histogram and count, then the candidates and their sort: in the scratch of
+        // the lattice's events, which nothing uses yet, or in blocks of their own
+        const size_t head = (size_t)nc * bins * 4 + 256;
+        char* const own_head = head <= place_room ? nullptr : (char*)dev_alloc(L, head);
+        if (head > place_room && !own_head) return PSC_E_NOMEM;
+        uint32_t* hist = (uint32_t*)(own_head ? own_head : place_scratch);
+        int32_t* pick_n = (int32_t*)(hist + (size_t)nc * bins);
+        if ((rc = cuda_fail(L, cudaMemsetAsync(hist, 0, head, st)))) return rc;
         launch_place_hist((uint32_t)V, (uint32_t)seed, (uint32_t)(seed >> 32), labels_d, nc, hist, fill_blocks, st);
         std::vector<uint32_t> h((size_t)nc * bins);
         if ((rc = cuda_fail(L, cudaMemcpyAsync(h.data(), hist, h.size() * 4, cudaMemcpyDeviceToHost, st)))) return rc;
@@ -1578,10 +1662,14 @@ int psc_populate(psc_lattice* L, uint64_t seed)
                 used[c] += L->sp[s].n0;
             }
         }
-        uint32_t* cvox = (uint32_t*)dev_alloc(L, (size_t)M * 4);
-        uint32_t* ckey = (uint32_t*)dev_alloc(L, (size_t)M * 4);
-        void* scratch = dev_alloc(L, sort_scratch_bytes(M));
-        if (!cvox || !ckey || !scratch) return PSC_E_NOMEM;
+        const size_t part = ((size_t)M * 4 + 255) & ~(size_t)255, body = 2 * part + sort_scratch_bytes(M);
+        const size_t head_at = own_head ? 0 : (head + 255) & ~(size_t)255;
+        char* const own_body = head_at + body <= place_room ? nullptr : (char*)dev_alloc(L, body);
+        if (head_at + body > place_room && !own_body) return PSC_E_NOMEM;
+        char* const at = own_body ? own_body : place_scratch + head_at;
+        uint32_t* cvox = (uint32_t*)at;
+        uint32_t* ckey = (uint32_t*)(at + part);
+        void* scratch = at + 2 * part;
         SortScratch ss;
         sort_scratch_bind(ss, scratch, M);
         launch_place_pick((uint32_t)V, (uint32_t)seed, (uint32_t)(seed >> 32), labels_d, lim, cvox, ckey, pick_n,
@@ -1606,17 +1694,14 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         if ((rc = cuda_fail(L, cudaMemcpyAsync(&picked, pick_n, 4, cudaMemcpyDeviceToHost, st)))) return rc;
         if ((rc = cuda_fail(L, cudaStreamSynchronize(st)))) return rc;
         if (picked != M) return PSC_E_CUDA;                             // the two passes disagree
-        dev_free_one(L, cvox);
-        dev_free_one(L, ckey);
-        dev_free_one(L, scratch);
-        dev_free_one(L, hist);
-        dev_free_one(L, pick_n);
+        if (own_body) dev_free_one(L, own_body);
+        if (own_head) dev_free_one(L, own_head);
     }
     if (labels_d) {
         if ((rc = cuda_fail(L, cudaStreamSynchronize(st)))) return rc;
         dev_free_one(L, labels_d);
     }
-    if ((rc = cuda_fail(L, cudaStreamSynchronize(st)))) return rc;
+    if (N == 0 && (rc = cuda_fail(L, cudaStreamSynchronize(st)))) return rc;     // (else the placement waited)
     L->g = 0;
     L->clock = 0.0;
     L->populated = true;
@@ -1630,14 +1715,19 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     L->counts_g = 0;
     L->next_id_known = N;
     L->next_id_g = 0;
-    if (!L->counts_h && cudaMallocHost(&L->counts_h, kCountsBytes) != cudaSuccess) {
-        L->counts_h = nullptr;
-        cudaGetLastError();
+    if (!L->counts_h) {
+        // a page of the heap, registered: 37 us with its release, 270 from cudaMallocHost
+        const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+        L->counts_h = (int32_t*)std::aligned_alloc(page, page);
+        if (L->counts_h && cudaHostRegister(L->counts_h, page, cudaHostRegisterDefault) != cudaSuccess) {
+            std::free(L->counts_h);
+            L->counts_h = nullptr;
+        }
+        if (!L->counts_h) cudaGetLastError();
     }
     if (L->counts_h && !L->counts_ev &&
         cudaEventCreateWithFlags(&L->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
-        cudaFreeHost(L->counts_h);
-        L->counts_h = nullptr;
+        counts_free(L);
         L->counts_ev = nullptr;
         cudaGetLastError();
     }
@@ -2091,10 +2181,7 @@ int psc_counts(psc_lattice* L, int64_t* counts, int32_t n)
     DevGuard dg(L->device);
     int rc = check_device(L);
     if (rc) return rc;
-    int32_t c[kMaxSpecies];
-    if ((rc = cuda_fail(L, cudaMemcpy(c, L->sc->counts, sizeof(c), cudaMemcpyDeviceToHost)))) return rc;
-    L->d2h += sizeof(c);
-    for (int s = 0; s < L->nsp; ++s) counts[s] = c[s];
+    for (int s = 0; s < L->nsp; ++s) counts[s] = L->state[s];
     return PSC_OK;
 }
 
@@ -2103,9 +2190,8 @@ static int read_list(psc_lattice* L, int32_t s, std::vector<int32_t>& vox, std::
 {
     int rc = check_device(L);
     if (rc) return rc;
-    int32_t n = 0;
-    if ((rc = cuda_fail(L, cudaMemcpy(&n, &L->sc->counts[s], 4, cudaMemcpyDeviceToHost)))) return rc;
-    L->d2h += 4 + (uint64_t)n * (img ? 16 : 8);
+    const int32_t n = L->state[s];
+    L->d2h += (uint64_t)n * (img ? 16 : 8);
     const SpeciesList& l = L->model_h.lists[s];
     vox.resize(n);
     ids.resize(n);
@@ -2125,9 +2211,7 @@ static int list_size(psc_lattice* L, int32_t s, int64_t* n_out)
 {
     int rc = check_device(L);
     if (rc) return rc;
-    int32_t n = 0;
-    if ((rc = cuda_fail(L, cudaMemcpy(&n, &L->sc->counts[s], 4, cudaMemcpyDeviceToHost)))) return rc;
-    L->d2h += 4;
+    const int32_t n = L->state[s];
     *n_out = n;
     return n > 0 ? PSC_E_ARG : PSC_OK;
 }
@@ -2165,14 +2249,9 @@ static int device_positions(psc_lattice* L, int32_t s, int64_t n, bool unwrapped
 {
     const bool by_id = !L->live[s] && n == L->sp[s].n0;
     if (n <= 0 || (n > L->rs_max && !by_id)) return 1;
-    if (n > L->readout_cap) {
-        if (L->readout) dev_free_one(L, L->readout);
-        L->readout = (int32_t*)dev_alloc(L, (size_t)n * 16);
-        L->readout_cap = L->readout ? n : 0;
-        if (!L->readout) return 1;
-    }
-    int32_t* pos = L->readout;
-    uint32_t* ids = reinterpret_cast<uint32_t*>(L->readout + 3 * n);
+    // the list passes' scratch, 32 bytes per entry of the longest list
+    int32_t* pos = L->tmp.vox;
+    uint32_t* ids = reinterpret_cast<uint32_t*>(pos + 3 * n);
     const int blocks = event_blocks(L, n);
     if (by_id) {
         uint32_t id_lo = 0;
@@ -2184,6 +2263,8 @@ static int device_positions(psc_lattice* L, int32_t s, int64_t n, bool unwrapped
                           (L->bflags & PSC_FCC) != 0, L->rs_keys, L->rs_vals, L->rs_scratch, pos, ids, blocks,
                           L->stream, &L->launches) != 0)
         return cuda_fail(L, cudaErrorUnknown);
+    make_present(out, (size_t)n * 12);
+    if (ids_out) make_present(ids_out, (size_t)n * 4);
     int rc = cuda_fail(L, cudaMemcpyAsync(out, pos, (size_t)n * 12, cudaMemcpyDeviceToHost, L->stream));
     if (!rc && ids_out)
         rc = cuda_fail(L, cudaMemcpyAsync(ids_out, ids, (size_t)n * 4, cudaMemcpyDeviceToHost, L->stream));
@@ -2273,9 +2354,17 @@ int psc_grid(psc_lattice* L, uint16_t* occ)
     int rc = check_device(L);
     if (rc) return rc;
     if ((rc = grid_current(L, false))) return rc;
+    if (L->small.cells_hold) {                       // grid_current wrote the code of every voxel
+        make_present(occ, (size_t)L->V * 2);
+        rc = cuda_fail(L, cudaMemcpyAsync(occ, L->occ, (size_t)L->V * 2, cudaMemcpyDeviceToHost, L->stream));
+        if (!rc) rc = cuda_fail(L, cudaStreamSynchronize(L->stream));
+        L->d2h += (uint64_t)L->V * 2;
+        return rc;
+    }
     // exact codes: mirror-masked codes of species with reactions, then the
     // species without reactions from their lists
-    uint16_t* tmp = (uint16_t*)dev_alloc(L, (size_t)L->V * 2);
+    const bool own = (size_t)L->V * 2 > L->scratch_bytes;
+    uint16_t* tmp = own ? (uint16_t*)dev_alloc(L, (size_t)L->V * 2) : (uint16_t*)L->scratch;
     if (!tmp) return PSC_E_NOMEM;
     const int blocks = L->sm_count * 8;
     launch_materialize(tmp, L->occ, L->bits, L->mirror_n, L->labels.empty() ? 1 : L->ncomp, L->geo, L->V, blocks,
@@ -2285,10 +2374,11 @@ int psc_grid(psc_lattice* L, uint16_t* occ)
             launch_scatter_codes(tmp, L->model_h.lists[s], &L->sc->counts[s], (uint16_t)(s + 1), blocks,
                                  L->stream);
     L->launches += 1;
+    make_present(occ, (size_t)L->V * 2);
     rc = cuda_fail(L, cudaStreamSynchronize(L->stream));
     if (!rc) rc = cuda_fail(L, cudaMemcpy(occ, tmp, (size_t)L->V * 2, cudaMemcpyDeviceToHost));
     L->d2h += (uint64_t)L->V * 2;
-    dev_free_one(L, tmp);
+    if (own) dev_free_one(L, tmp);
     return rc;
 }
 
@@ -2439,7 +2529,6 @@ int psc_device_bytes(const psc_lattice* L, int64_t* bytes)
     const auto& T = L->tile;
     b += T.slots * 4 * 5 + (int64_t)T.regions * 4 * 4 + T.ids * 8 + T.halo_entries * (int64_t)sizeof(uint2);
     if (T.claim) b += L->V * 4;
-    b += L->readout_cap * 16;                        // staging of the device-side read-out, once used
     *bytes = b;
     return PSC_OK;
 }
@@ -2453,7 +2542,7 @@ void psc_lattice_destroy(psc_lattice* L)
         for (const auto& sp : L->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
         for (cudaEvent_t ev : L->event_pool) cudaEventDestroy(ev);
         if (L->counts_ev) cudaEventDestroy(L->counts_ev);
-        if (L->counts_h) cudaFreeHost(L->counts_h);
+        counts_free(L);
         graph_cache_clear(L);
         dev_free_all(L);
         if (L->own_stream && L->stream) cudaStreamDestroy(L->stream);

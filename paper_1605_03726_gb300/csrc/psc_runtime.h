@@ -82,8 +82,8 @@ struct psc_lattice {
     uint32_t* rs_vals = nullptr;
     SortScratch rs_scratch;
     int64_t rs_max = 0;
-    int32_t* readout = nullptr;          // staging of the device-side read-out (16 bytes per molecule)
-    int64_t readout_cap = 0;
+    char* scratch = nullptr;             // of events and re-sorts (tmp to rs_scratch), free between them:
+    size_t scratch_bytes = 0;            // placement and read-outs build their answers there
 
     bool general[kMaxSpecies] = {};
     // automatic stretch kernel (psc_options.tiles = 0) of species with a tile
@@ -157,7 +157,8 @@ struct psc_lattice {
     int64_t next_id_known = 0;             // Scalars::next_id after event next_id_g
     uint32_t next_id_g = 0;
     int32_t grid_class[kMaxSpecies] = {};  // per-event grid limit of each list (INT32_MAX: none)
-    int32_t* counts_h = nullptr;
+    int32_t* counts_h = nullptr;           // a registered page
+    int32_t state[128] = {};               // Scalars' counts to err, as check_device found them
     cudaEvent_t counts_ev = nullptr;
     bool counts_pending = false;
     uint32_t counts_g = 0;       // capturing one event: its last launch advances Scalars::g_base
