@@ -1620,8 +1620,8 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     // ---- placement (Sec. 3.4): voxels in (Philox key, voxel) order, per
     // compartment, dealt to the species.  Only the first voxels of each
     // compartment matter: a histogram of the keys' top bits finds the bin
-    // that covers them, and only the voxels up to it are sorted (by voxel,
-    // then stably by key, then by compartment). ----
+    // that covers them, and only the voxels up to it are sorted (by key, equal
+    // keys by voxel, then stably by compartment). ----
     if (N > 0) {
         const int nc = comps ? L->ncomp : 1;
         const int bins = 1 << kPlaceBits;
@@ -1674,11 +1674,13 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         sort_scratch_bind(ss, scratch, M);
         launch_place_pick((uint32_t)V, (uint32_t)seed, (uint32_t)(seed >> 32), labels_d, lim, cvox, ckey, pick_n,
                           (int32_t)M, &L->sc->err, fill_blocks, st);
-        int vbits = 1;
-        while (vbits < 31 && ((int64_t)1 << vbits) < L->V) ++vbits;
-        if (radix_sort_pairs(cvox, ckey, nullptr, M, M, vbits, ss, st, &L->launches) != 0 ||
-            radix_sort_pairs(ckey, cvox, nullptr, M, M, 32, ss, st, &L->launches) != 0)
+        int kbits = 32 - kPlaceBits;                   // of the candidates' keys
+        for (int c = 0; c < nc; ++c)
+            while (kbits < 32 && (lim.bin[c] >> (kbits - (32 - kPlaceBits))) > 0) ++kbits;
+        if (radix_sort_pairs(ckey, cvox, nullptr, M, M, kbits, ss, st, &L->launches) != 0)
             return cuda_fail(L, cudaErrorUnknown);
+        launch_sort_ties(ckey, cvox, M, fill_blocks, st);
+        L->launches += 1;
         if (comps) {
             launch_label_keys(cvox, labels_d, ckey, M, fill_blocks, st);
             if (radix_sort_pairs(ckey, cvox, nullptr, M, M, 8, ss, st, &L->launches) != 0)

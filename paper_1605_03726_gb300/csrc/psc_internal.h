@@ -562,6 +562,8 @@ size_t sort_scratch_bytes(int64_t max_n);
 void sort_scratch_bind(SortScratch& s, void* base, int64_t max_n);
 // exclusive scan of data[len] in place; sums: a word per 4096 of them
 void exclusive_scan(uint32_t* data, int64_t len, uint32_t* sums, cudaStream_t st, int64_t* launches);
+// values of equal keys, side by side after a sort, into ascending order
+void launch_sort_ties(const uint32_t* keys, uint32_t* vals, int64_t n, int blocks, cudaStream_t st);
 // After the call the sorted data is in (keys, vals) again.
 int radix_sort_pairs(uint32_t* keys, uint32_t* vals, const int32_t* n_dev, int64_t n_host,
                      int64_t max_n, int bits, SortScratch& scratch, cudaStream_t st,

@@ -203,6 +203,28 @@ void exclusive_scan(uint32_t* data, int64_t len, uint32_t* sums, cudaStream_t st
     if (launches) *launches += 3;
 }
 
+// Pairs sorted by key: the values of equal keys into ascending order.  Keys are
+// 32-bit draws, so a run of equal ones is a pair of them, seldom more: its first
+// thread sorts it where it stands.
+__global__ void k_sort_ties(const uint32_t* keys, uint32_t* vals, int64_t n)
+{
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r + 1 < n; r += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t k = keys[r];
+        if (keys[r + 1] != k || (r > 0 && keys[r - 1] == k)) continue;
+        for (int64_t x = r + 1; x < n && keys[x] == k; ++x) {
+            const uint32_t v = vals[x];
+            int64_t y = x;
+            for (; y > r && vals[y - 1] > v; --y) vals[y] = vals[y - 1];
+            vals[y] = v;
+        }
+    }
+}
+
+void launch_sort_ties(const uint32_t* keys, uint32_t* vals, int64_t n, int blocks, cudaStream_t st)
+{
+    k_sort_ties<<<blocks, 256, 0, st>>>(keys, vals, n);
+}
+
 int radix_sort_pairs(uint32_t* keys, uint32_t* vals, const int32_t* n_dev, int64_t n_host,
                      int64_t max_n, int bits, SortScratch& s, cudaStream_t st, int64_t* launches)
 {
@@ -210,18 +232,15 @@ int radix_sort_pairs(uint32_t* keys, uint32_t* vals, const int32_t* n_dev, int64
     if (max_n > s.max_n) return -1;
     const int tiles = (int)ceil_div(max_n, kSortTile);
     const int64_t hist_len = 256 * (int64_t)tiles;
-    const int scan_blocks = (int)ceil_div(hist_len, kScanTile);
     int passes = (bits + 7) / 8;
     if (passes & 1) ++passes;           // even: the result lands back in (keys, vals)
     uint32_t *ki = keys, *vi = vals, *ko = s.keys_alt, *vo = s.vals_alt;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
         k_hist<<<tiles, kSortThreads, 0, st>>>(ki, n_dev, n_host, shift, s.hist, tiles);
-        k_scan_reduce<<<scan_blocks, kScanThreads, 0, st>>>(s.hist, hist_len, s.block_sums);
-        k_scan_sums<<<1, kScanThreads, 0, st>>>(s.block_sums, scan_blocks);
-        k_scan_down<<<scan_blocks, kScanThreads, 0, st>>>(s.hist, hist_len, s.block_sums);
+        exclusive_scan(s.hist, hist_len, s.block_sums, st, launches);
         k_scatter<<<tiles, kSortThreads, 0, st>>>(ki, vi, ko, vo, n_dev, n_host, shift, s.hist, tiles);
-        if (launches) *launches += 5;
+        if (launches) *launches += 2;
         uint32_t* t = ki; ki = ko; ko = t;
         t = vi; vi = vo; vo = t;
     }
