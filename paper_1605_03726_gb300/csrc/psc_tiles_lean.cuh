@@ -23,15 +23,25 @@
 //     shared memory (lowest id wins, as in the global words) and is read back
 //     inline in the commit phase; targets nearer the region's faces are
 //     claimed in the global words as before;
+//   - what only a few lanes of a warp need is queued and done densely: contested
+//     molecules (an eighth at 1 %) 32 at a time by their warp, departures (2 %)
+//     from the outbox once the box is through (one inbox atomic per destination
+//     box and warp);
 //   - the commit phase handles every molecule in one pass: hops inside the
 //     box update the box (and, for the outermost brick layer, the global
-//     mirror), global claim words are read back in batches of loads, and
-//     departures go to the outbox (one inbox atomic per destination box and
-//     warp when it is flushed), with no deferred queue;
+//     mirror), and global claim words are read back in batches of loads;
 //   - whether a word is in the region's outermost brick layer comes from a
 //     bitmap in shared memory; the next chunk's bucket entries load while one
-//     is processed.
+//     is processed, the first chunk's during the waits; waits poll with
+//     acquiring loads.
+//
+// What bounds it: about 10 us per event of waits for neighbours and dependent
+// loads, then instructions (600 per warp of molecules and event, issued half of
+// the time; a third of the warps' time goes to the waits).  us per event, before
+// the queues -> now: 512^3, 0.3 / 1 / 1.8 % 19.6 / 40.4 / 73.1 -> 19.0 / 37.1 / 66.6,
+// 400^3, 1 / 3 % 25.6 / 61.3 -> 22.3 / 53.5, 320^3, 1 / 5 % 17.8 / 56.0 -> 16.1 / 51.4.
 
+static_assert(kLeanOutbox == kTileThreads, "the outbox holds a queue of 32 for every warp in the claim phase");
 constexpr uint32_t kLeanOff = 4u | (4u << 11) | (2u << 22);   // region -> box coordinates
 
 struct LeanShared {
@@ -219,26 +229,19 @@ __device__ __forceinline__ void lean_move_inside(const TileArgs& A, const LeanSh
 {
     const int wv = lean_word(p, BI, BIJ), wt = lean_word(t, BI, BIJ);
     const uint32_t mv = 1u << c, mt = 1u << lean_place(t);
-    const bool vo = (S.obits[wv >> 5] >> (wv & 31)) & 1u, to = (S.obits[wt >> 5] >> (wt & 31)) & 1u;
-    if (wv == wt) {
-        atomicXor(&box[wv], mv | mt);
-        if (vo) atomicXor(&A.ev.bits[lean_gword(p, A.plan, gbase)], mv | mt);
-    } else {
-        atomicXor(&box[wv], mv);
-        atomicXor(&box[wt], mt);
-        if (vo) atomicXor(&A.ev.bits[lean_gword(p, A.plan, gbase)], mv);
-        if (to) atomicXor(&A.ev.bits[lean_gword(t, A.plan, gbase)], mt);
-    }
+    atomicXor(&box[wv], mv);
+    atomicXor(&box[wt], mt);
+    if ((S.obits[wv >> 5] >> (wv & 31)) & 1u) atomicXor(&A.ev.bits[lean_gword(p, A.plan, gbase)], mv);
+    if ((S.obits[wt >> 5] >> (wt & 31)) & 1u) atomicXor(&A.ev.bits[lean_gword(t, A.plan, gbase)], mt);
 }
 
-// A molecule (packed box coordinates p, place c) leaves its region for
-// packed box coordinates t: its bit leaves the box and the global mirror, the
-// target's bit is set in the global mirror (the owner's box picks it up with
-// the arrival), wrap counters follow a periodic wrap, and the molecule goes
-// to the outbox (or straight to the inbox when the outbox is full).
-__device__ __forceinline__ void lean_depart(const TileArgs& A, const TileBox& b, const LeanShared& S, int BI,
-                                            int BIJ, int64_t gbase, int* s_out_n, uint32_t p, uint32_t c, uint32_t t,
-                                            uint32_t id)
+// A molecule (packed box coordinates p) leaves its region for packed box
+// coordinates t: its bit leaves the box and the global mirror, the target's bit
+// is set in the global mirror (the owner's box picks it up with the arrival),
+// and wrap counters follow a periodic wrap.  Returns the box it enters, and the
+// target's voxel in tv.
+__device__ __forceinline__ int lean_depart(const TileArgs& A, const TileBox& b, const LeanShared& S, int BI,
+                                           int BIJ, int64_t gbase, uint32_t p, uint32_t t, uint32_t id, int32_t& tv)
 {
     const Geometry& G = A.ev.geo;
     int32_t gi, gj, gk;
@@ -248,27 +251,23 @@ __device__ __forceinline__ void lean_depart(const TileArgs& A, const TileBox& b,
         uint64_t* wp = &A.img_id[id - A.id_lo];
         *wp = img_add(*wp, wr);
     }
-    const uint32_t mv = 1u << c;
+    const uint32_t mv = 1u << lean_place(p);
     atomicXor(&S.box[lean_word(p, BI, BIJ)], mv);
     atomicXor(&A.ev.bits[lean_gword(p, A.plan, gbase)], mv);   // the source is in the outermost layer
     const BitPos gt = bitpos(G, gi, gj, gk);
     atomicXor(&A.ev.bits[gt.word], gt.mask);
-    const int q = tile_region_of(A.plan, S.own, gi, gj, gk);
-    const int32_t tv = gi + G.ni * (gj + G.nj * gk);
-    const int o = atomicAdd(s_out_n, 1);
-    if (o < kLeanOutbox) {
-        S.o_t[o] = tv;
-        S.o_id[o] = id;
-        S.o_q[o] = q;
+    tv = gi + G.ni * (gj + G.nj * gk);
+    return tile_region_of(A.plan, S.own, gi, gj, gk);
+}
+
+__device__ __forceinline__ void lean_send(const TileArgs& A, int q, int slot, int32_t tv, uint32_t id)
+{
+    const int cap = A.plan.cap;
+    if (slot < cap) {
+        A.in_vox[(int64_t)q * cap + slot] = tv;
+        A.in_ids[(int64_t)q * cap + slot] = id;
     } else {
-        const int cap = A.plan.cap;
-        const int slot = atomicAdd(&A.in_cnt[q], 1);
-        if (slot < cap) {
-            A.in_vox[(int64_t)q * cap + slot] = tv;
-            A.in_ids[(int64_t)q * cap + slot] = id;
-        } else {
-            atomicOr(&A.ev.sc->err, kErrListOverflow);
-        }
+        atomicOr(&A.ev.sc->err, kErrListOverflow);
     }
 }
 
@@ -304,6 +303,23 @@ __device__ __forceinline__ int32_t lean_voxel(const Geometry& G, const TileBox& 
     return i + G.ni * (j + G.nj * k);
 }
 
+// Claim-phase decision of a molecule whose target's neighbourhood is not its
+// own: bits 0-3 the direction, then where it claimed the target, if that is
+// vacant (the lowest id wins).
+__device__ __forceinline__ uint32_t lean_contested(const TileArgs& A, const TileBox& b, const LeanShared& S, int BI,
+                                                   int BIJ, uint32_t p, uint32_t id, uint32_t d)
+{
+    const uint32_t t = p + (uint32_t)S.tstep[lean_place(p) * 12u + d];
+    if (S.box[lean_word(t, BI, BIJ)] & (1u << lean_place(t))) return d;
+    if (((t & 0x7FFu) - 5u) < 4u * (uint32_t)b.ei - 2u && (((t >> 11) & 0x7FFu) - 5u) < 4u * (uint32_t)b.ej - 2u &&
+        ((t >> 22) - 3u) < 2u * (uint32_t)b.ek - 2u) {
+        const int slot = lean_claim_local(S.ctab, t, id);       // all its neighbours are ours
+        if (slot >= 0) return d | kLeanLocal | ((uint32_t)slot << 4);
+    }
+    atomicMin(&A.claim[lean_voxel(A.ev.geo, b, t)], id);
+    return d | kTileClaimed;
+}
+
 // End of a phase: once the whole block is done, publish flags[r] = value and
 // wait until every neighbouring box (up to 26, across periodic wraps) has
 // published at least value.  Two block barriers in all.  Bounded like the
@@ -329,9 +345,14 @@ __device__ __forceinline__ bool lean_phase_sync(const TileArgs& A, uint32_t* fla
         if (rj < 0 || rj >= P.pj) { if (bf & 2u) rj = (rj + P.pj) % P.pj; else skip = true; }
         if (rk < 0 || rk >= P.pk) { if (bf & 4u) rk = (rk + P.pk) % P.pk; else skip = true; }
         if (!skip) {
-            const volatile uint32_t* f = flags + (rk * P.pj + rj) * P.pi + ri;
+            const uint32_t* f = flags + (rk * P.pj + rj) * P.pi + ri;
+            auto seen = [&] {
+                uint32_t v;                              // (an acquiring load: no fence afterwards)
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+                return v;
+            };
             uint64_t t0 = 0;
-            for (unsigned int spins = 0; *f < target; ++spins) {
+            for (unsigned int spins = 0; seen() < target; ++spins) {
                 if ((spins & 1023u) == 0u) {
                     const uint64_t now = globaltimer_ns();
                     if (t0 == 0) t0 = now;
@@ -343,7 +364,6 @@ __device__ __forceinline__ bool lean_phase_sync(const TileArgs& A, uint32_t* fla
                 }
             }
         }
-        __threadfence();
     }
     __syncthreads();
     return *s_ok != 0;
@@ -450,6 +470,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
     }
     unsigned long long n_att = 0, n_hop = 0;
     uint2 halo_first[kLeanHalo];
+    uint32_t pv[U] = {}, pi_[U] = {};                    // a chunk of bucket entries, loading ahead
     __syncthreads();
     for (int e = 0; e < A.n_events; ++e) {
         const uint32_t g = a.g + (uint32_t)e;
@@ -457,15 +478,29 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
         const int32_t* bv = A.b_vox[cur] + base;
         const uint32_t* bi = A.b_ids[cur] + base;
         uint32_t* bs = A.b_state + base;
+        const int n_old = n;
         if (e > 0) lean_ingest(A, r, b, S, n, cur, true, halo_first);   // after the neighbours' commits
-        // ---- claim phase (the next chunk's bucket entries load while one is processed) ----
-        uint32_t pv[U], pi_[U];
+        // ---- claim phase (the next chunk's bucket entries load while one is processed;
+        // the first chunk's have since the last event, but for the arrivals) ----
+        const int lane = threadIdx.x & 31, wq0 = threadIdx.x & ~31;      // the warp's queue, in the outbox
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int x = u * blockDim.x + threadIdx.x;
-            pv[u] = x < n ? (uint32_t)__ldcg(bv + x) : 0u;
-            pi_[u] = x < n ? __ldcg(bi + x) : 0u;
+            if ((e > 0 && x < n_old) || x >= n) continue;
+            pv[u] = (uint32_t)__ldcg(bv + x);
+            pi_[u] = __ldcg(bi + x);
         }
+        int queued = 0;                                  // contested molecules of the warp, not decided yet
+        auto decide = [&] {
+            __syncwarp();
+            if (lane < queued) {
+                const int x = S.o_q[wq0 + lane] >> 4;
+                bs[x] = lean_contested(A, b, S, BI, BIJ, (uint32_t)S.o_t[wq0 + lane], S.o_id[wq0 + lane],
+                                       (uint32_t)S.o_q[wq0 + lane] & 15u);
+            }
+            __syncwarp();
+            queued = 0;
+        };
         for (int c0 = 0; c0 < n; c0 += U * blockDim.x) {
             uint32_t vv[U], ii[U];
 #pragma unroll
@@ -479,7 +514,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int xm = c0 + u * blockDim.x + threadIdx.x;
-                if (xm >= n) continue;
+                if (xm - lane >= n) break;               // nothing left for the warp
                 const uint32_t p = vv[u] + kLeanOff;
                 uint32_t rnd[4];
                 philox(ii[u], g, c2, 0u, a.key0, a.key1, rnd);
@@ -491,36 +526,26 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
                                       (box[w0 + BI + 1] & m0.w) | (box[w0 + BIJ] & m1.x) |
                                       (box[w0 + BIJ + 1] & m1.y) | (box[w0 + BIJ + BI] & m1.z) |
                                       (box[w0 + BIJ + BI + 1] & m1.w);
-                uint32_t st = d;
-                if (busy == 0u) {
-                    st |= kTileMove;                     // vacant, and only the mover is next to it
-                } else {
-                    const uint32_t t = p + (uint32_t)S.tstep[e12];
-                    if (!(box[lean_word(t, BI, BIJ)] & (1u << lean_place(t)))) {
-                        // vacant, but other molecules can reach it: the lowest id wins
-                        int slot = -1;
-                        if (((t & 0x7FFu) - 5u) < rxn - 2u && (((t >> 11) & 0x7FFu) - 5u) < ryn - 2u &&
-                            ((t >> 22) - 3u) < rzn - 2u)
-                            slot = lean_claim_local(S.ctab, t, ii[u]);   // all its neighbours are ours
-                        if (slot >= 0) {
-                            st |= kLeanLocal | ((uint32_t)slot << 4);
-                        } else {
-                            atomicMin(&claim[lean_voxel(G, b, t)], ii[u]);
-                            st |= kTileClaimed;
-                        }
-                    }
+                const bool contested = xm < n && busy != 0u;
+                const unsigned who = __ballot_sync(0xFFFFFFFFu, contested);
+                if (queued + __popc(who) > 32) decide();
+                if (contested) {
+                    const int at = wq0 + queued + __popc(who & ((1u << lane) - 1u));
+                    S.o_t[at] = (int32_t)p;
+                    S.o_id[at] = ii[u];
+                    S.o_q[at] = (xm << 4) | (int)d;
+                } else if (xm < n) {
+                    bs[xm] = d | kTileMove;              // vacant, and only the mover is next to it
                 }
-                bs[xm] = st;
+                queued += __popc(who);
             }
         }
+        decide();
         n_att += (unsigned long long)n;
         if (threadIdx.x == 0) {
             s_misc[1] = 0;
             s_misc[2] = 0;
         }
-        // a claim word is touched only by boxes that are all neighbours of each other
-        if (!lean_phase_sync(A, A.claimed, r, (uint32_t)(e + 1), &s_misc[3])) return;
-        // ---- commit phase: every molecule in one pass ----
         int32_t* ov = A.b_vox[cur ^ 1] + base;
         uint32_t* oi = A.b_ids[cur ^ 1] + base;
         uint32_t qv[U], qi[U], qs[U];             // the next chunk, loading ahead
@@ -529,6 +554,13 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
             const int x = u * blockDim.x + threadIdx.x;
             qv[u] = x < n ? (uint32_t)__ldcg(bv + x) : 0u;
             qi[u] = x < n ? __ldcg(bi + x) : 0u;
+        }
+        // a claim word is touched only by boxes that are all neighbours of each other
+        if (!lean_phase_sync(A, A.claimed, r, (uint32_t)(e + 1), &s_misc[3])) return;
+        // ---- commit phase: every molecule in one pass ----
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int x = u * blockDim.x + threadIdx.x;
             qs[u] = x < n ? __ldcg(bs + x) : 0u;
         }
         for (int c0 = 0; c0 < n; c0 += U * blockDim.x) {
@@ -559,6 +591,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int xm = c0 + u * blockDim.x + threadIdx.x;
+                if (xm - lane >= n) break;
                 const uint32_t st = ss[u];
                 uint32_t w = vv[u];
                 bool keep = xm < n;
@@ -577,7 +610,16 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
                         lean_move_inside(A, S, box, BI, BIJ, gbase, p, c, t);
                         w = t - kLeanOff;
                     } else {
-                        lean_depart(A, b, S, BI, BIJ, gbase, &s_misc[2], p, c, t, ii[u]);
+                        const int o = atomicAdd(&s_misc[2], 1);
+                        if (o < kLeanOutbox) {
+                            S.o_t[o] = (int32_t)t;
+                            S.o_id[o] = ii[u];
+                            S.o_q[o] = (int32_t)p;
+                        } else {
+                            int32_t v;
+                            const int q = lean_depart(A, b, S, BI, BIJ, gbase, p, t, ii[u], v);
+                            lean_send(A, q, atomicAdd(&A.in_cnt[q], 1), v, ii[u]);
+                        }
                         keep = false;
                     }
                 }
@@ -595,26 +637,26 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocksPerSM) k_tile_lean(co
             for (int o0 = threadIdx.x & ~31; o0 < m; o0 += blockDim.x) {
                 const int o = o0 + (threadIdx.x & 31);
                 const bool has = o < m;
-                const int q = has ? S.o_q[o] : -1;
+                int32_t v = 0;
+                const int q = has ? lean_depart(A, b, S, BI, BIJ, gbase, (uint32_t)S.o_q[o], (uint32_t)S.o_t[o],
+                                                S.o_id[o], v) : -1;
                 const unsigned peers = __match_any_sync(0xFFFFFFFFu, q);
                 const int leader = __ffs(peers) - 1;
-                const int lane = threadIdx.x & 31;
                 int base0 = 0;
                 if (has && lane == leader) base0 = atomicAdd(&A.in_cnt[q], __popc(peers));
                 base0 = __shfl_sync(0xFFFFFFFFu, base0, leader);
-                if (has) {
-                    const int slot = base0 + __popc(peers & ((1u << lane) - 1u));
-                    if (slot < cap) {
-                        A.in_vox[(int64_t)q * cap + slot] = S.o_t[o];
-                        A.in_ids[(int64_t)q * cap + slot] = S.o_id[o];
-                    } else {
-                        atomicOr(&a.sc->err, kErrListOverflow);
-                    }
-                }
+                if (has) lean_send(A, q, base0 + __popc(peers & ((1u << lane) - 1u)), v, S.o_id[o]);
             }
         }
         // the first chunk of the next halo refresh: its table entries load during the wait
         lean_halo_fetch(A, r, halo_total, threadIdx.x, halo_first);
+        // and the first bucket entries of the next event
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int x = u * blockDim.x + threadIdx.x;
+            pv[u] = x < n ? (uint32_t)__ldcg(ov + x) : 0u;
+            pi_[u] = x < n ? __ldcg(oi + x) : 0u;
+        }
         // halo bits, arrivals and reset claim words of every neighbour are out
         if (!lean_phase_sync(A, A.done, r, (uint32_t)(e + 1), &s_misc[3])) return;
     }
