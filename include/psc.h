@@ -152,8 +152,9 @@ typedef struct {
     int32_t persistent;       /* 1 = run stretches of events in one launch
                                  (default): of a lattice without reactions and
                                  compartments whose molecules fit in shared
-                                 memory (up to 2.8 million, 28 million voxels),
-                                 all its species in turn; of any lattice of up
+                                 memory (up to 2.8 million, 28 million voxels;
+                                 up to 2^27 voxels with less than 262,144 of
+                                 each species), all its species in turn; of any lattice of up
                                  to 2^26 voxels with a claim word per voxel, its
                                  species in scheduler order, while no mobile
                                  species has more than 2^22 molecules (without

@@ -1034,6 +1034,16 @@ static int64_t walk_slots(const psc_lattice* L, int64_t threads)
     return slots;
 }
 
+// A lattice of a size that k_walk_run takes with its molecules
+static bool walk_size(const psc_lattice* L)
+{
+    if (L->V <= kWalkVoxels) return true;
+    if (L->V > kWalkVoxelsFew) return false;
+    for (int s = 0; s < L->nsp; ++s)
+        if (L->sp[s].D > 0.0 && L->sp[s].n0 >= kOpenList) return false;
+    return true;
+}
+
 // Can the lattice's events run in stretches of k_walk_run?  No reactions, no
 // compartments, a claim word per voxel, molecules that fit in shared memory.
 static bool walk_fits(psc_lattice* L, int s)
@@ -1041,7 +1051,7 @@ static bool walk_fits(psc_lattice* L, int s)
     // (kernel timing keeps to the kernels it tells apart)
     if (!L->walk_only || !L->claim || L->opt.persistent <= 0 || L->opt.run_per_thread > 0 || L->opt.time_kernels > 0)
         return false;
-    if (L->V > kWalkVoxels) return false;
+    if (!walk_size(L)) return false;
     if (!L->shapes_known) device_shapes(L);
     if (walk_slots(L, (int64_t)kWalkThreads * L->sm_count) * kWalkThreads * 12 > L->walk_smem) return false;
     TilePlan P{};
@@ -1482,12 +1492,12 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     L->batchable = direct || 2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V;
     if (L->opt.claim_table == 1) L->batchable = true;
     if (L->opt.claim_table == 2 && hb_max > 0) L->batchable = false;
-    // lattices without reactions whose claim words fit in the L2 cache take
-    // k_walk_run while their molecules fit in shared memory
+    // lattices without reactions take k_walk_run while their molecules fit in
+    // shared memory
     L->walk_only = L->nrx == 0 && !comps && L->opt.subvolume <= 0;
-    if (L->walk_only && L->V <= kWalkVoxels &&
-        walk_slots(L, (int64_t)kWalkThreads * L->sm_count) * kWalkThreads * 12 <= kWalkSmem)
-        direct = true;
+    const bool walk = L->walk_only && walk_size(L) &&
+                      walk_slots(L, (int64_t)kWalkThreads * L->sm_count) * kWalkThreads * 12 <= kWalkSmem;
+    if (walk && L->V <= kWalkVoxels) direct = true;
     // tables at least as large as a word per voxel buy nothing, and the
     // per-event kernels empty the previous table in full every event (species
     // that are reaction products get lists sized for the lattice)
@@ -1505,18 +1515,20 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     bool stretch = L->stretches && L->V <= kCellVoxels && L->opt.subvolume <= 0;
     for (int s = 0; s < L->nsp; ++s)
         stretch = stretch && (!(L->sp[s].D > 0.0) || L->sp[s].n0 <= (L->nrx > 0 ? kSmallList : kSmallWalk));
+    stretch = stretch || (L->stretches && walk);
     if (L->opt.claim_table == 1) direct = true;
     if (L->opt.claim_table == 2 && hb_max > 0) direct = open = stretch = false;
+    // (k_walk_run orders them as the mirror's bits, whole bricks)
+    const int64_t claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
     if ((open || stretch) && !direct) {
-        L->claim_n = L->V;
-        L->claim = (uint32_t*)dev_alloc(L, V * sizeof(uint32_t));
+        L->claim_n = claim_n;
+        L->claim = (uint32_t*)dev_alloc(L, (size_t)claim_n * sizeof(uint32_t));
         direct = L->claim != nullptr;                // no room: tables
         if (!direct) cudaGetLastError();
     }
     L->open_claims = open && direct;
     if (direct && !L->claim) {
-        // (k_walk_run orders them as the mirror's bits, whole bricks)
-        L->claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
+        L->claim_n = claim_n;
         carve.add(&L->claim, (size_t)L->claim_n * sizeof(uint32_t));
     } else if (!direct) {
         L->table_slots = (int64_t)1 << hb_max;

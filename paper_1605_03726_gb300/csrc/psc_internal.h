@@ -308,7 +308,14 @@ constexpr int64_t kWalkCluster = 16384;    // molecules a cluster takes
 // event either way, 629,000 on 128^3 13.7 sorted every 64 events, 15.1 unsorted.
 constexpr int64_t kWalkSorted = 200000;
 constexpr int kWalkClusterSmem = 36 * 1024;        // shared memory of its blocks, at most
-constexpr int64_t kWalkVoxels = 28000000;  // largest lattice that gets claim words for it (112 MB)
+// Largest lattice that runs in them, its claim words in the L2 cache (112 MB);
+// and with lists shorter than kOpenList, where the claims are too few for that
+// to matter: 100,000 walkers on 320^3 9.3 -> 7.0 us per event (k_small_run),
+// 200,000 on 400^3 17.2 -> 10.2 (tables, a launch per phase), 125,000 on 500^3
+// 15.2 -> 10.9; but 640,000 on 400^3 22.1 -> 32, 400,000 on 500^3 19.3 -> 24.9
+// (the lean tile kernel).
+constexpr int64_t kWalkVoxels = 28000000;
+constexpr int64_t kWalkVoxelsFew = 1 << 27;
 constexpr int64_t kWalkSmem = 225 * 1024;  // shared memory of its blocks
 struct WalkArgs {
     Geometry geo;

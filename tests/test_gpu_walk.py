@@ -33,6 +33,7 @@ CASES = [
     ("ragged_mixed", (37, 30, 23), 2, walkers((0.0, 4000), (1e-12, 6000), (3e-12, 900)), (1, 130)),
     ("fcc", (41, 28, 36), 7 | psc.FCC, walkers((2e-12, 9000), (2e-12, 300)), (1, 130)),
     ("fcc_walls", (33, 27, 31), psc.PERIODIC_I | psc.FCC, walkers((1e-12, 14000)), (90,)),
+    ("large_few", (320, 304, 290), 5, walkers((1e-12, 20000), (0.4e-12, 300)), (1, 130)),
     ("sorted_two", (96, 80, 64), 7, walkers((1e-12, 210000), (0.8e-12, 205000), (0.0, 30000)), (70, 90)),
 ]
 
