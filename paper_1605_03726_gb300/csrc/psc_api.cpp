@@ -1510,8 +1510,8 @@ int psc_populate(psc_lattice* L, uint64_t seed)
                         L->opt.subvolume <= 0);
     // the rest, as far as their events run in stretches of k_small_run (tables and
     // a launch per phase before: A + B <-> C of 2000 + 1000 molecules on 200^3 9.9 ->
-    // 3.9 us per event, 200,000 + 100,000 on 256^3 27.5 -> 15.8, 100,000 + 50,000 on
-    // 400^3 24.6 -> 12.9; 60,000 walkers on 400^3 15.9 -> 6.0)
+    // 3.9 us per event, 200,000 + 100,000 on 256^3 27.5 -> 15.1, 100,000 + 50,000 on
+    // 400^3 24.6 -> 12.2; 60,000 walkers on 400^3 15.9 -> 4.7)
     bool stretch = L->stretches && L->V <= kCellVoxels && L->opt.subvolume <= 0;
     for (int s = 0; s < L->nsp; ++s)
         stretch = stretch && (!(L->sp[s].D > 0.0) || L->sp[s].n0 <= (L->nrx > 0 ? kSmallList : kSmallWalk));

@@ -274,8 +274,9 @@ constexpr int64_t kCellIds = (1ll << 27) - (1ll << 23);    // next id when a str
 // (128^3: 63,000 walkers 6.0 us per event against 10.8, 210,000 14.4 against 13.0).
 constexpr int64_t kSmallList = 1 << 22;
 constexpr int64_t kSmallWalk = 131072;
-// The longest list that runs in one cluster of 16 blocks: 16,000 molecules take
-// 3.1 us per event there and 4.8 in a grid, 30,000 13.1 and 6.8.
+// The longest list that runs in one cluster of 16 blocks: A + B -> C of 2000
+// molecules each takes 4.2 us per event there and 6.3 in a grid, of 12,000 6.4 and
+// 6.7, of 24,000 10.3 and 6.8.
 constexpr int64_t kSmallCluster = 16384;
 struct SmallArgs {
     const EventArgs* ev;       // [nsp] templates on the device (event_args with g unset)

@@ -35,9 +35,11 @@
 // replayed from CUDA graphs, or the molecule-list kernel for walkers): A + B -> C
 // of 2000 + 2000 molecules on 64^3 12.5 -> 4.2, a cascade of 22 species of up to
 // 16,000 molecules on 200^3 10.5 -> 3.1, 30,000 ligands and 5000 receptors in a
-// cell on 128^3 19.8 -> 6.8, reversible A + B <-> C under 30 % crowding with 839,000
-// A on 256^3 40.0 -> 25.3, with 1.6M on 320^3 92 -> 52, with 3.2M on 400^3
-// 180 -> 126.  The order of a list makes no difference here (26.3 sorted on
+// cell on 128^3 19.8 -> 6.2, reversible A + B <-> C under 30 % crowding with 839,000
+// A on 256^3 40.0 -> 24.6, with 1.6M on 320^3 92 -> 48, with 3.2M on 400^3
+// 180 -> 126.  Tried: the next event's entries read, and their draws made, before
+// the barrier that ends an event (the first 4.2 -> 4.5, the second 3.1 -> 3.7: every
+// thread's extra instructions cost more than the load they hide).  The order of a list makes no difference here (26.3 sorted on
 // 256^3), so these stretches have no re-sorts.
 
 // Event arguments and model of the lattice, copied to shared memory once per
@@ -700,6 +702,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(const SmallArgs 
 
 // Stretches of many lattices in one cooperative launch, each with a group of
 // consecutive blocks and at its own pace: no lattice waits for another.
+// Measured (us for an event of every member, the first 64 events / after 450;
+// before: a launch per phase for all of them): 64 members of 96^3 with 5 % A and B
+// 171 / 31 -> 106 / 15; 64 of 160^3 with 2 % 446 / 155 -> 261 / 74, bound by
+// scattered DRAM accesses, as the members' cells are 1 GB.
 // counts: list lengths and next id afterwards, [lattice][kSmallCounts], for the
 // next launch's groups.
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArgs* args, const int2* group,

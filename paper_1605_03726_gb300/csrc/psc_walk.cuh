@@ -24,7 +24,14 @@
 //     while the read-backs are on their way.
 // Several species may take turns in a stretch; immobile ones are voxels whose
 // word is 0.
-// Tried: claims that return the old value, with losses noted through a map
+// Measured (us per event; before: the molecule-list kernel, the tile kernels one
+// species at a time): 2621 walkers on 64^3 8.2 -> 3.2, 1.23M (30 %) on 160^3
+// 39.2 -> 19.5, 708,000 on FCC 192^3 37.7 -> 15.4, 797,000 on 301 x 251 x 211
+// 39.6 -> 17.8, two species of 503,000 and 336,000 among crowders on 256^3
+// 69.7 -> 13.2.
+// Tried: the words in the shared memory of a cluster, for lattices they fit in
+// (2621 walkers on 64^3 the same, 16,000 on 92^3 6.5 against 5.1: minima on another
+// SM's memory are slower than L2's).  Claims that return the old value, with losses noted through a map
 // from id to list entry instead of the read-back (two accesses): a returning
 // atomic takes as long as a claim and a read-back (160^3 at 30 % 22.3 us per
 // event against 22.0, 256^3 at 5 % 18.5 against 19.9, 2621 walkers on 64^3 3.4
