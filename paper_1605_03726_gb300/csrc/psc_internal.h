@@ -353,8 +353,8 @@ void launch_commit(const EventArgs& a, bool general, int blocks, int threads, cu
 void launch_open_claim(const EventArgs& a, int64_t n, int sm_count, cudaStream_t st);
 void launch_open_commit(const EventArgs& a, int64_t n, int sm_count, cudaStream_t st);
 constexpr int64_t kOpenList = 1 << 18;      // shortest list they take
-// Where the lean tile kernel can run, it does up to here: 2.0M walkers on 512^3
-// 60.5 us per event against 70.6, 2.7M 85.3 against 82.7, 3.4M 118 against 104.
+// Where the lean tile kernel can run, it does up to here: 2.5M walkers on 512^3
+// 70.7 us per event against 73.0, 2.7M 79.9 against 76.8, 3.4M 118 against 101.
 // (The general tile kernel never: 1.4M on a ragged lattice 102 against 45.)
 constexpr int64_t kOpenOverLean = 2600000;
 // claim, commit and the own-list fill of one event of a species with

@@ -9,10 +9,12 @@
 // to eight mirror words around the target; in a list in Morton order a block's
 // molecules share them in the L1 cache (the mirror does not change during the
 // claim launch), so each block takes a stretch of consecutive entries.
+// Entries load a row or two ahead: a thread's loads would otherwise be one chain
+// per molecule (1024^3 339 us per event without, 512^3 338, the closed one 172).
 // Measured, us per event (before: plain claims of every hop in hash tables, or
 // the tile kernel where its boxes fit in shared memory): 10.7M walkers on
-// 1024^3 843 -> 335, 9.4M on 512^3 547 -> 337, 4.8M on a closed
-// 401 x 399 x 301 lattice 348 -> 174, 9.8M on 320^3 (30 %) 407 -> 290.
+// 1024^3 843 -> 331, 9.4M on 512^3 547 -> 325, 4.8M on a closed
+// 401 x 399 x 301 lattice 348 -> 167.
 constexpr uint8_t kDecOpen = 16;            // flag: hop without a claim, direction in the low bits
 
 // Occupied voxels among the target (ti, tj, tk) and its neighbours: 1 is the
@@ -108,8 +110,17 @@ __global__ void __launch_bounds__(256, 6) k_open_claim(const EventArgs a)
     int lo, hi;
     open_range(n, lo, hi);
     unsigned n_att = 0;
+    uint32_t v1 = 0u, id1 = 0u;                                 // the next row's entry, on its way
+    if (lo + (int)threadIdx.x < hi) {
+        v1 = (uint32_t)a.list.vox[lo + threadIdx.x];
+        id1 = a.list.ids[lo + threadIdx.x];
+    }
     for (int idx = lo + threadIdx.x; idx < hi; idx += blockDim.x) {
-        const uint32_t v = (uint32_t)a.list.vox[idx], id = a.list.ids[idx];
+        const uint32_t v = v1, id = id1;
+        if (idx + (int)blockDim.x < hi) {
+            v1 = (uint32_t)a.list.vox[idx + blockDim.x];
+            id1 = a.list.ids[idx + blockDim.x];
+        }
         const uint32_t d = walk_draw(a.key0, a.key1, id, g, c2);
         int32_t i, j, k;
         decode(G, v, i, j, k);
@@ -148,9 +159,24 @@ __global__ void __launch_bounds__(256, 6) k_open_commit(const EventArgs a)
             a.ct.clear[x] = kEmptySlot;
     }
     unsigned n_hop = 0;
+    constexpr int A = 2;                                        // rows on their way
+    uint32_t dn[A], vn[A];
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        const int x = lo + u * (int)blockDim.x + (int)threadIdx.x;
+        dn[u] = x < hi ? a.dec[x] : (uint32_t)kDecNone;
+        vn[u] = x < hi ? (uint32_t)a.list.vox[x] : 0u;
+    }
     for (int idx = lo + threadIdx.x; idx < hi; idx += blockDim.x) {
-        const uint32_t dec = a.dec[idx];
-        const uint32_t v = (uint32_t)a.list.vox[idx];
+        const uint32_t dec = dn[0], v = vn[0];
+#pragma unroll
+        for (int u = 0; u + 1 < A; ++u) {
+            dn[u] = dn[u + 1];
+            vn[u] = vn[u + 1];
+        }
+        const int x = idx + A * (int)blockDim.x;
+        dn[A - 1] = x < hi ? a.dec[x] : (uint32_t)kDecNone;
+        vn[A - 1] = x < hi ? (uint32_t)a.list.vox[x] : 0u;
         if (dec == kDecNone) continue;
         int32_t i, j, k;
         decode(G, v, i, j, k);
@@ -171,7 +197,8 @@ __global__ void __launch_bounds__(256, 6) k_open_commit(const EventArgs a)
 
 // Blocks for n entries: one to eight rows of 256 each, so that the longest
 // lists fill several waves and the shortest every SM (a wave is six blocks per
-// SM; 1.34M walkers on 512^3 44 us per event with four rows, 48 with two).
+// SM; 1.34M walkers on 512^3 44 us per event with four rows, 48 with two; 10.7M on
+// 1024^3 331 with eight, 348 with sixteen).
 static int open_blocks(int64_t n, int sm_count)
 {
     const int64_t rows = (n + 255) / 256;

@@ -39,8 +39,9 @@
 // A on 256^3 40.0 -> 24.6, with 1.6M on 320^3 92 -> 48, with 3.2M on 400^3
 // 180 -> 126.  Tried: the next event's entries read, and their draws made, before
 // the barrier that ends an event (the first 4.2 -> 4.5, the second 3.1 -> 3.7: every
-// thread's extra instructions cost more than the load they hide).  The order of a list makes no difference here (26.3 sorted on
-// 256^3), so these stretches have no re-sorts.
+// thread's extra instructions cost more than the load they hide); molecules kept in
+// shared memory between the phases (crowded 256^3 26.1).  The order of a list makes
+// no difference here (26.3 sorted on 256^3), so these stretches have no re-sorts.
 
 // Event arguments and model of the lattice, copied to shared memory once per
 // launch: after a barrier a load of them from global memory would go to L2.
