@@ -251,12 +251,14 @@ void refresh_estimates(psc_lattice* L)
                 return;
             }
         }
-        for (int s = 0; s < L->nsp; ++s) {
-            L->est[s] = L->counts_h[s];
-            L->grid_class[s] = grid_class_for(L, s, L->est[s], L->grid_class[s]);
+        if (L->counts_g >= L->next_id_g) {           // (a batch may have brought newer ones)
+            for (int s = 0; s < L->nsp; ++s) {
+                L->est[s] = L->counts_h[s];
+                L->grid_class[s] = grid_class_for(L, s, L->est[s], L->grid_class[s]);
+            }
+            L->next_id_known = (uint32_t)L->counts_h[offsetof(Scalars, next_id) / 4];
+            L->next_id_g = L->counts_g;
         }
-        L->next_id_known = (uint32_t)L->counts_h[offsetof(Scalars, next_id) / 4];
-        L->next_id_g = L->counts_g;
         L->counts_pending = false;
     }
     if (L->g - L->counts_g < 64u) return;

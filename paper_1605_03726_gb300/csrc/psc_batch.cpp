@@ -52,7 +52,8 @@ struct psc_batch {
     int32_t* counts_h = nullptr;          // pinned copy, for the next stretch's groups
     cudaEvent_t counts_ev = nullptr;
     bool counts_pending = false;
-    std::vector<std::pair<psc_lattice*, uint32_t>> counts_of;  // whose lengths counts_h holds, after which event
+    std::vector<std::pair<psc_lattice*, uint32_t>> counts_of;  // whose lengths counts_h holds (null: no member
+                                                               // any more), after which event
 };
 
 namespace {
@@ -252,12 +253,12 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         B->counts_pending = false;
         for (size_t r = 0; r < B->counts_of.size(); ++r) {
             psc_lattice* L = B->counts_of[r].first;
-            bool member = false;
-            for (int i = 0; i < kBatchMax && !member; ++i) member = B->slot[i].L == L;
+            // (null: it left the batch; it may also have run on by itself and know better)
+            if (!L || B->counts_of[r].second < L->next_id_g) continue;
             const int32_t* h = B->counts_h + r * kSmallCounts;
-            for (int s = 0; member && s < L->nsp; ++s)
+            for (int s = 0; s < L->nsp; ++s)
                 if (h[s] >= 0) L->est[s] = h[s];
-            if (member && h[kMaxSpecies] > 0) {
+            if (h[kMaxSpecies] > 0) {
                 L->next_id_known = h[kMaxSpecies];
                 L->next_id_g = B->counts_of[r].second;
             }
@@ -436,6 +437,10 @@ int psc_batch_remove(psc_batch* B, psc_lattice* L)
         if (B->slot[i].L == L) {
             B->slot[i].L = nullptr;
             B->size--;
+            // list lengths on their way are of the lattice as it was: it may be destroyed,
+            // and its address the next member's, before they are looked at
+            for (auto& c : B->counts_of)
+                if (c.first == L) c.first = nullptr;
             return PSC_OK;
         }
     }

@@ -1,0 +1,71 @@
+"""Members of a batch that come and go between stretches.
+
+The batch keeps the list lengths a stretch ended with for the next one.  They
+belong to the member as it was then: a lattice that left the batch (and ran on
+alone, or was destroyed, its address perhaps given to the next lattice) must
+not be judged by them.  With births a stale pair of next id and event index
+would put the member beyond the ids that stretches hold, and leave it in
+launches per event phase for good.
+"""
+import numpy as np
+import pytest
+
+import paper_1605_03726_gb300 as psc
+
+pytestmark = pytest.mark.gpu
+
+TAU = 6.666666666666667e-05             # hop interval at D = 1 um^2/s, r_v = 10 nm
+SHAPE = (24, 24, 24)
+
+
+def splitting(stream, seed):
+    """A splits into A + C, and takes C away again."""
+    L = psc.Lattice(*SHAPE, voxel_radius=1e-8, stream=stream)
+    L.set_options(claim_table=1, resort_period=-1)
+    a = L.add_species(1e-12, 60)
+    c = L.add_species(0.0, 0)
+    L.add_reaction([a], [a, c], 0.002 / TAU)
+    L.add_reaction([a, c], [a], 1e-19)
+    L.populate(seed)
+    return L
+
+
+def events_in_stretches(B, n):
+    before = B.launches()
+    B.run_events(n)
+    return B.launches() - before == 1                    # (per event phase: four or more an event)
+
+
+def test_member_that_ran_alone_meanwhile_goes_on_in_stretches():
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+    B = psc.Batch(stream=stream)
+    L, solo = splitting(stream, 3), splitting(None, 3)
+    B.add(L)
+    assert events_in_stretches(B, 2)
+    B.remove(L)
+    # 8192 births an event at most: enough events for 2^27 ids
+    L.run_events(17000)
+    B.add(L)
+    assert events_in_stretches(B, 2)                  # (takes up what the last stretch left)
+    assert events_in_stretches(B, 100)
+    solo.run_events(17104)
+    assert np.array_equal(L.grid(), solo.grid()) and np.array_equal(L.counts(), solo.counts())
+    B.close()
+
+
+def test_new_members_do_not_inherit_list_lengths():
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+    B = psc.Batch(stream=stream)
+    for r in range(6):                                   # addresses come back
+        L, solo = splitting(stream, r), splitting(None, r)
+        B.add(L)
+        assert events_in_stretches(B, 2), r
+        assert events_in_stretches(B, 300), r
+        solo.run_events(302)
+        assert np.array_equal(L.counts(), solo.counts()), r
+        B.remove(L)
+        L.close()
+        solo.close()
+    B.close()
