@@ -214,28 +214,34 @@ int stretch_buffers(psc_batch* B, psc_lattice* L)
     return PSC_OK;
 }
 
-// May L run in stretches?  extra: bytes of its buffers for that, at most `room`.
-bool member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra)
+// May L run in stretches (*yes)?  extra: bytes of its buffers for that, at most
+// `room`.  Without room on the device it runs in batched launches.
+int member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra, bool* yes)
 {
     *extra = 0;
+    *yes = false;
     if (L->opt.persistent <= 0 || L->opt.time_kernels > 0 || L->opt.subvolume > 0 || L->opt.barrier_phantom > 0)
-        return false;
+        return PSC_OK;
     stretch_buffers(B, L);
-    if (B->stretch_blocks <= 0) return false;
-    if (L->V > kCellVoxels) return false;
+    if (B->stretch_blocks <= 0) return PSC_OK;
+    if (L->V > kCellVoxels) return PSC_OK;
     for (int s = 0; s < L->nsp; ++s)
-        if (L->model_h.lists[s].cap > kCellVoxels) return false;
+        if (L->model_h.lists[s].cap > kCellVoxels) return PSC_OK;
     const int64_t lacks = small_lacks(L, true);
-    if (lacks > room) return false;
-    if (small_buffers(L, true) != PSC_OK) {
+    if (lacks > room) return PSC_OK;
+    const int sticky = L->sticky;         // an error it brings along stays
+    const int rc = small_buffers(L, true);
+    if (rc == PSC_E_NOMEM) {
         cudaGetLastError();
-        L->sticky = PSC_OK;               // no room on the device: batched launches
-        return false;
+        L->sticky = sticky;
+        return PSC_OK;
     }
+    if (rc) return rc;
     // a group's barrier goes on from whatever complete barriers left there
-    if (cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), B->stream) != cudaSuccess) return false;
+    if (cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), B->stream) != cudaSuccess) return PSC_E_CUDA;
     *extra = lacks;
-    return true;
+    *yes = true;
+    return PSC_OK;
 }
 
 // Up to n_events next events of every member that runs in stretches, up to
@@ -386,9 +392,11 @@ int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop, int64_t room, i
     DevGuard dg(B->device);
     int rc = upload_templates(B, free_slot, L);
     if (rc) return rc;
+    bool stretch = false;
+    if ((rc = member_stretches(B, L, room, extra, &stretch))) return rc;
     B->slot[free_slot].L = L;
     B->slot[free_slot].t_stop = t_stop;
-    B->slot[free_slot].stretch = member_stretches(B, L, room, extra);
+    B->slot[free_slot].stretch = stretch;
     B->size++;
     return PSC_OK;
 }

@@ -5,7 +5,8 @@ belong to the member as it was then: a lattice that left the batch (and ran on
 alone, or was destroyed, its address perhaps given to the next lattice) must
 not be judged by them.  With births a stale pair of next id and event index
 would put the member beyond the ids that stretches hold, and leave it in
-launches per event phase for good.
+launches per event phase for good.  A lattice that carries an error keeps it
+when it joins a batch.
 """
 import numpy as np
 import pytest
@@ -69,3 +70,33 @@ def test_new_members_do_not_inherit_list_lengths():
         L.close()
         solo.close()
     B.close()
+
+
+def test_error_stays_with_a_lattice_that_joins_a_batch():
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+    B = psc.Batch(stream=stream)
+    L = psc.Lattice(48, 48, 48, voxel_radius=1e-8, stream=stream)
+    L.set_options(claim_table=1, barrier_timeout_us=20000, barrier_phantom=1)
+    L.add_species(1e-12, 3000)
+    L.populate(17)
+    L.run_events(4)                                      # a barrier that awaits a block that is not there
+    with pytest.raises(psc.EngineError) as err:
+        L.synchronize()
+    assert err.value.rc == psc.E_TIMEOUT
+    L.set_options(barrier_phantom=-1)
+    g = L.event_index()
+    none = psc.ALLOC_FN(lambda nbytes, device, stream, ctx: None)
+    no_free = psc.FREE_FN(lambda ptr, device, stream, ctx: None)
+    assert psc.lib().psc_set_allocator(none, no_free, None) == psc.OK
+    try:
+        B.add(L)                                         # no room for the buffers of stretches
+    finally:
+        psc.use_cuda_malloc()
+    B.run_events(3)
+    assert L.event_index() == g
+    with pytest.raises(psc.EngineError) as err:
+        L.counts()
+    assert err.value.rc == psc.E_TIMEOUT
+    B.close()
+    L.close()
