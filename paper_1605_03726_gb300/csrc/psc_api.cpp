@@ -70,6 +70,7 @@ void* dev_alloc(psc_lattice* L, size_t bytes)
         if (g_alloc) p = g_alloc(bytes, L->device, L->stream, g_alloc_ctx);
         else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
     }
+    if (!p) cudaGetLastError();                      // reported by the caller; not the next launch's error
     if (p) L->allocs.push_back(p);
     return p;
 }
