@@ -387,7 +387,12 @@ double psc_p_ab(const psc_lattice *L, int32_t reaction);
 
 /* Bytes of device memory the lattice holds after psc_populate (or would hold,
    computed from its shape and model, before), including the tile kernel's
-   buffers once a stretch has run under it. */
+   buffers once a stretch has run under it, and those of the stretches of species
+   with reactions (psc_options.persistent; 4 bytes per voxel, and 8 bytes for each
+   of up to 1.2 million entries or six per molecule of the longest list where that
+   exceeds 16,384): with the lattice up to 2^22 voxels, else once one has run.
+   Without room for them events run in per-event launches, until options are set
+   again. */
 int psc_device_bytes(const psc_lattice *L, int64_t *bytes);
 
 /* Free the lattice and its device memory (waits for its queued work). */

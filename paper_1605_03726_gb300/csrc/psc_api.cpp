@@ -838,14 +838,14 @@ static int small_setup(psc_lattice* L)
     }
     std::vector<EventArgs> ev((size_t)L->nsp);
     for (int s = 0; s < L->nsp; ++s) ev[(size_t)s] = event_args(L, s);
-    EventArgs* d = (EventArgs*)dev_alloc(L, sizeof(EventArgs) * ev.size());
-    if (!d) return PSC_E_NOMEM;
+    if (!B.ev) B.ev = (EventArgs*)dev_alloc(L, sizeof(EventArgs) * ev.size());
+    if (!B.ev) return PSC_E_NOMEM;
     // (from pageable memory: the copy has left it when the call returns)
-    const int rc = cuda_fail(L, cudaMemcpyAsync(d, ev.data(), sizeof(EventArgs) * ev.size(), cudaMemcpyHostToDevice,
+    const int rc = cuda_fail(L, cudaMemcpyAsync(B.ev, ev.data(), sizeof(EventArgs) * ev.size(), cudaMemcpyHostToDevice,
                                                 L->stream));
     if (rc) return rc;
     L->h2d += sizeof(EventArgs) * ev.size();
-    B.ev = d;
+    B.ev_set = true;
     return PSC_OK;
 }
 
@@ -864,7 +864,7 @@ int64_t ids_bound(const psc_lattice* L)
 static bool small_fits(psc_lattice* L)
 {
     if (!L->claim || L->opt.persistent <= 0 || L->opt.barrier_phantom > 0 || L->V > kCellVoxels ||
-        ids_bound(L) > kCellIds)
+        ids_bound(L) > kCellIds || L->small.no_room)
         return false;
     for (int s = 0; s < L->nsp; ++s)
         if (L->model_h.lists[s].cap > kCellVoxels) return false;
@@ -913,7 +913,7 @@ int64_t small_lacks(const psc_lattice* L, bool scratch)
 int small_buffers(psc_lattice* L, bool scratch)
 {
     auto& B = L->small;
-    if (!B.ev) {
+    if (!B.ev_set) {
         const int rc = small_setup(L);
         if (rc) return rc;
     }
@@ -979,12 +979,21 @@ int grid_current(psc_lattice* L, bool leave)
 
 // A stretch of consecutive events, starting with species s at time t: one
 // launch.  *n = events queued.
+// Without room for its buffers *n is 0, and the events take the kernels that need
+// none, until options are set the next time.
 static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
 {
     auto& B = L->small;
     bool grid = false;                               // a stretch may take a grid
     for (int x = 0; x < L->nsp; ++x) grid = grid || (L->sp[x].D > 0.0 && L->est[x] > kSmallCluster);
+    *n = 0;
+    const int sticky = L->sticky;
     int rc = small_buffers(L, grid);
+    if (rc == PSC_E_NOMEM) {
+        L->sticky = sticky;
+        B.no_room = true;
+        return PSC_OK;
+    }
     if (rc) return rc;
     SmallArgs A{};
     if ((rc = small_args(L, &A))) return rc;
@@ -1536,6 +1545,14 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     } else if (!direct) {
         L->table_slots = (int64_t)1 << hb_max;
         for (int t = 0; t < 2; ++t) carve.add(&L->tables[t], ((size_t)1 << hb_max) * sizeof(uint64_t));
+    }
+    // reactions on lattices of up to 2^22 voxels run in stretches: their templates and
+    // cells come with the block (16 MB at most), so that events allocate nothing
+    bool general = false;
+    for (int s = 0; s < L->nsp; ++s) general = general || L->general[s];
+    if (general && stretch && direct && L->opt.persistent > 0 && L->V <= (1ll << 22)) {
+        carve.add(&L->small.ev, sizeof(EventArgs) * (size_t)L->nsp);
+        carve.add(&L->small.cell, nwords * 128);
     }
     for (int s = 0; s < L->nsp; ++s) {
         SpeciesList& l = M.lists[s];
@@ -2091,7 +2108,7 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             int rc = small_stretch(L, s, t, t_end, max_events - queued, &e);
             if (rc) return rc;
             queued += e;
-            continue;
+            if (e > 0) continue;
         }
         if (int rc = grid_current(L, true)) return rc;
         int threads = 0, blocks = 0;
@@ -2447,6 +2464,7 @@ int psc_set_options(psc_lattice* L, const psc_options* o)
     if (o->blocks_per_sm < 0) return PSC_E_ARG;
     graph_cache_clear(L);                            // captured launches follow the options
     std::memset(L->open_auto, 0, sizeof(L->open_auto));
+    L->small.no_room = false;
     if (o->resort_period) L->opt.resort_period = o->resort_period;
     if (o->block_threads) L->opt.block_threads = o->block_threads;
     if (o->blocks_per_sm) L->opt.blocks_per_sm = o->blocks_per_sm;

@@ -110,8 +110,10 @@ struct psc_lattice {
     // stretches of events in one launch (k_small_run): per-species argument
     // templates on the device, a cell per voxel and the scratch of closing lists up
     struct SmallBuffers {
-        EventArgs* ev = nullptr;       // written at the first stretch
-        uint32_t* cell = nullptr;      // the cells, allocated with the first stretch
+        EventArgs* ev = nullptr;       // allocated by the first stretch where the lattice's block has none
+        bool ev_set = false;           // written, by the first stretch
+        uint32_t* cell = nullptr;      // the cells, as ev
+        bool no_room = false;          // no memory for these: stretches are off until options are set
         int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
         int32_t scratch_n = 0;
         bool cells_hold = false;       // the cells agree with the lists
