@@ -148,7 +148,9 @@ typedef struct {
                                  run in stretches, see persistent; without
                                  reactions also from 262,144 molecules of a
                                  species on; the last two if the memory is
-                                 there)                                        */
+                                 there: 4 bytes per voxel, 4.3 GB at 1024^3,
+                                 where the tables of 10.7 million molecules
+                                 take 0.54; 2 leaves it to others)             */
     int32_t persistent;       /* 1 = run stretches of events in one launch
                                  (default): of a lattice without reactions and
                                  compartments whose molecules fit in shared

@@ -1352,10 +1352,10 @@ double psc_p_ab(const psc_lattice* L, int32_t r)
     return acceptance(R.k, L->sp[R.r[0]].D, L->sp[R.r[1]].D, L->rv);
 }
 
-int psc_populate(psc_lattice* L, uint64_t seed)
+// spare: claim words and list room that only stretches and the open kernels want
+// may be taken (claim words then instead of hash tables).
+static int populate(psc_lattice* L, uint64_t seed, bool spare)
 {
-    if (!L) return PSC_E_ARG;
-    if (L->populated) return PSC_E_ORDER;
     int64_t N = 0;
     for (int s = 0; s < L->nsp; ++s) N += L->sp[s].n0;
     if (N > L->V) return PSC_E_FULL;
@@ -1471,7 +1471,7 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     }
     // lists of products that are not sized for the lattice keep room for the
     // tombstones of k_small_run
-    L->list_slack = growth || !L->stretches ? 0 : std::min<int64_t>(2 * N, 262144);
+    L->list_slack = growth || !L->stretches || !spare ? 0 : std::min<int64_t>(2 * N, 262144);
     bool any_fo2 = false;
     for (int s = 0; s < L->nsp; ++s) any_fo2 = any_fo2 || L->fo2[s];
 
@@ -1499,21 +1499,19 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         L->hash_bits[s] = hb;
         if (L->sp[s].D > 0.0 && hb > hb_max) hb_max = hb;
     }
-    bool direct = L->V <= (1ll << 22) || hb_max == 0;
-    // (batches take the lattices that have claim words by these rules)
-    L->batchable = direct || 2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V;
-    if (L->opt.claim_table == 1) L->batchable = true;
-    if (L->opt.claim_table == 2 && hb_max > 0) L->batchable = false;
+    // (tables at least as large as a word per voxel buy nothing, and the
+    // per-event kernels empty the previous table in full every event: species
+    // that are reaction products get lists sized for the lattice)
+    bool direct = L->V <= (1ll << 22) || hb_max == 0 ||
+                  2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V;
+    if (L->opt.claim_table == 1) direct = true;
+    if (L->opt.claim_table == 2 && hb_max > 0) direct = spare = false;
+    L->batchable = direct;                           // batches take the lattices that have claim words by these rules
     // lattices without reactions take k_walk_run while their molecules fit in
     // shared memory
     L->walk_only = L->nrx == 0 && !comps && L->opt.subvolume <= 0;
     const bool walk = L->walk_only && walk_size(L) &&
                       walk_slots(L, (int64_t)kWalkThreads * L->sm_count) * kWalkThreads * 12 <= kWalkSmem;
-    if (walk && L->V <= kWalkVoxels) direct = true;
-    // tables at least as large as a word per voxel buy nothing, and the
-    // per-event kernels empty the previous table in full every event (species
-    // that are reaction products get lists sized for the lattice)
-    if (2.0 * 8.0 * (double)(1ll << hb_max) >= 4.0 * (double)L->V) direct = true;
     // larger ones with long lists and no reactions skip most claims: words need
     // no table to be emptied (and the tile kernel wants them too)
     bool open = false;
@@ -1527,16 +1525,14 @@ int psc_populate(psc_lattice* L, uint64_t seed)
     bool stretch = L->stretches && L->V <= kCellVoxels && L->opt.subvolume <= 0;
     for (int s = 0; s < L->nsp; ++s)
         stretch = stretch && (!(L->sp[s].D > 0.0) || L->sp[s].n0 <= (L->nrx > 0 ? kSmallList : kSmallWalk));
-    stretch = stretch || (L->stretches && walk);
-    if (L->opt.claim_table == 1) direct = true;
-    if (L->opt.claim_table == 2 && hb_max > 0) direct = open = stretch = false;
     // (k_walk_run orders them as the mirror's bits, whole bricks)
     const int64_t claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
-    if ((open || stretch) && !direct) {
+    L->spare_claims = !direct && spare &&
+                      (open || stretch || (walk && (L->stretches || L->V <= kWalkVoxels)));
+    if (L->spare_claims) {
         L->claim_n = claim_n;
         L->claim = (uint32_t*)dev_alloc(L, (size_t)claim_n * sizeof(uint32_t));
         direct = L->claim != nullptr;                // no room: tables
-        if (!direct) cudaGetLastError();
     }
     L->open_claims = open && direct;
     if (direct && !L->claim) {
@@ -1770,6 +1766,33 @@ int psc_populate(psc_lattice* L, uint64_t seed)
         for (int s = 0; s < L->nsp; ++s)
             if (L->est[s] > 0) L->grid_class[s] = grid_class_for(L, s, L->est[s], 0);
     return L->clamped ? PSC_W_PCLAMP : PSC_OK;
+}
+
+int psc_populate(psc_lattice* L, uint64_t seed)
+{
+    if (!L) return PSC_E_ARG;
+    if (L->populated) return PSC_E_ORDER;
+    const int sticky = L->sticky;
+    int rc = populate(L, seed, true);
+    // what was allocated goes back; where claim words were taken that the lattice can do
+    // without, it may fit with tables
+    for (bool again = true; rc < 0; again = false) {
+        const bool retry = again && rc == PSC_E_NOMEM && L->spare_claims;
+        DevGuard dg(L->device);
+        cudaStreamSynchronize(L->stream);
+        dev_free_all(L);
+        L->claim = nullptr;
+        L->claim_n = 0;
+        L->tables[0] = L->tables[1] = nullptr;
+        L->table_slots = 0;
+        L->small.ev = nullptr;
+        L->small.cell = nullptr;
+        L->subvol = {};
+        if (!retry) break;
+        L->sticky = sticky;
+        rc = populate(L, seed, false);
+    }
+    return rc;
 }
 
 }  // extern "C"

@@ -68,6 +68,7 @@ struct psc_lattice {
     std::vector<uint8_t> labels;       // compartment of every voxel (empty: all 0)
     uint32_t* claim = nullptr;         // per-voxel claim words (small lattices)
     int64_t claim_n = 0;               // their number
+    bool spare_claims = false;         // taken for speed only, or tried to: tables would do
     uint64_t* tables[2] = {nullptr, nullptr};   // claim hash tables (large lattices)
     uint32_t table_used[2] = {0, 0};   // slots written by the event that used it
     int64_t table_slots = 0;

@@ -1,9 +1,9 @@
 """Lattices where device memory is short.
 
-What only makes events faster (the cells of stretches) is given up where there
-is no room for it, and the lattice runs in the kernels that do without; results
-stay the same.  A failed
-allocation of one lattice is not taken for an error of the next.
+What only makes events faster (claim words in place of hash tables, the cells
+of stretches) is given up where there is no room for it, and the lattice runs in
+the kernels that do without; results stay the same.  A failed allocation of one
+lattice is not taken for an error of the next.
 """
 import numpy as np
 import pytest
@@ -90,6 +90,34 @@ def test_reactions_run_without_room_for_stretches(memory, n, cells):
     assert L.stats()["launches"] - before < 10
     same(state(L), expected[1])
     L.close()
+
+
+@pytest.mark.parametrize("shape,n", [((200, 200, 192), 100000), ((400, 300, 240), 270000)])
+def test_walkers_take_tables_without_room_for_claim_words(memory, shape, n):
+    def lattice(**options):
+        L = psc.Lattice(*shape, voxel_radius=1e-8)
+        L.set_options(**options)
+        models.diffusion_only(L, n)
+        L.populate(5)
+        return L
+
+    L = lattice(claim_table=2)
+    tables = memory.used()
+    L.close()
+    L = lattice()
+    words = memory.used()
+    L.run_events(40)
+    expected = state(L)
+    L.close()
+    assert words > tables + (8 << 20)
+    for cap in (words - 1, tables + (4 << 20)):          # a byte too little; room for tables only
+        memory.cap = cap
+        L = lattice()
+        assert L.device_bytes() < tables + (4 << 20)
+        memory.cap = 1 << 60                             # (the tile kernel's buffers)
+        L.run_events(40)
+        same(state(L), expected)
+        L.close()
 
 
 def test_failed_allocation_is_not_the_next_lattice_s_error():
