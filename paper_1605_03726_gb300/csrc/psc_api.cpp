@@ -863,7 +863,7 @@ int64_t ids_bound(const psc_lattice* L)
 // lattice.
 static bool small_fits(psc_lattice* L)
 {
-    if (!L->claim || L->opt.persistent <= 0 || L->opt.barrier_phantom > 0 || L->V > kCellVoxels ||
+    if (!L->claim || L->opt.persistent <= 0 || L->V > kCellVoxels ||
         ids_bound(L) > kCellIds || L->small.no_room)
         return false;
     for (int s = 0; s < L->nsp; ++s)
@@ -955,6 +955,7 @@ int small_args(psc_lattice* L, SmallArgs* A)
     A->scratch_n = B.scratch_n;
     A->barrier = L->barrier;
     A->barrier_timeout_ns = (uint64_t)L->opt.barrier_timeout_us * 1000ull;
+    A->barrier_phantom = (uint32_t)L->opt.barrier_phantom;
     A->nsp = L->nsp;
     A->collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
     A->general = B.general;
@@ -1012,7 +1013,8 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
     // blocks, or 128 threads in each, short lists got slower: 2621 walkers 3.9 us
     // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM, of
     // half the threads while they suffice
-    const bool cluster = longest <= kSmallCluster;
+    // (a cluster's hardware barrier knows no phantoms)
+    const bool cluster = longest <= kSmallCluster && A.barrier_phantom == 0;
     const int threads = !cluster && longest <= 65536 ? kSmallThreads / 2 : kSmallThreads;
     const int blocks = cluster ? B.cluster : B.grid;
     if (!cluster) rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream));
@@ -1169,6 +1171,13 @@ bool next_event(const psc_lattice* L, int* s_out, double* t_out)
     return best >= 0;
 }
 
+int note_errors(psc_lattice* L, int32_t err)
+{
+    if (err & kErrBarrierTimeout) L->sticky = PSC_E_TIMEOUT;
+    else if (err) L->sticky = PSC_E_CAPACITY;
+    return L->sticky;
+}
+
 int check_device(psc_lattice* L)
 {
     if (!L->populated) {
@@ -1182,10 +1191,7 @@ int check_device(psc_lattice* L)
     if (e != cudaSuccess) return cuda_fail(L, e);
     if (state != L->state) std::memcpy(L->state, state, kStateBytes);
     L->d2h += kStateBytes;
-    const int32_t err = L->state[offsetof(Scalars, err) / 4];
-    if (err & kErrBarrierTimeout) L->sticky = PSC_E_TIMEOUT;
-    else if (err) L->sticky = PSC_E_CAPACITY;
-    return L->sticky;
+    return note_errors(L, L->state[offsetof(Scalars, err) / 4]);
 }
 
 

@@ -220,8 +220,7 @@ int member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra,
 {
     *extra = 0;
     *yes = false;
-    if (L->opt.persistent <= 0 || L->opt.time_kernels > 0 || L->opt.subvolume > 0 || L->opt.barrier_phantom > 0)
-        return PSC_OK;
+    if (L->opt.persistent <= 0 || L->opt.time_kernels > 0 || L->opt.subvolume > 0) return PSC_OK;
     stretch_buffers(B, L);
     if (B->stretch_blocks <= 0) return PSC_OK;
     if (L->V > kCellVoxels) return PSC_OK;
@@ -262,6 +261,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
             // (null: it left the batch; it may also have run on by itself and know better)
             if (!L || B->counts_of[r].second < L->next_id_g) continue;
             const int32_t* h = B->counts_h + r * kSmallCounts;
+            if (note_errors(L, h[kMaxSpecies + 1])) continue;      // (a wait that ran out: no further events of it)
             for (int s = 0; s < L->nsp; ++s)
                 if (h[s] >= 0) L->est[s] = h[s];
             if (h[kMaxSpecies] > 0) {
@@ -327,8 +327,6 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
                             cudaMemcpyHostToDevice, B->stream) != cudaSuccess ||
             cudaMemcpyAsync(B->group_d, group.data(), sizeof(int2) * group.size(), cudaMemcpyHostToDevice, B->stream) !=
                 cudaSuccess ||
-            (l == 0 && cudaMemsetAsync(B->counts_d, 0xFF, sizeof(int32_t) * kSmallCounts * (size_t)total, B->stream) !=
-                           cudaSuccess) ||
             launch_small_batch(B->args_d, B->group_d, B->counts_d, (int)group.size(), births, B->stream) !=
                 cudaSuccess) {
             *rc_out = PSC_E_CUDA;

@@ -263,7 +263,7 @@ struct ReconcileArgs {
 // per-voxel claim words (k_small_run).
 constexpr int kSmallEvents = 512;          // events of one launch
 constexpr int kSmallThreads = 512;         // threads of a block
-constexpr int kSmallCounts = kMaxSpecies + 1;      // list lengths and next id, per lattice of a batch
+constexpr int kSmallCounts = kMaxSpecies + 2;      // list lengths, next id and error bits, per lattice of a batch
 // limits of a cell's fields
 constexpr int64_t kCellVoxels = 1ll << 26; // (list slots)
 constexpr int64_t kCellIds = (1ll << 27) - (1ll << 23);    // next id when a stretch starts; a stretch makes at
@@ -288,6 +288,7 @@ struct SmallArgs {
     int32_t scratch_n;
     BarrierState* barrier;
     uint64_t barrier_timeout_ns;
+    uint32_t barrier_phantom;
     uint32_t g;                // index of the first event
     int32_t n_events;
     int32_t nsp;

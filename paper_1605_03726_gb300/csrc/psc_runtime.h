@@ -221,6 +221,8 @@ EventArgs event_args(const psc_lattice* L, int s);
 ReconcileArgs reconcile_args(const psc_lattice* L, int x);
 bool next_event(const psc_lattice* L, int* s_out, double* t_out);
 int check_device(psc_lattice* L);
+// error bits of Scalars::err that a copy brought: the lattice keeps them from then on
+int note_errors(psc_lattice* L, int32_t err);
 // stretches of k_small_run (and of batches): buffers still lacking, their
 // allocation, the arguments but the events
 int64_t small_lacks(const psc_lattice* L, bool scratch);

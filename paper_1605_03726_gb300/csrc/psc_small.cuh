@@ -84,11 +84,11 @@ __device__ __forceinline__ bool small_barrier(const SmallArgs& A, const SmallBlo
         cluster_barrier();
         return true;
     }
-    if (MODE == kSmallInGroup && B.nblk == 1) {
+    if (MODE == kSmallInGroup && B.nblk == 1 && A.barrier_phantom == 0u) {
         __syncthreads();                                        // what a block wrote, the block sees
         return true;
     }
-    return block_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, 0u, B.blk, B.nblk);
+    return block_barrier(A.barrier, &A.sc->err, A.barrier_timeout_ns, A.barrier_phantom, B.blk, B.nblk);
 }
 
 // Cells, in the mirror's order (place = mirror word << 5 | bit).  Top bit set:
@@ -600,8 +600,9 @@ __device__ __forceinline__ bool small_event(const SmallArgs& A, const SmallBlock
     return small_barrier<MODE>(A, B);
 }
 
+// false: a wait ran out
 template <SmallMode MODE>
-__device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, const SmallBlocks& B)
+__device__ __forceinline__ bool small_run(const SmallArgs& A, SmallShared& S, const SmallBlocks& B)
 {
     // a list is dealt out warp by warp over the blocks, so that a short one
     // keeps every SM of the launch busy
@@ -624,7 +625,7 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
         S.n[threadIdx.x] = A.sc->counts[threadIdx.x];
     }
     __syncthreads();
-    if (!small_barrier<MODE>(A, B)) return;
+    if (!small_barrier<MODE>(A, B)) return false;
     const ModelDev& M = S.model;
     bool prev_fo2 = false, loaded = false;
     SmallMol m[kSmallCarry];
@@ -661,7 +662,7 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
             if (born) {
                 if (blk == 0) births_body(S.ev[S.seq[e - 1]], A.cell);
                 prev_fo2 = false;
-                if (!small_barrier<MODE>(A, B)) return;
+                if (!small_barrier<MODE>(A, B)) return false;
                 continue;
             }
             if (last) break;
@@ -671,27 +672,27 @@ __device__ __forceinline__ void small_run(const SmallArgs& A, SmallShared& S, co
                                 (int64_t)__reduce_add_sync(0xFFFFFFFFu, holes) + 2 * (int64_t)n >
                                     (int64_t)A.scratch_n);
             if (!tight) break;
-            if (!small_barrier<MODE>(A, B)) return;             // the counts are read
-            if (!small_close<MODE>(A, S, B, t0, stride)) return;
-            if (!small_barrier<MODE>(A, B)) return;
+            if (!small_barrier<MODE>(A, B)) return false;             // the counts are read
+            if (!small_close<MODE>(A, S, B, t0, stride)) return false;
+            if (!small_barrier<MODE>(A, B)) return false;
             if (t0 < kMaxSpecies) A.sc->hole_n[t0] = A.sc->surv_n[t0] = 0;
         }
         if (last) {
-            if (A.general) small_close<MODE>(A, S, B, t0, stride);
-            return;
+            return A.general ? small_close<MODE>(A, S, B, t0, stride) : true;
         }
         n = min(n, a.list.cap);
         if ((A.general >> s) & 1u) {
             // word g & 1 was last read an event ago
             if (t0 == 0) A.sc->touched[g & 1u] = 0u;
-            if (!small_event<true, MODE>(A, B, a, M, g, t0, stride, n, m, nullptr)) return;
+            if (!small_event<true, MODE>(A, B, a, M, g, t0, stride, n, m, nullptr)) return false;
         } else {
             const EventArgs* next = (A.general || e + 1 == A.n_events) ? nullptr : &S.ev[S.seq[e + 1]];
-            if (!small_event<false, MODE>(A, B, a, M, g, t0, stride, n, m, next)) return;
+            if (!small_event<false, MODE>(A, B, a, M, g, t0, stride, n, m, next)) return false;
             loaded = next != nullptr;
         }
         prev_fo2 = (A.fo2 >> s) & 1u;
     }
+    return true;
 }
 
 template <bool CLUSTER>
@@ -707,8 +708,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(const SmallArgs 
 // before: a launch per phase for all of them): 64 members of 96^3 with 5 % A and B
 // 171 / 31 -> 106 / 15; 64 of 160^3 with 2 % 446 / 155 -> 261 / 74, bound by
 // scattered DRAM accesses, as the members' cells are 1 GB.
-// counts: list lengths and next id afterwards, [lattice][kSmallCounts], for the
-// next launch's groups.
+// counts: list lengths (-1 where they are not known), next id and error bits
+// afterwards, [lattice][kSmallCounts], for the next launch's groups.
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArgs* args, const int2* group,
                                                                   int32_t* counts)
 {
@@ -718,10 +719,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArg
     small_copy(&A, args + mine.x, sizeof(SmallArgs));
     __syncthreads();
     const SmallBlocks B{(int)blockIdx.x - mine.y, A.blocks};
-    small_run<kSmallInGroup>(A, S, B);
+    const bool done = small_run<kSmallInGroup>(A, S, B);
     int32_t* out = counts + mine.x * kSmallCounts;
-    if (A.general && B.blk == 0 && (int)threadIdx.x < A.nsp) out[threadIdx.x] = S.n[threadIdx.x] - S.k[threadIdx.x];
-    if (B.blk == 0 && threadIdx.x == 0) out[kMaxSpecies] = (int32_t)min(A.sc->next_id, 0x7FFFFFFFu);
+    if (B.blk == 0 && (int)threadIdx.x < A.nsp)
+        out[threadIdx.x] = done && A.general ? S.n[threadIdx.x] - S.k[threadIdx.x] : -1;
+    if (B.blk == 0 && threadIdx.x == 0) {
+        out[kMaxSpecies] = (int32_t)min(A.sc->next_id, 0x7FFFFFFFu);
+        out[kMaxSpecies + 1] = __ldcg(&A.sc->err);
+    }
 }
 
 int small_batch_blocks(int sm_count)
