@@ -160,8 +160,10 @@ typedef struct {
                                  to 2^26 voxels with a claim word per voxel, its
                                  species in scheduler order, while no mobile
                                  species has more than 2^22 molecules (without
-                                 reactions 131,072); of a species without
-                                 reactions otherwise;
+                                 reactions 131,072), and no 2^18 walkers among
+                                 species with reactions have much the most
+                                 events; of a species without reactions
+                                 otherwise;
                                  -1 = claim and commit launches per event       */
     int32_t slot_map;         /* home slot of a claim in the hash table:
                                  1 = hashed voxel index (default), 2 = Morton

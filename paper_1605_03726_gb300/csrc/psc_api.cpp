@@ -855,9 +855,22 @@ int64_t ids_bound(const psc_lattice* L)
     return L->next_id_known + (L->births_cap > 1 ? (int64_t)(L->g - L->next_id_g) * L->births_cap : 0);
 }
 
+// Do the events of walkers s among species with reactions, whose diffusion
+// coefficients add up to `others`, come in runs too long for k_small_run?
+static bool small_run_long(const psc_lattice* L, int s, double others)
+{
+    const double n = (double)L->est[s];
+    int threads, blocks;
+    if (n < (double)kSmallRunList) return false;
+    const double run = L->V > kWalkVoxels ? kSmallRunLarge / n
+                                          : run_width(L, s, &threads, &blocks) > 0 ? kSmallRun / n : kSmallRunDense;
+    return L->sp[s].D > std::max(run, kSmallRunLeast) * others;
+}
+
 // Do the lattice's events run in stretches of k_small_run?  Every mobile
 // species' list holds at most kSmallList molecules, in lattices without
-// reactions kSmallWalk (by the estimates: a list that has grown past it in the
+// reactions kSmallWalk, and no long list of walkers among species with reactions
+// has its events in long runs (by the estimates: a list that has grown past it in the
 // meantime only takes longer).  All of them or none: the other kernels want
 // mirrors and codes, which these stretches bring up to date by a pass over the
 // lattice.
@@ -871,9 +884,12 @@ static bool small_fits(psc_lattice* L)
     if (!L->shapes_known) device_shapes(L);
     if (L->small.cluster <= 0 || L->small.grid <= 0) return false;
     const int64_t most = L->nrx > 0 ? kSmallList : kSmallWalk;
+    double rate = 0.0;                               // of all species' events
+    for (int s = 0; s < L->nsp; ++s) rate += L->sp[s].D;
     for (int s = 0; s < L->nsp; ++s) {
         if (!(L->sp[s].D > 0.0)) continue;
         if (L->est[s] > most) return false;
+        if (!L->general[s] && small_run_long(L, s, rate - L->sp[s].D)) return false;
         // kernel timing keeps the phases of a reaction event apart; without the background
         // copies of the list lengths nothing is known of them
         if (L->general[s] && (L->opt.time_kernels > 0 || !L->counts_h)) return false;

@@ -274,6 +274,22 @@ constexpr int64_t kCellIds = (1ll << 27) - (1ll << 23);    // next id when a str
 // (128^3: 63,000 walkers 6.0 us per event against 10.8, 210,000 14.4 against 13.0).
 constexpr int64_t kSmallList = 1 << 22;
 constexpr int64_t kSmallWalk = 131072;
+// Walkers among species with reactions: the tile and molecule-list kernels take
+// fewer accesses for a walker, but start anew after every event of another species.
+// So long lists of walkers leave these stretches to them, with all events of the
+// lattice, where a run (walkers' events for one of all other species) is longer
+// than kSmallRun / molecules; than kSmallRunLarge / molecules where the cells do not
+// fit in the L2 cache; than kSmallRunDense where they do and the list is too long
+// for the molecule-list kernel; and in no case for runs of kSmallRunLeast.  us per
+// event, those kernels / stretches, with a pair of 2000 molecules each that react, at
+// runs of 0.5, 4 and 50 events: 270,000 walkers on 256^3 35.0 / 9.4, 19.8 / 13.8,
+// 14.1 / 15.6; 1.0M on 256^3 45.0 / 19.0, 37.9 / 36.6, 34.9 / 43.4; 2.5M on 256^3
+// 81.7 / 36.8, 87.9 / 78.8, 90.4 / 94.9; 500,000 on 128^3 19.9 / 12.1, 19.8 / 20.4,
+// 19.8 / 23.6; 1.0M on 400^3 48.3 / 30.1, 34.7 / 62.7, 29.6 / 75.4; 2.5M on 400^3
+// 81.0 / 70.8, 77.5 / 160, 76.9 / 195.
+// 131,072 walkers are faster in stretches at any run (400^3 at 50 events 12.4 / 9.8).
+constexpr int64_t kSmallRunList = 1 << 18;
+constexpr double kSmallRun = 1.5e6, kSmallRunLarge = 1e6, kSmallRunDense = 3.0, kSmallRunLeast = 0.6;
 // The longest list that runs in one cluster of 16 blocks: A + B -> C of 2000
 // molecules each takes 4.2 us per event there and 6.3 in a grid, of 12,000 6.4 and
 // 6.7, of 24,000 10.3 and 6.8.

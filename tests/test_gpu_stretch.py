@@ -144,3 +144,27 @@ def test_members_in_stretches_and_in_launches_together():
                 a, b = m.coords(s), solo.coords(s)
                 assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     B.close()
+
+
+@pytest.mark.parametrize("D,stretches", [(1e-12, True), (1e-11, False)])
+def test_long_runs_of_walkers_leave_stretches(D, stretches):
+    # many walkers among rare reactions: one of their events for two of the reacting
+    # species', or a hundred in a row (the tile and molecule-list kernels take those)
+    def lattice(**options):
+        L = psc.Lattice(96, 92, 100, voxel_radius=1e-8)
+        L.set_options(resort_period=-1, **options)
+        models.reaction_diffusion_ab(L, 500, 500, D=1e-12 if stretches else 5e-14)
+        L.add_species(D, 270000)
+        L.populate(8)
+        return L
+
+    a, b = lattice(), lattice(persistent=-1)
+    for n in (3, 230):
+        before = a.stats()["launches"]
+        a.run_events(n)
+        launches = a.stats()["launches"] - before
+        b.run_events(n)
+        assert np.array_equal(a.grid(), b.grid())
+        for s in range(4):
+            assert np.array_equal(a.unwrapped(s)[0], b.unwrapped(s)[0])
+    assert (launches <= 3) == stretches
