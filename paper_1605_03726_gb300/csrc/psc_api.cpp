@@ -406,6 +406,17 @@ ReconcileArgs reconcile_args(const psc_lattice* L, int x)
     return r;
 }
 
+// Do claim and commit launches of species s look for hops that need no claim
+// (psc_open.cuh)?  Long lists of species without reactions, on lattices whose
+// claim words do not fit in the L2 cache and that are not crowded.
+static bool open_pays(const psc_lattice* L, int s)
+{
+    if (L->general[s] || L->est[s] < kOpenList || L->V <= kWalkVoxels) return false;
+    int64_t molecules = 0;
+    for (int x = 0; x < L->nsp; ++x) molecules += L->est[x];
+    return (double)molecules <= kOpenOccupied * (double)L->V;
+}
+
 int enqueue_event(psc_lattice* L, int s)
 {
     const EventArgs a = event_args(L, s);
@@ -425,7 +436,7 @@ int enqueue_event(psc_lattice* L, int s)
         launch_event_one(a1, L->stream);
         span_close(L, sp, kSpanClaim);
         L->launches += 1;
-    } else if (!L->general[s] && L->est[s] >= kOpenList) {
+    } else if (open_pays(L, s)) {
         launch_open_claim(a, L->est[s], L->sm_count, L->stream);
         span_close(L, sp, kSpanClaim);
         sp = span_open(L);

@@ -370,6 +370,13 @@ void launch_commit(const EventArgs& a, bool general, int blocks, int threads, cu
 void launch_open_claim(const EventArgs& a, int64_t n, int sm_count, cudaStream_t st);
 void launch_open_commit(const EventArgs& a, int64_t n, int sm_count, cudaStream_t st);
 constexpr int64_t kOpenList = 1 << 18;      // shortest list they take
+// They take lattices of more than kWalkVoxels voxels up to this share of occupied ones.
+// us per event, plain claims / these, both in claim words: 320^3 at 5 / 10 / 20 / 30 / 50 %
+// 69.8 / 54.1, 130 / 110, 221 / 207, 286 / 284, 346 / 416; 512^3 at 5 / 30 / 50 % 338 / 219,
+// 1213 / 1117, 1457 / 1691.  Where the words fit in the L2 cache a claim costs less than
+// the test: 256^3 at 2 / 5 / 10 / 30 % 16.4 / 18.7, 29.2 / 32.6, 50.6 / 57.5, 134 / 151,
+// 160^3 at 10 / 30 % 17.4 / 22.3, 37.3 / 47.2.
+constexpr double kOpenOccupied = 0.3;
 // Where the lean tile kernel can run, it does up to here: 2.5M walkers on 512^3
 // 70.7 us per event against 73.0, 2.7M 79.9 against 76.8, 3.4M 118 against 101.
 // (The general tile kernel never: 1.4M on a ragged lattice 102 against 45.)

@@ -1,5 +1,6 @@
 // psc_open.cuh -- claim and commit launches of one event of a species without
-// reactions on a sparse lattice.  Part of psc_kernels.cu's translation unit.
+// reactions on a large, sparse lattice (kOpenList, kWalkVoxels, kOpenOccupied).  Part
+// of psc_kernels.cu's translation unit.
 //
 // What bounds them: scattered accesses, to DRAM where the claim words (or
 // tables) of the lattice do not fit in the L2 cache.  A molecule whose target is
