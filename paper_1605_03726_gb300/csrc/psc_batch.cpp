@@ -46,12 +46,14 @@ struct psc_batch {
     // stretches of the members' events, one launch for many members
     int stretch_blocks = -1;              // most blocks of a launch (-1: not asked, 0: no stretches)
     bool use_stretches = true;
-    SmallArgs* args_d = nullptr;          // [kBatchMax], device: one for each member that takes part
-    int2* group_d = nullptr;              // [stretch_blocks]
+    SmallArgs* args_d = nullptr;          // [kBatchMax], device: a member's, but for its events
+    std::vector<SmallArgs> args_h;        // as last copied there
+    char* upload_d = nullptr;             // stretches, blocks' groups and events of a call
     int32_t* counts_d = nullptr;          // [kBatchMax][kSmallCounts] list lengths after a stretch
     int32_t* counts_h = nullptr;          // pinned copy, for the next stretch's groups
     cudaEvent_t counts_ev = nullptr;
     bool counts_pending = false;
+    int64_t counts_age = INT64_MAX / 2;   // events of a call since the last copy was queued
     std::vector<std::pair<psc_lattice*, uint32_t>> counts_of;  // whose lengths counts_h holds (null: no member
                                                                // any more), after which event
 };
@@ -199,12 +201,19 @@ int batch_event(psc_batch* B, double t_cap, bool all, int* rc_out)
 // stretches: every member's events in a group of blocks of its own, at its own
 // pace, one launch for as many members as there are blocks on the device
 // ---------------------------------------------------------------------------
+// of a call that advances kBatchMax members by kSmallEvents events, in launches of at
+// most `blocks` blocks, at least one for each member (the last launch may be short)
+size_t upload_bytes(int blocks)
+{
+    return kBatchMax * (sizeof(SmallStretch) + kSmallEvents + sizeof(int32_t)) + (size_t)blocks * sizeof(int32_t);
+}
+
 int stretch_buffers(psc_batch* B, psc_lattice* L)
 {
     if (B->stretch_blocks < 0) B->stretch_blocks = small_batch_blocks(L->sm_count);
     if (B->stretch_blocks == 0 || B->args_d) return PSC_OK;
     if (cudaMalloc(&B->args_d, sizeof(SmallArgs) * kBatchMax) != cudaSuccess ||
-        cudaMalloc(&B->group_d, sizeof(int2) * (size_t)B->stretch_blocks) != cudaSuccess ||
+        cudaMalloc(&B->upload_d, upload_bytes(B->stretch_blocks)) != cudaSuccess ||
         cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
@@ -243,14 +252,23 @@ int member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra,
     return PSC_OK;
 }
 
+// A copy of the members' list lengths every so many events, and the age at
+// which the host waits for one.  (Waited for by every call, with two copies up
+// and a memset in every launch, run_events(1) took 52 us of 64 A + B -> C members on 48^3
+// and 133 of 300 on 32^3; now 27 and 40; in launches
+// per event phase 38 and 55.)
+constexpr int64_t kCountsEvery = 64, kCountsWait = 256;
+
 // Up to n_events next events of every member that runs in stretches, up to
 // its t_stop and t_cap; the number of members that had any.
 int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
 {
     *rc_out = PSC_OK;
     if (!B->use_stretches || B->stretch_blocks <= 0) return 0;
-    // the list lengths after the last stretch: groups follow them
-    if (B->counts_pending) {
+    // list lengths after an earlier stretch: groups follow them.  They come in the
+    // background, and once they are kCountsWait events old the host waits for them
+    // (the device still has as many queued)
+    if (B->counts_pending && (B->counts_age >= kCountsWait || cudaEventQuery(B->counts_ev) == cudaSuccess)) {
         if (cudaEventSynchronize(B->counts_ev) != cudaSuccess) {
             *rc_out = PSC_E_CUDA;
             return 1;
@@ -270,10 +288,12 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
             }
         }
     }
-    std::vector<SmallArgs> args;
+    std::vector<SmallStretch> stretch;
+    std::vector<uint8_t> seq;
     std::vector<double> work;             // molecules per event
-    B->counts_of.clear();
+    std::vector<std::pair<psc_lattice*, uint32_t>> of;
     bool births = false;
+    B->args_h.resize(kBatchMax);
     for (int i = 0; i < kBatchMax; ++i) {
         psc_lattice* L = B->slot[i].L;
         if (!L || L->sticky || !B->slot[i].stretch) continue;
@@ -287,27 +307,41 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         if ((*rc_out = claims_free(L))) return 1;
         SmallArgs A{};
         if ((*rc_out = small_args(L, &A))) return 1;
-        A.g = L->g;
+        constexpr size_t fixed = offsetof(SmallArgs, seq);
+        if (std::memcmp(&A, &B->args_h[(size_t)i], fixed) != 0) {
+            if (cudaMemcpyAsync(B->args_d + i, &A, fixed, cudaMemcpyHostToDevice, B->stream) != cudaSuccess) {
+                *rc_out = PSC_E_CUDA;
+                return 1;
+            }
+            std::memcpy(&B->args_h[(size_t)i], &A, fixed);
+        }
+        SmallStretch x{};
+        x.slot = i;
+        x.g = L->g;
+        x.seq = (uint32_t)seq.size();
         const int64_t limit = std::min<int64_t>(std::min<int64_t>(n_events, kSmallEvents), (int64_t)UINT32_MAX - L->g);
         double molecules = 0.0;
         do {
-            A.seq[A.n_events++] = (uint8_t)s;
+            seq.push_back((uint8_t)s);
+            x.n_events++;
             molecules += (double)L->est[s];
             L->sp[s].done++;
             L->g++;
             L->clock = t;
-        } while (A.n_events < limit && next_event(L, &s, &t) && t <= B->slot[i].t_stop && t <= t_cap);
+        } while (x.n_events < limit && next_event(L, &s, &t) && t <= B->slot[i].t_stop && t <= t_cap);
         births = births || A.fo2 != 0u;
-        L->events += (uint64_t)A.n_events;
+        L->events += (uint64_t)x.n_events;
         L->launches += 1;
-        work.push_back(molecules / A.n_events);
-        args.push_back(A);
-        B->counts_of.emplace_back(L, L->g);
+        work.push_back(molecules / x.n_events);
+        stretch.push_back(x);
+        of.emplace_back(L, L->g);
     }
-    if (args.empty()) return 0;
-    const int total = (int)args.size();
+    if (stretch.empty()) return 0;
+    B->counts_age += n_events;
+    const int total = (int)stretch.size();
     const int launches = (total + B->stretch_blocks - 1) / B->stretch_blocks;
-    std::vector<int2> group;
+    std::vector<int32_t> group;           // of all launches' blocks
+    std::vector<int> first;               // block of each launch
     for (int l = 0; l < launches; ++l) {
         const int lo = (int)((int64_t)total * l / launches), hi = (int)((int64_t)total * (l + 1) / launches);
         // blocks by work; an event takes about as long with no molecules as
@@ -315,31 +349,46 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         double sum = 0.0;
         for (int r = lo; r < hi; ++r) sum += work[(size_t)r] + 600.0;
         const int spare = B->stretch_blocks - (hi - lo);
-        group.clear();
+        first.push_back((int)group.size());
         for (int r = lo; r < hi; ++r) {
             const int more = (int)(spare * (work[(size_t)r] + 600.0) / sum);
             const int most = (int)(work[(size_t)r] / kSmallThreads);           // with it, a molecule per thread
-            const int blocks = 1 + std::min(more, most);
-            args[(size_t)r].blocks = blocks;
-            group.insert(group.end(), (size_t)blocks, make_int2(r, (int)group.size()));
+            stretch[(size_t)r].blocks = 1 + std::min(more, most);
+            stretch[(size_t)r].block0 = (int)group.size() - first.back();
+            group.insert(group.end(), (size_t)stretch[(size_t)r].blocks, r);
         }
-        if (cudaMemcpyAsync(B->args_d + lo, args.data() + lo, sizeof(SmallArgs) * (size_t)(hi - lo),
-                            cudaMemcpyHostToDevice, B->stream) != cudaSuccess ||
-            cudaMemcpyAsync(B->group_d, group.data(), sizeof(int2) * group.size(), cudaMemcpyHostToDevice, B->stream) !=
-                cudaSuccess ||
-            launch_small_batch(B->args_d, B->group_d, B->counts_d, (int)group.size(), births, B->stream) !=
-                cudaSuccess) {
+    }
+    first.push_back((int)group.size());
+    // one copy up: stretches, groups, events
+    const size_t at_group = sizeof(SmallStretch) * (size_t)total, at_seq = at_group + sizeof(int32_t) * group.size();
+    std::vector<char> up(at_seq + seq.size());
+    std::memcpy(up.data(), stretch.data(), at_group);
+    std::memcpy(up.data() + at_group, group.data(), at_seq - at_group);
+    std::memcpy(up.data() + at_seq, seq.data(), seq.size());
+    if (cudaMemcpyAsync(B->upload_d, up.data(), up.size(), cudaMemcpyHostToDevice, B->stream) != cudaSuccess) {
+        *rc_out = PSC_E_CUDA;
+        return total;
+    }
+    for (int l = 0; l < launches; ++l) {
+        if (launch_small_batch(B->args_d, (const SmallStretch*)B->upload_d,
+                               (const int32_t*)(B->upload_d + at_group) + first[(size_t)l],
+                               (const uint8_t*)B->upload_d + at_seq, B->counts_d,
+                               first[(size_t)l + 1] - first[(size_t)l], births, B->stream) != cudaSuccess) {
             *rc_out = PSC_E_CUDA;
             return total;
         }
         B->launches += 1;
     }
+    if (B->counts_pending || B->counts_age < kCountsEvery) return total;
+    B->counts_of.swap(of);
     if (cudaMemcpyAsync(B->counts_h, B->counts_d, sizeof(int32_t) * kSmallCounts * (size_t)total,
                         cudaMemcpyDeviceToHost, B->stream) != cudaSuccess ||
-        cudaEventRecord(B->counts_ev, B->stream) != cudaSuccess)
+        cudaEventRecord(B->counts_ev, B->stream) != cudaSuccess) {
         *rc_out = PSC_E_CUDA;
-    else
+    } else {
         B->counts_pending = true;
+        B->counts_age = 0;
+    }
     return total;
 }
 
@@ -602,7 +651,7 @@ void psc_batch_destroy(psc_batch* B)
         cudaFree(B->tmpl_ev);
         cudaFree(B->tmpl_rc);
         cudaFree(B->args_d);
-        cudaFree(B->group_d);
+        cudaFree(B->upload_d);
         cudaFree(B->counts_d);
         if (B->counts_h) cudaFreeHost(B->counts_h);
         if (B->counts_ev) cudaEventDestroy(B->counts_ev);

@@ -309,11 +309,20 @@ struct SmallArgs {
     int32_t n_events;
     int32_t nsp;
     int32_t collect_stats;
-    int32_t blocks;            // blocks of the lattice's group (batched launches)
     uint32_t general;          // bit s: species s has reactions
     uint32_t fo2;              // bit s: a first-order reaction of s has two products
     uint32_t products[kMaxSpecies];        // bit y: an event of s may append to list y
-    uint8_t seq[kSmallEvents]; // species of each event
+    uint8_t seq[kSmallEvents]; // species of each event (batched launches: see SmallStretch)
+};
+
+// A lattice's stretch in a batched launch: what changes from one to the next (the
+// rest of its SmallArgs stays on the device)
+struct SmallStretch {
+    int32_t slot;              // of its SmallArgs
+    int32_t block0, blocks;    // its group of the launch's blocks
+    uint32_t g;
+    int32_t n_events;
+    uint32_t seq;              // where its events' species begin
 };
 
 // A stretch of events of a lattice without reactions (k_walk_run): every
@@ -480,11 +489,12 @@ void launch_cells_build(uint32_t* cell, const uint32_t* bits0, uint64_t words, i
                         const int32_t* counts, int nsp, const Geometry& geo, int blocks, cudaStream_t st);
 void launch_cells_grid(const uint32_t* cell, uint32_t* bits0, uint64_t words, int n_mirrors, uint16_t* occ,
                        const Geometry& geo, int blocks, cudaStream_t st);
-// stretches of many lattices in one launch of `blocks` blocks: args on the
-// device per lattice, group[block] = (lattice, first block of its group)
+// stretches of many lattices in one launch of `blocks` blocks: per block the
+// stretch it belongs to, species of all their events; stretch r leaves list
+// lengths in counts + r * kSmallCounts (all on the device)
 int small_batch_blocks(int sm_count);       // most blocks on the current device (0: not at all)
-cudaError_t launch_small_batch(const SmallArgs* args, const int2* group, int32_t* counts, int blocks, bool births,
-                               cudaStream_t st);
+cudaError_t launch_small_batch(const SmallArgs* args, const SmallStretch* stretch, const int32_t* group,
+                               const uint8_t* seq, int32_t* counts, int blocks, bool births, cudaStream_t st);
 cudaError_t launch_small(const SmallArgs& A, int blocks, int threads, bool cluster, cudaStream_t st);
 void launch_fill_u32(uint32_t* p, uint32_t value, size_t n, int blocks, cudaStream_t st);
 // molecule r (ids in species order, species s owning [offsets[s],

@@ -710,17 +710,26 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_run(const SmallArgs 
 // scattered DRAM accesses, as the members' cells are 1 GB.
 // counts: list lengths (-1 where they are not known), next id and error bits
 // afterwards, [lattice][kSmallCounts], for the next launch's groups.
-__global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArgs* args, const int2* group,
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArgs* args, const SmallStretch* stretch,
+                                                                  const int32_t* group, const uint8_t* seq,
                                                                   int32_t* counts)
 {
     __shared__ SmallShared S;
     __shared__ SmallArgs A;
-    const int2 mine = group[blockIdx.x];                        // lattice, first block of its group
-    small_copy(&A, args + mine.x, sizeof(SmallArgs));
+    static_assert(offsetof(SmallArgs, seq) % 4 == 0, "copied by words");
+    const int32_t r = group[blockIdx.x];
+    const SmallStretch mine = stretch[r];
+    small_copy(&A, args + mine.slot, offsetof(SmallArgs, seq));
+    for (int e = threadIdx.x; e < mine.n_events; e += blockDim.x) A.seq[e] = seq[mine.seq + e];
     __syncthreads();
-    const SmallBlocks B{(int)blockIdx.x - mine.y, A.blocks};
+    if (threadIdx.x == 0) {
+        A.g = mine.g;
+        A.n_events = mine.n_events;
+    }
+    __syncthreads();
+    const SmallBlocks B{(int)blockIdx.x - mine.block0, mine.blocks};
     const bool done = small_run<kSmallInGroup>(A, S, B);
-    int32_t* out = counts + mine.x * kSmallCounts;
+    int32_t* out = counts + r * kSmallCounts;
     if (B.blk == 0 && (int)threadIdx.x < A.nsp)
         out[threadIdx.x] = done && A.general ? S.n[threadIdx.x] - S.k[threadIdx.x] : -1;
     if (B.blk == 0 && threadIdx.x == 0) {
@@ -741,10 +750,10 @@ int small_batch_blocks(int sm_count)
     return per_sm * sm_count;
 }
 
-cudaError_t launch_small_batch(const SmallArgs* args, const int2* group, int32_t* counts, int blocks, bool births,
-                               cudaStream_t st)
+cudaError_t launch_small_batch(const SmallArgs* args, const SmallStretch* stretch, const int32_t* group,
+                               const uint8_t* seq, int32_t* counts, int blocks, bool births, cudaStream_t st)
 {
-    void* p[] = {&args, &group, &counts};
+    void* p[] = {&args, &stretch, &group, &seq, &counts};
     return cudaLaunchCooperativeKernel((const void*)k_small_batch, dim3(blocks), dim3(kSmallThreads), p,
                                        births ? (size_t)kBirthSortMax * sizeof(unsigned long long) : 0, st);
 }

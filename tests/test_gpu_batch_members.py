@@ -72,6 +72,34 @@ def test_new_members_do_not_inherit_list_lengths():
     B.close()
 
 
+def test_many_short_calls():
+    # list lengths come in the background, members join, leave and differ in their
+    # options between calls; more members than one launch has blocks for
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+    B = psc.Batch(stream=stream)
+    members = [(splitting(stream, r), r) for r in range(170)]
+    for L, r in members:
+        B.add(L)
+    late, _ = members[-1]
+    B.remove(late)
+    for call in range(150):
+        if call == 40:
+            B.add(late)
+        if call == 90:
+            members[0][0].set_options(collect_stats=1)
+        B.run_events(1 + call % 2)
+    for L, r in (members[0], members[85], members[-1]):
+        solo = splitting(None, r)
+        solo.run_events(L.event_index())
+        assert L.event_index() == (225 if L is not late else 165)
+        assert np.array_equal(L.grid(), solo.grid()) and np.array_equal(L.counts(), solo.counts())
+        solo.close()
+    attempts = members[0][0].stats()["attempts"]
+    assert attempts > 100 * 30 and members[1][0].stats()["attempts"] == 0
+    B.close()
+
+
 def test_error_stays_with_a_lattice_that_joins_a_batch():
     import torch
     stream = torch.cuda.Stream().cuda_stream
