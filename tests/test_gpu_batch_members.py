@@ -11,6 +11,7 @@ when it joins a batch.
 import numpy as np
 import pytest
 
+import models
 import paper_1605_03726_gb300 as psc
 
 pytestmark = pytest.mark.gpu
@@ -128,3 +129,36 @@ def test_error_stays_with_a_lattice_that_joins_a_batch():
     assert err.value.rc == psc.E_TIMEOUT
     B.close()
     L.close()
+
+
+def test_members_take_turns_where_their_cells_exceed_the_cache():
+    # 136 MB of cells, 1.9 million molecules: several launches for a call of many events,
+    # one for a call of few
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+
+    def member(r, stream):
+        L = psc.Lattice(100, 96 + 2 * (r % 3), 104, voxel_radius=1e-8, stream=stream)
+        L.set_options(claim_table=1, resort_period=-1)
+        if r % 2:
+            models.reaction_diffusion_ab(L, 56000, 56000)
+        else:
+            models.diffusion_only(L, 56000, D=1e-12)
+        L.populate(r)
+        return L
+
+    B = psc.Batch(stream=stream)
+    members = [member(r, stream) for r in range(34)]
+    for L in members:
+        B.add(L)
+    B.run_events(3)
+    assert B.launches() == 1
+    B.run_events(40)
+    assert B.launches() > 2
+    for r in (0, 1, 16, 17, 32, 33):
+        solo = member(r, None)
+        solo.run_events(43)
+        assert np.array_equal(members[r].grid(), solo.grid())
+        assert np.array_equal(members[r].unwrapped(0)[0], solo.unwrapped(0)[0])
+        solo.close()
+    B.close()
