@@ -211,19 +211,18 @@ size_t upload_bytes(int blocks)
 }
 
 // Launches of a call over `total` members with so many bytes of cells and molecules
-// an event: as few as there are blocks for.  For stretches of kSplitEvents events
-// and more whose cells do not fit in the L2 cache, members take turns instead, each
-// launch with the cells that fit, as long as it has kSplitMolecules molecules per
-// block and its groups fill the blocks to 0.85.  us for an event of every member,
-// launches per event phase / all members at once / in turns: 64 walkers' lattices of 160^3
-// at 2 % 455 / 517 / 250, of 96^3 at 30 % 834 / 973 / 641, 32 of 128^3 at 20 % 761 / 884 / 544, 64 of
-// A + B -> C on 160^3 at 2 % 401 / 236 / 173.
-constexpr int64_t kSplitEvents = 16;
+// an event: as few as there are blocks for.  Where the cells do not fit in the L2
+// cache together, members take turns instead, each launch with the cells that fit, as
+// long as it has kSplitMolecules molecules per block and its groups fill the blocks
+// to 0.85.  us for an event of every member, launches per event phase / all members
+// at once / in turns, calls of 64 events: 64 walkers' lattices of 160^3 at 2 % 455 / 517 /
+// 250, of 96^3 at 30 % 834 / 973 / 641, 32 of 128^3 at 20 % 761 / 884 / 544, 64 of A + B -> C on
+// 160^3 at 2 % 401 / 236 / 173; calls of one event: 470 / 560 / 470, 828 / 1029 / 708,
+// 759 / 941 / 613, 420 / 283 / 300.
 constexpr double kSplitMolecules = 4096.0, kSplitBytes = 4.0 * (double)kWalkVoxels;
-int stretch_launches(int total, int blocks, double bytes, double molecules, int64_t n_events)
+int stretch_launches(int total, int blocks, double bytes, double molecules)
 {
     const int least = (total + blocks - 1) / blocks;
-    if (n_events < kSplitEvents) return least;
     const int most = (int)std::min<double>({molecules / (kSplitMolecules * blocks), (double)total, (double)kUploadLaunches});
     for (int l = std::min((int)std::min(std::ceil(bytes / kSplitBytes), (double)kUploadLaunches), most); l <= most; ++l) {
         const int members = (total + std::max(l, 1) - 1) / std::max(l, 1);
@@ -368,7 +367,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         bytes += 128.0 * (double)of[(size_t)r].first->mirror_n;
         molecules += work[(size_t)r];
     }
-    const int launches = stretch_launches(total, B->stretch_blocks, bytes, molecules, n_events);
+    const int launches = stretch_launches(total, B->stretch_blocks, bytes, molecules);
     std::vector<int32_t> group;           // of all launches' blocks
     std::vector<int> first;               // block of each launch
     for (int l = 0; l < launches; ++l) {

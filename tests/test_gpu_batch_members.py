@@ -132,8 +132,7 @@ def test_error_stays_with_a_lattice_that_joins_a_batch():
 
 
 def test_members_take_turns_where_their_cells_exceed_the_cache():
-    # 136 MB of cells, 1.9 million molecules: several launches for a call of many events,
-    # one for a call of few
+    # 136 MB of cells, 1.9 million molecules
     import torch
     stream = torch.cuda.Stream().cuda_stream
 
@@ -151,10 +150,9 @@ def test_members_take_turns_where_their_cells_exceed_the_cache():
     members = [member(r, stream) for r in range(34)]
     for L in members:
         B.add(L)
-    B.run_events(3)
-    assert B.launches() == 1
-    B.run_events(40)
-    assert B.launches() > 2
+    B.run_events(1)
+    assert B.launches() > 1
+    B.run_events(42)
     for r in (0, 1, 16, 17, 32, 33):
         solo = member(r, None)
         solo.run_events(43)
