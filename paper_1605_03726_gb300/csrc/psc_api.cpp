@@ -1012,7 +1012,7 @@ int grid_current(psc_lattice* L, bool leave)
 static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t max_events, int64_t* n)
 {
     auto& B = L->small;
-    bool grid = false;                               // a stretch may take a grid
+    bool grid = false;                               // the stretch takes a grid
     for (int x = 0; x < L->nsp; ++x) grid = grid || (L->sp[x].D > 0.0 && L->est[x] > kSmallCluster);
     *n = 0;
     const int sticky = L->sticky;
@@ -1024,28 +1024,36 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
     }
     if (rc) return rc;
     SmallArgs A{};
-    if ((rc = small_args(L, &A))) return rc;
-    A.g = L->g;
     const int64_t limit = std::min<int64_t>(std::min<int64_t>(max_events, kSmallEvents),
                                             (int64_t)UINT32_MAX - L->g);
-    int64_t longest = 0;
+    A.g = L->g;
+    int64_t longest = 0, closed = 0;                 // lists of due species; lists that may be closed up
     do {
         A.seq[A.n_events++] = (uint8_t)s;
         longest = std::max(longest, L->est[s]);
+        for (int x : L->reconcile[s]) closed = std::max(closed, L->est[x]);
         L->sp[s].done++;
         L->g++;
         L->clock = t;
     } while (A.n_events < limit && next_event(L, &s, &t) && t <= t_end);
     // the shape: a cluster of 16 blocks up to kSmallCluster entries (with fewer
     // blocks, or 128 threads in each, short lists got slower: 2621 walkers 3.9 us
-    // per event, 4.4 on 8 blocks, 5.5 with 128 threads); then a block per SM, of
-    // half the threads while they suffice
+    // per event, 4.4 on 8 blocks, 5.5 with 128 threads), but for few events where
+    // closing up the lists would take longer than the cluster spares; then a block
+    // per SM, of half the threads while they suffice
     // (a cluster's hardware barrier knows no phantoms)
-    const bool cluster = longest <= kSmallCluster && A.barrier_phantom == 0;
-    const int threads = !cluster && longest <= 65536 ? kSmallThreads / 2 : kSmallThreads;
+    const double spare = (double)A.n_events * std::max(0.0, 1.0 - (double)longest / (double)kSmallCluster);
+    bool cluster = longest <= kSmallCluster && L->opt.barrier_phantom <= 0;
+    if (cluster && (double)closed > kSmallClosed * (1.0 + spare)) {
+        rc = small_buffers(L, true);
+        if (rc == PSC_E_NOMEM) L->sticky = sticky;   // (no scratch: in a cluster all the same)
+        else if (rc) return rc;
+        else cluster = false;
+    }
+    if ((rc = small_args(L, &A))) return rc;
+    const int threads = !cluster && longest <= 65536 && closed <= 1 << 20 ? kSmallThreads / 2 : kSmallThreads;
     const int blocks = cluster ? B.cluster : B.grid;
-    if (!cluster) rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream));
-    if (rc) return rc;
+    if (!cluster && (rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream)))) return rc;
     cudaEvent_t sp = span_open(L);
     rc = cuda_fail(L, launch_small(A, blocks, threads, cluster, L->stream));
     span_close(L, sp, kSpanRun, A.n_events);

@@ -313,7 +313,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
     }
     std::vector<SmallStretch> stretch;
     std::vector<uint8_t> seq;
-    std::vector<double> work;             // molecules per event
+    std::vector<double> work;             // molecules per event, entries looked through at the end among them
     std::vector<std::pair<psc_lattice*, uint32_t>> of;
     bool births = false;
     B->args_h.resize(kBatchMax);
@@ -343,11 +343,13 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         x.g = L->g;
         x.seq = (uint32_t)seq.size();
         const int64_t limit = std::min<int64_t>(std::min<int64_t>(n_events, kSmallEvents), (int64_t)UINT32_MAX - L->g);
-        double molecules = 0.0;
+        double molecules = 0.0, closed = 0.0;                    // closed: lists that may be closed up at the end
+        uint32_t may_close = 0;
         do {
             seq.push_back((uint8_t)s);
             x.n_events++;
             molecules += (double)L->est[s];
+            for (int q : L->reconcile[s]) may_close |= 1u << q;
             L->sp[s].done++;
             L->g++;
             L->clock = t;
@@ -355,7 +357,9 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         births = births || A.fo2 != 0u;
         L->events += (uint64_t)x.n_events;
         L->launches += 1;
-        work.push_back(molecules / x.n_events);
+        for (int q = 0; q < L->nsp; ++q)
+            if ((may_close >> q) & 1u) closed += (double)L->est[q];
+        work.push_back((molecules + 0.25 * closed) / x.n_events);
         stretch.push_back(x);
         of.emplace_back(L, L->g);
     }

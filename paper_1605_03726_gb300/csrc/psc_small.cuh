@@ -432,12 +432,19 @@ __device__ bool small_close(const SmallArgs& A, SmallShared& S, const SmallBlock
         if (S.k[x] <= 0) continue;
         const int32_t n = S.n[x], n2 = n - S.k[x];
         const int32_t* vox = M.lists[x].vox;
-        for (int idx = t0; idx - (t0 & 31) < n; idx += stride) {      // whole warps
-            const bool live = idx < n && __ldcg(vox + idx) >= 0;
-            const int h = warp_alloc(&A.sc->hole_n[x], idx < n2 && !live);
-            if (h >= 0) A.holes[base + h] = idx;
-            const int q = warp_alloc(&A.sc->surv_n[x], idx >= n2 && live);
-            if (q >= 0) A.surv[base + q] = idx;
+        constexpr int U = 4;                                    // entries in flight
+        for (int idx0 = t0; idx0 - (t0 & 31) < n; idx0 += U * stride) {      // whole warps
+            int32_t v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = idx0 + u * stride < n ? __ldcg(vox + idx0 + u * stride) : -1;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int idx = idx0 + u * stride;
+                const int h = warp_alloc(&A.sc->hole_n[x], idx < n2 && v[u] < 0);
+                if (h >= 0) A.holes[base + h] = idx;
+                const int q = warp_alloc(&A.sc->surv_n[x], idx >= n2 && v[u] >= 0);
+                if (q >= 0) A.surv[base + q] = idx;
+            }
         }
         base += S.k[x];
     }

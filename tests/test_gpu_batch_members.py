@@ -8,6 +8,8 @@ would put the member beyond the ids that stretches hold, and leave it in
 launches per event phase for good.  A lattice that carries an error keeps it
 when it joins a batch.
 """
+import gc
+
 import numpy as np
 import pytest
 
@@ -115,6 +117,7 @@ def test_error_stays_with_a_lattice_that_joins_a_batch():
     assert err.value.rc == psc.E_TIMEOUT
     L.set_options(barrier_phantom=-1)
     g = L.event_index()
+    gc.collect()                                         # no other lattice goes through these
     none = psc.ALLOC_FN(lambda nbytes, device, stream, ctx: None)
     no_free = psc.FREE_FN(lambda ptr, device, stream, ctx: None)
     assert psc.lib().psc_set_allocator(none, no_free, None) == psc.OK

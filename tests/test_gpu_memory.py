@@ -5,6 +5,8 @@ of stretches) is given up where there is no room for it, and the lattice runs in
 the kernels that do without; results stay the same.  A failed allocation of one
 lattice is not taken for an error of the next.
 """
+import gc
+
 import numpy as np
 import pytest
 
@@ -43,6 +45,7 @@ class Capped:
 
 @pytest.fixture
 def memory():
+    gc.collect()                                         # lattices of other tests go back where they came from
     m = Capped()
     assert psc.lib().psc_set_allocator(m.hooks[0], m.hooks[1], None) == psc.OK
     yield m

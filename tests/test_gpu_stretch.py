@@ -168,3 +168,20 @@ def test_long_runs_of_walkers_leave_stretches(D, stretches):
         for s in range(4):
             assert np.array_equal(a.unwrapped(s)[0], b.unwrapped(s)[0])
     assert (launches <= 3) == stretches
+
+
+@pytest.mark.parametrize("shape,n,partners", [((64, 60, 64), 500, 40000), ((36, 40, 44), 6000, 9000)])
+def test_short_calls_with_long_lists_to_close_up(shape, n, partners):
+    # calls of few events close the lists up in a grid, longer ones in a cluster
+    def recipe(L):
+        a = L.add_species(1e-12, n)
+        x = L.add_species(0.0, partners)
+        y = L.add_species(0.0, 0)
+        L.add_reaction([a, x], [a, y], 2e-20)
+        L.add_reaction([a, y], [x, a], 1e-20)
+
+    g, o = build_both(shape, recipe, 23)
+    for k in (1, 1, 2, 513, 3, 70):
+        g.run_events(k)
+        o.run_events(k)
+        assert_same(g, o, k)
