@@ -1053,7 +1053,12 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
     if ((rc = small_args(L, &A))) return rc;
     const int threads = !cluster && longest <= 65536 && closed <= 1 << 20 ? kSmallThreads / 2 : kSmallThreads;
     const int blocks = cluster ? B.cluster : B.grid;
-    if (!cluster && (rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream)))) return rc;
+    if (!cluster && !B.barrier_set) {
+        // (it goes on from whatever complete barriers left there; after one that ran out
+        // the lattice runs no more)
+        if ((rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream)))) return rc;
+        B.barrier_set = true;
+    }
     cudaEvent_t sp = span_open(L);
     rc = cuda_fail(L, launch_small(A, blocks, threads, cluster, L->stream));
     span_close(L, sp, kSpanRun, A.n_events);

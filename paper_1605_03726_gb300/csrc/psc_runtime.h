@@ -114,6 +114,7 @@ struct psc_lattice {
         EventArgs* ev = nullptr;       // allocated by the first stretch where the lattice's block has none
         bool ev_set = false;           // written, by the first stretch
         uint32_t* cell = nullptr;      // the cells, as ev
+        bool barrier_set = false;      // the barrier word was zeroed once
         bool no_room = false;          // no memory for these: stretches are off until options are set
         int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
         int32_t scratch_n = 0;

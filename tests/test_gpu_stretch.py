@@ -170,8 +170,9 @@ def test_long_runs_of_walkers_leave_stretches(D, stretches):
     assert (launches <= 3) == stretches
 
 
+@pytest.mark.parametrize("calls", [(1, 1, 2, 513, 3, 70), (513, 1, 2)])
 @pytest.mark.parametrize("shape,n,partners", [((64, 60, 64), 500, 40000), ((36, 40, 44), 6000, 9000)])
-def test_short_calls_with_long_lists_to_close_up(shape, n, partners):
+def test_short_calls_with_long_lists_to_close_up(shape, n, partners, calls):
     # calls of few events close the lists up in a grid, longer ones in a cluster
     def recipe(L):
         a = L.add_species(1e-12, n)
@@ -181,7 +182,7 @@ def test_short_calls_with_long_lists_to_close_up(shape, n, partners):
         L.add_reaction([a, y], [x, a], 1e-20)
 
     g, o = build_both(shape, recipe, 23)
-    for k in (1, 1, 2, 513, 3, 70):
+    for k in calls:
         g.run_events(k)
         o.run_events(k)
         assert_same(g, o, k)
