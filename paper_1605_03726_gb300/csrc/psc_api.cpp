@@ -1134,18 +1134,41 @@ static int walk_stretch(psc_lattice* L, int s, double t, double t_end, int64_t m
     A.key1 = (uint32_t)(L->seed >> 32);
     A.g = L->g;
     A.collect_stats = L->opt.collect_stats > 0 ? 1 : 0;
+    // claims stay below all ones: epochs 1 .. 2^(32 - id bits) - 2
+    int64_t largest = 0;
+    for (int x = 0; x < L->nsp; ++x) largest = std::max<int64_t>(largest, L->sp[x].D > 0.0 ? L->sp[x].n0 : 0);
+    while ((1ll << A.id_bits) < largest) ++A.id_bits;
+    const int64_t epochs = ((int64_t)1 << (32 - A.id_bits)) - 2;
+    const bool words = !L->claim_vacancy || (int64_t)L->walk_epoch >= epochs;      // they are made (anew)
+    const int64_t limit = std::min<int64_t>({max_events, kWalkEvents, (int64_t)UINT32_MAX - L->g,
+                                             epochs - (words ? 0 : (int64_t)L->walk_epoch)});
+    const uint64_t period = L->opt.resort_period > 0 ? (uint64_t)L->opt.resort_period : UINT64_MAX;
+    bool due = false;                                // a list's re-sort ends the stretch
+    bool used[kMaxSpecies] = {};                     // species with events in it: the others' molecules stay put
+    do {
+        A.seq[A.n_events++] = (uint8_t)s;
+        used[s] = true;
+        if (++L->since_resort[s] >= period && walk_sorts(L, s)) due = true;
+        L->sp[s].done++;
+        L->g++;
+        L->clock = t;
+    } while (!due && A.n_events < limit && next_event(L, &s, &t) && t <= t_end);
+    auto slots = [&](int64_t threads) {
+        int64_t m = 0;
+        for (int x = 0; x < L->nsp; ++x) m += used[x] ? (L->sp[x].n0 + threads - 1) / threads : 0;
+        return m;
+    };
     int64_t most = 0;
-    for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, L->sp[x].D > 0.0 ? L->sp[x].n0 : 0);
+    for (int x = 0; x < L->nsp; ++x) most = std::max<int64_t>(most, used[x] ? L->sp[x].n0 : 0);
     const bool cluster = most <= kWalkCluster && L->walk_cluster > 0 && A.barrier_phantom == 0 &&
-                         walk_slots(L, (int64_t)kWalkClusterThreads * L->walk_cluster) * kWalkClusterThreads * 12 <=
+                         slots((int64_t)kWalkClusterThreads * L->walk_cluster) * kWalkClusterThreads * 12 <=
                              kWalkClusterSmem - 1024;
     const int blocks = cluster ? L->walk_cluster : L->sm_count;
     const int64_t T = (int64_t)blocks * (cluster ? kWalkClusterThreads : kWalkThreads);
     int place[kMaxSpecies] = {};
     uint32_t id_lo = 0;                              // ids are the ones placement gave, species by species
-    while ((1ll << A.id_bits) < most) ++A.id_bits;
     for (int x = 0; x < L->nsp; id_lo += (uint32_t)L->sp[x].n0, ++x) {
-        if (!(L->sp[x].D > 0.0)) continue;
+        if (!used[x]) continue;
         A.id_lo[A.n_species] = id_lo;
         place[x] = A.n_species;
         A.n[A.n_species] = (int32_t)L->sp[x].n0;
@@ -1155,32 +1178,19 @@ static int walk_stretch(psc_lattice* L, int s, double t, double t_end, int64_t m
         A.slots += (int32_t)((L->sp[x].n0 + T - 1) / T);
         A.n_species++;
     }
+    for (int e = 0; e < A.n_events; ++e) A.seq[e] = (uint8_t)place[A.seq[e]];
     int rc = PSC_OK;
     for (int x = 0; x < L->nsp; ++x) {
-        if (!L->placed_order[x] || !walk_sorts(L, x)) continue;
+        if (!used[x] || !L->placed_order[x] || !walk_sorts(L, x)) continue;
         if ((rc = resort(L, x))) return rc;
     }
-    // claims stay below all ones: epochs 1 .. 2^(32 - id bits) - 2
-    const int64_t epochs = ((int64_t)1 << (32 - A.id_bits)) - 2;
-    const bool spent = (int64_t)L->walk_epoch >= epochs;
-    if (!L->claim_vacancy || spent) {
+    if (words) {
         launch_walk_words(L->claim, L->claim_vacancy ? nullptr : L->bits, L->mirror_n, L->sm_count * 8, L->stream);
         L->launches += 1;
         L->claim_vacancy = true;
         L->walk_epoch = 0;
     }
     A.epoch = L->walk_epoch + 1;
-    const int64_t limit = std::min<int64_t>({max_events, kWalkEvents, (int64_t)UINT32_MAX - L->g,
-                                             epochs - (int64_t)L->walk_epoch});
-    const uint64_t period = L->opt.resort_period > 0 ? (uint64_t)L->opt.resort_period : UINT64_MAX;
-    bool due = false;                                // a list's re-sort ends the stretch
-    do {
-        A.seq[A.n_events++] = (uint8_t)place[s];
-        if (++L->since_resort[s] >= period && walk_sorts(L, s)) due = true;
-        L->sp[s].done++;
-        L->g++;
-        L->clock = t;
-    } while (!due && A.n_events < limit && next_event(L, &s, &t) && t <= t_end);
     L->walk_epoch += (uint32_t)A.n_events;
     if (!cluster && (rc = cuda_fail(L, cudaMemsetAsync(L->barrier, 0, sizeof(BarrierState), L->stream)))) return rc;
     if ((rc = cuda_fail(L, launch_walk(A, blocks, cluster, L->stream)))) return rc;

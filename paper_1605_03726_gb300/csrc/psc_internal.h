@@ -369,7 +369,7 @@ struct WalkArgs {
     uint32_t g;                // index of the first event
     int32_t n_events;
     int32_t collect_stats;
-    int32_t n_species;         // mobile species with molecules
+    int32_t n_species;         // species with events in the stretch
     int32_t slots;             // molecules a thread holds at most, over all species
     int32_t n[kMaxSpecies];    // per species: molecules, first slot, index, list
     int32_t slot0[kMaxSpecies];

@@ -107,3 +107,14 @@ def test_claims_epochs_run_out():
         out.append(L.unwrapped(0))
         L.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+def test_stretches_of_some_of_the_species():
+    # only the species with events in a stretch take part in it: calls of one event,
+    # in a cluster or a grid by the species due, one without molecules among them
+    recipe = walkers((1e-12, 40000), (0.9e-12, 300), (1.7e-12, 0), (0.0, 9000), (0.3e-12, 17000))
+    g, o = build_both((64, 60, 62), recipe, 31, boundary=5)
+    for n in (1,) * 12 + (3, 40, 1):
+        g.run_events(n)
+        o.run_events(n)
+        assert_same(g, o, n)
