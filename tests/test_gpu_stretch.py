@@ -186,3 +186,18 @@ def test_short_calls_with_long_lists_to_close_up(shape, n, partners, calls):
         g.run_events(k)
         o.run_events(k)
         assert_same(g, o, k)
+
+
+@pytest.mark.parametrize("n,per_event", [(12000, 0.3), (30000, 0.2), (700, 0.9), (33, 0.5)])
+def test_thousands_of_births_per_event(n, per_event):
+    # ids follow the parents' order, whichever block appends a birth
+    def recipe(L):
+        a = L.add_species(1e-12, n)
+        c = L.add_species(0.0, 10)
+        L.add_reaction([a], [a, c], -np.log(1.0 - per_event) / TAU)
+
+    g, o = build_both((64, 60, 64), recipe, 77)
+    for k in (1, 3, 4):
+        g.run_events(k)
+        o.run_events(k)
+        assert_same(g, o, k)
