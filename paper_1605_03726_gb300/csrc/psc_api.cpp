@@ -214,10 +214,17 @@ bool sorted_order_pays(const psc_lattice* L, int x)
 
 // Lists come from the placement in no order: the first sort of list s is due
 // at its first event, not a period later (1.23M walkers at 30 %: 33 us per
-// event before it, 21 after).
+// event before it, 21 after).  It takes as long as a few events gain: calls of fewer
+// put it off.
+constexpr int64_t kSortFirst = 8;
+static bool first_sort_due(const psc_lattice* L, int s)
+{
+    return L->placed_order[s] && (L->ahead >= kSortFirst || L->since_resort[s] >= (uint64_t)kSortFirst);
+}
+
 int sort_first(psc_lattice* L, int s)
 {
-    if (L->placed_order[s] && L->opt.resort_period > 0) {
+    if (L->opt.resort_period > 0 && first_sort_due(L, s)) {
         L->placed_order[s] = false;
         if (sorted_order_pays(L, s)) return resort(L, s);
     }
@@ -966,6 +973,7 @@ int small_args(psc_lattice* L, SmallArgs* A)
 {
     auto& B = L->small;
     if (!B.cells_hold) {
+        L->waited = 0;
         launch_cells_build(B.cell, L->bits, L->mirror_n, L->labels.empty() ? 1 : L->ncomp, L->model_d, L->sc->counts,
                            L->nsp, L->geo, L->sm_count * 8, L->stream);
         L->launches += 2;
@@ -1181,10 +1189,11 @@ static int walk_stretch(psc_lattice* L, int s, double t, double t_end, int64_t m
     for (int e = 0; e < A.n_events; ++e) A.seq[e] = (uint8_t)place[A.seq[e]];
     int rc = PSC_OK;
     for (int x = 0; x < L->nsp; ++x) {
-        if (!used[x] || !L->placed_order[x] || !walk_sorts(L, x)) continue;
+        if (!used[x] || !first_sort_due(L, x) || !walk_sorts(L, x)) continue;
         if ((rc = resort(L, x))) return rc;
     }
     if (words) {
+        L->waited = 0;
         launch_walk_words(L->claim, L->claim_vacancy ? nullptr : L->bits, L->mirror_n, L->sm_count * 8, L->stream);
         L->launches += 1;
         L->claim_vacancy = true;
@@ -2136,12 +2145,38 @@ static int graph_run(psc_lattice* L, double t_end, int64_t room, int64_t* done)
     return PSC_OK;
 }
 
+// Events of a call up to t_end, at most max_events (an estimate).
+static int64_t events_ahead(const psc_lattice* L, double t_end, int64_t max_events)
+{
+    double n = 0.0;
+    for (int s = 0; s < L->nsp && t_end < INFINITY; ++s)
+        if (L->sp[s].D > 0.0) n += std::max(0.0, std::floor(t_end / L->sp[s].tau) - (double)L->sp[s].done);
+    return t_end < INFINITY && n < (double)max_events ? (int64_t)n : max_events;
+}
+
+// Stretches of large lattices start with a pass over the voxels, their first ones with
+// an allocation too: 100 us at 400^3 for k_walk_run, 280 for k_small_run, as long as 15
+// and 30 events of short lists in the other kernels (events of lists of a million gain
+// twice as much).  Calls with fewer events than these stay there, until as many have run so.
+// us of a first call of 1 / 5 events on 400^3, with the pass / put off: 100,000 walkers
+// 143 / 170, 34 / 82; A + B -> C of 1000 molecules each 320 / 330, 38 / 119.
+static bool pass_pays(const psc_lattice* L, int64_t events)
+{
+    int64_t longest = 0;
+    for (int s = 0; s < L->nsp; ++s)
+        if (L->sp[s].D > 0.0) longest = std::max<int64_t>(longest, L->est[s]);
+    return L->ahead >= events * (1 << 20) / ((1 << 20) + longest) - L->waited;
+}
+
 // Queue events in scheduler order until max_events are queued or the next
 // event lies after t_end.  Consecutive events of one species without
 // reactions are grouped into persistent stretches (cut at re-sort points).
 int drive(psc_lattice* L, double t_end, int64_t max_events)
 {
     int64_t queued = 0;
+    L->ahead = events_ahead(L, t_end, max_events);
+    const bool walks = L->claim_vacancy || L->V <= kWalkVoxels || pass_pays(L, L->V >> 22);
+    const bool smalls = L->small.cells_hold || L->V <= (1ll << 22) || pass_pays(L, L->V >> 21);
     while (queued < max_events) {
         int s;
         double t;
@@ -2173,7 +2208,8 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             queued += e;
             continue;
         }
-        if (walk_fits(L, s)) {
+        const bool walk = walk_fits(L, s);
+        if (walk && walks) {
             int64_t e = 0;
             if (int rc = grid_current(L, true)) return rc;
             int rc = walk_stretch(L, s, t, t_end, max_events - queued, &e);
@@ -2182,13 +2218,16 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             continue;
         }
         if (int rc = claims_free(L)) return rc;
-        if (small_fits(L)) {
+        const bool small = small_fits(L);
+        if (small && smalls) {
             int64_t e = 0;
             int rc = small_stretch(L, s, t, t_end, max_events - queued, &e);
             if (rc) return rc;
             queued += e;
             if (e > 0) continue;
         }
+        const bool waits = (walk && !walks) || (small && !smalls);
+        if (waits) L->waited++;
         if (int rc = grid_current(L, true)) return rc;
         int threads = 0, blocks = 0;
         const bool open = open_route(L, s);
@@ -2225,6 +2264,7 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
             L->g = g0 + (uint32_t)e;
             if (rc) return rc;
             queued += e;
+            if (waits) L->waited += e - 1;
             if (tiles) continue;
             L->since_resort[s] += (uint64_t)e;
             if (L->opt.resort_period > 0 && L->since_resort[s] >= (uint64_t)L->opt.resort_period) {
@@ -2236,6 +2276,15 @@ int drive(psc_lattice* L, double t_end, int64_t max_events)
                     if (rc) return rc;
                 }
             }
+            continue;
+        }
+        if (waits) {                                 // (nor are graphs captured for these few)
+            int rc = enqueue_event(L, s);
+            L->sp[s].done++;
+            L->g++;
+            L->clock = t;
+            if (rc) return rc;
+            ++queued;
             continue;
         }
         if (L->opt.graph_events > 1) {

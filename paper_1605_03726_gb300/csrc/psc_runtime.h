@@ -132,6 +132,8 @@ struct psc_lattice {
     bool claim_vacancy = false;        // the claim words tell vacancy (else all free between events)
     uint32_t walk_epoch = 0;           // of the last event that claimed in them
     int walk_cluster = 0, walk_smem = 0;       // blocks of a cluster, shared memory of a block (0: none)
+    int64_t ahead = 0;                 // events of the running call (an estimate)
+    int64_t waited = 0;                // events run elsewhere since a stretch was last given up or put off
     bool shapes_known = false;         // the device was asked for these and for small.cluster, small.grid
     bool stretches = true;             // false: made for a batch, no room for tombstones is kept
     int64_t list_slack = 0;            // entries of room for tombstones in the lists of reaction products

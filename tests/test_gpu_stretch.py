@@ -201,3 +201,33 @@ def test_thousands_of_births_per_event(n, per_event):
         g.run_events(k)
         o.run_events(k)
         assert_same(g, o, k)
+
+
+@pytest.mark.parametrize("shape,recipe", [
+    ((320, 304, 300), lambda L: L.add_species(1e-12, 20000)),
+    ((200, 192, 180), lambda L: models.reaction_diffusion_ab(L, 3000, 3000)),
+    ((200, 192, 180), lambda L: [models.reaction_diffusion_ab(L, 3000, 3000), L.add_species(1e-12, 50000)]),
+    ((96, 92, 88), lambda L: L.add_species(1e-12, 230000))])
+def test_first_calls_of_few_events(shape, recipe):
+    # large lattices put stretches off, long lists their first sort, until enough events
+    # are ahead: the same lattice whatever the calls
+    arms = []
+    for calls in ((1,) * 14 + (3, 22, 1), (40,), None):
+        L = psc.Lattice(*shape, voxel_radius=1e-8)
+        recipe(L)
+        L.populate(9)
+        if calls:
+            for n in calls:
+                L.run_events(n)
+        else:
+            t = L.tau(0)
+            while L.event_index() < 40:
+                L.run(min(L.time() + 0.6 * t, 1.0))
+            if L.event_index() > 40:
+                L.close()
+                continue
+        arms.append([L.grid()] + [L.unwrapped(s)[0] for s in range(L.n_species)])
+        L.close()
+    for arm in arms[1:]:
+        for a, b in zip(arms[0], arm):
+            assert np.array_equal(a, b)
