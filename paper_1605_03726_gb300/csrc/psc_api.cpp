@@ -1590,10 +1590,16 @@ static int populate(psc_lattice* L, uint64_t seed, bool spare)
     bool stretch = L->stretches && L->V <= kCellVoxels && L->opt.subvolume <= 0;
     for (int s = 0; s < L->nsp; ++s)
         stretch = stretch && (!(L->sp[s].D > 0.0) || L->sp[s].n0 <= (L->nrx > 0 ? kSmallList : kSmallWalk));
+    // with stretches off their words pay only where they fit in the L2 cache or the lists
+    // are short (400^3, A + B -> C of 1.0M each 121 us per event in tables, 139 in words; of
+    // 100,000 26 and 23)
+    int64_t longest = 0;
+    for (int s = 0; s < L->nsp; ++s) longest = std::max<int64_t>(longest, L->sp[s].D > 0.0 ? L->sp[s].n0 : 0);
+    const bool others = L->opt.persistent > 0 || L->V <= kWalkVoxels || longest <= kSmallWalk;
     // (k_walk_run orders them as the mirror's bits, whole bricks)
     const int64_t claim_n = std::max<int64_t>(L->V, L->walk_only ? (int64_t)nwords * 32 : 0);
     L->spare_claims = !direct && spare &&
-                      (open || stretch || (walk && (L->stretches || L->V <= kWalkVoxels)));
+                      (open || (others && (stretch || (walk && (L->stretches || L->V <= kWalkVoxels)))));
     if (L->spare_claims) {
         L->claim_n = claim_n;
         L->claim = (uint32_t*)dev_alloc(L, (size_t)claim_n * sizeof(uint32_t));
