@@ -845,6 +845,7 @@ static int small_setup(psc_lattice* L)
     for (int s = 0; s < L->nsp; ++s) {
         if (L->general[s]) B.general |= 1u << s;
         if (L->fo2[s]) B.fo2 |= 1u << s;
+        for (int x : L->reconcile[s]) B.closes[s] |= 1u << x;
         auto products = [&](const Reaction& R) {
             for (int q = 0; q < R.np; ++q) B.products[s] |= 1u << R.p[q];
         };
@@ -957,6 +958,7 @@ int small_buffers(psc_lattice* L, bool scratch)
     }
     // (a list that has doubled since wants more)
     if (scratch && B.general && (!B.scratch || (int64_t)small_scratch(L) > 2 * (int64_t)B.scratch_n)) {
+        B.version++;
         if (B.scratch) dev_free_one(L, B.scratch);
         B.scratch_n = small_scratch(L);
         B.scratch = (int32_t*)dev_alloc(L, (size_t)B.scratch_n * 8);
@@ -2599,6 +2601,7 @@ int psc_set_options(psc_lattice* L, const psc_options* o)
     graph_cache_clear(L);                            // captured launches follow the options
     std::memset(L->open_auto, 0, sizeof(L->open_auto));
     L->small.no_room = false;
+    L->small.version++;
     if (o->resort_period) L->opt.resort_period = o->resort_period;
     if (o->block_threads) L->opt.block_threads = o->block_threads;
     if (o->blocks_per_sm) L->opt.blocks_per_sm = o->blocks_per_sm;

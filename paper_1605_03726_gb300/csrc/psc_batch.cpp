@@ -26,10 +26,14 @@ constexpr int kItemThreadsDefault = 256;   // threads per block of the batched l
 struct Member {
     psc_lattice* L = nullptr;
     double t_stop = INFINITY;             // run events up to this time
+    uint32_t args = 0;                    // SmallBuffers::version of what args_d holds of it (0: nothing)
     bool stretch = false;                 // runs in stretches (else in batched launches per event phase)
 };
 
 }  // namespace
+
+constexpr int kNarrow = 2;
+constexpr int kNarrowThreads[kNarrow] = {kSmallThreads / 2, kSmallThreads / 4};
 
 struct psc_batch {
     int device = 0;
@@ -45,9 +49,9 @@ struct psc_batch {
     int32_t resort_period = -1;           // events of a member's species between Morton re-sorts (-1 never)
     // stretches of the members' events, one launch for many members
     int stretch_blocks = -1;              // most blocks of a launch (-1: not asked, 0: no stretches)
+    int narrow_blocks[kNarrow][2] = {};   // of fewer threads; without and with births
     bool use_stretches = true;
     SmallArgs* args_d = nullptr;          // [kBatchMax], device: a member's, but for its events
-    std::vector<SmallArgs> args_h;        // as last copied there
     char* upload_d = nullptr;             // stretches, blocks' groups and events of a call
     int32_t* counts_d = nullptr;          // [kBatchMax][kSmallCounts] list lengths after a stretch
     int32_t* counts_h = nullptr;          // pinned copy, for the next stretch's groups
@@ -233,10 +237,16 @@ int stretch_launches(int total, int blocks, double bytes, double molecules)
 
 int stretch_buffers(psc_batch* B, psc_lattice* L)
 {
-    if (B->stretch_blocks < 0) B->stretch_blocks = small_batch_blocks(L->sm_count);
+    if (B->stretch_blocks < 0) {
+        B->stretch_blocks = small_batch_blocks(L->sm_count, kSmallThreads, true);
+        for (int w = 0; w < kNarrow; ++w)
+            for (int births = 0; births < 2; ++births)
+                B->narrow_blocks[w][births] = small_batch_blocks(L->sm_count, kNarrowThreads[w], births != 0);
+    }
     if (B->stretch_blocks == 0 || B->args_d) return PSC_OK;
     if (cudaMalloc(&B->args_d, sizeof(SmallArgs) * kBatchMax) != cudaSuccess ||
-        cudaMalloc(&B->upload_d, upload_bytes(B->stretch_blocks)) != cudaSuccess ||
+        cudaMalloc(&B->upload_d, upload_bytes(std::max({B->stretch_blocks, B->narrow_blocks[0][0],
+                                                        B->narrow_blocks[kNarrow - 1][0]}))) != cudaSuccess ||
         cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
@@ -316,7 +326,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
     std::vector<double> work;             // molecules per event, entries looked through at the end among them
     std::vector<std::pair<psc_lattice*, uint32_t>> of;
     bool births = false;
-    B->args_h.resize(kBatchMax);
+    SmallArgs A{};
     for (int i = 0; i < kBatchMax; ++i) {
         psc_lattice* L = B->slot[i].L;
         if (!L || L->sticky || !B->slot[i].stretch) continue;
@@ -328,16 +338,16 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         double t;
         if (!next_event(L, &s, &t) || t > B->slot[i].t_stop || t > t_cap || L->g == UINT32_MAX) continue;
         if ((*rc_out = claims_free(L))) return 1;
-        SmallArgs A{};
-        if ((*rc_out = small_args(L, &A))) return 1;
-        constexpr size_t fixed = offsetof(SmallArgs, seq);
-        if (std::memcmp(&A, &B->args_h[(size_t)i], fixed) != 0) {
-            if (cudaMemcpyAsync(B->args_d + i, &A, fixed, cudaMemcpyHostToDevice, B->stream) != cudaSuccess) {
+        if (!L->small.cells_hold || B->slot[i].args != L->small.version) {
+            if ((*rc_out = small_args(L, &A))) return 1;
+            if (cudaMemcpyAsync(B->args_d + i, &A, offsetof(SmallArgs, seq), cudaMemcpyHostToDevice, B->stream) !=
+                cudaSuccess) {
                 *rc_out = PSC_E_CUDA;
                 return 1;
             }
-            std::memcpy(&B->args_h[(size_t)i], &A, fixed);
+            B->slot[i].args = L->small.version;
         }
+        L->small.grid_stale = true;
         SmallStretch x{};
         x.slot = i;
         x.g = L->g;
@@ -349,16 +359,15 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
             seq.push_back((uint8_t)s);
             x.n_events++;
             molecules += (double)L->est[s];
-            for (int q : L->reconcile[s]) may_close |= 1u << q;
+            may_close |= L->small.closes[s];
             L->sp[s].done++;
             L->g++;
             L->clock = t;
         } while (x.n_events < limit && next_event(L, &s, &t) && t <= B->slot[i].t_stop && t <= t_cap);
-        births = births || A.fo2 != 0u;
+        births = births || L->small.fo2 != 0u;
         L->events += (uint64_t)x.n_events;
         L->launches += 1;
-        for (int q = 0; q < L->nsp; ++q)
-            if ((may_close >> q) & 1u) closed += (double)L->est[q];
+        for (; may_close != 0; may_close &= may_close - 1) closed += (double)L->est[__builtin_ctz(may_close)];
         work.push_back((molecules + 0.25 * closed) / x.n_events);
         stretch.push_back(x);
         of.emplace_back(L, L->g);
@@ -371,7 +380,20 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         bytes += 128.0 * (double)of[(size_t)r].first->mirror_n;
         molecules += work[(size_t)r];
     }
-    const int launches = stretch_launches(total, B->stretch_blocks, bytes, molecules);
+    int blocks_most = B->stretch_blocks, threads = kSmallThreads;
+    int launches = stretch_launches(total, blocks_most, bytes, molecules);
+    // more members than blocks: narrower blocks, several on an SM, as long as their
+    // threads hold the molecules of an event (500 members of 400 molecules on 24^3, calls of
+    // 1 / 64 events: 64 / 19.7 us per event in launches one after the other, 27 / 9.6 so)
+    for (int w = 0; w < kNarrow; ++w) {
+        const int narrow = B->narrow_blocks[w][births ? 1 : 0];
+        if (total <= B->stretch_blocks || narrow <= blocks_most || molecules > 2.0 * kNarrowThreads[w] * total ||
+            (total + narrow - 1) / narrow >= launches)
+            continue;
+        blocks_most = narrow;
+        threads = kNarrowThreads[w];
+        launches = (total + narrow - 1) / narrow;
+    }
     std::vector<int32_t> group;           // of all launches' blocks
     std::vector<int> first;               // block of each launch
     for (int l = 0; l < launches; ++l) {
@@ -380,11 +402,11 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         // with 600 per block
         double sum = 0.0;
         for (int r = lo; r < hi; ++r) sum += work[(size_t)r] + 600.0;
-        const int spare = B->stretch_blocks - (hi - lo);
+        const int spare = blocks_most - (hi - lo);
         first.push_back((int)group.size());
         for (int r = lo; r < hi; ++r) {
             const int more = (int)(spare * (work[(size_t)r] + 600.0) / sum);
-            const int most = (int)(work[(size_t)r] / kSmallThreads);           // with it, a molecule per thread
+            const int most = (int)(work[(size_t)r] / threads);           // with it, a molecule per thread
             stretch[(size_t)r].blocks = 1 + std::min(more, most);
             stretch[(size_t)r].block0 = (int)group.size() - first.back();
             group.insert(group.end(), (size_t)stretch[(size_t)r].blocks, r);
@@ -405,7 +427,7 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
         if (launch_small_batch(B->args_d, (const SmallStretch*)B->upload_d,
                                (const int32_t*)(B->upload_d + at_group) + first[(size_t)l],
                                (const uint8_t*)B->upload_d + at_seq, B->counts_d,
-                               first[(size_t)l + 1] - first[(size_t)l], births, B->stream) != cudaSuccess) {
+                               first[(size_t)l + 1] - first[(size_t)l], threads, births, B->stream) != cudaSuccess) {
             *rc_out = PSC_E_CUDA;
             return total;
         }
@@ -476,6 +498,7 @@ int batch_add_until(psc_batch* B, psc_lattice* L, double t_stop, int64_t room, i
     B->slot[free_slot].L = L;
     B->slot[free_slot].t_stop = t_stop;
     B->slot[free_slot].stretch = stretch;
+    B->slot[free_slot].args = 0;
     B->size++;
     return PSC_OK;
 }

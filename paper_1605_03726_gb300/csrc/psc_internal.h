@@ -500,9 +500,10 @@ void launch_cells_grid(const uint32_t* cell, uint32_t* bits0, uint64_t words, in
 // stretches of many lattices in one launch of `blocks` blocks: per block the
 // stretch it belongs to, species of all their events; stretch r leaves list
 // lengths in counts + r * kSmallCounts (all on the device)
-int small_batch_blocks(int sm_count);       // most blocks on the current device (0: not at all)
+int small_batch_blocks(int sm_count, int threads, bool births);    // most blocks on the current device (0: not at all)
 cudaError_t launch_small_batch(const SmallArgs* args, const SmallStretch* stretch, const int32_t* group,
-                               const uint8_t* seq, int32_t* counts, int blocks, bool births, cudaStream_t st);
+                               const uint8_t* seq, int32_t* counts, int blocks, int threads, bool births,
+                               cudaStream_t st);
 cudaError_t launch_small(const SmallArgs& A, int blocks, int threads, bool cluster, cudaStream_t st);
 void launch_fill_u32(uint32_t* p, uint32_t value, size_t n, int blocks, cudaStream_t st);
 // molecule r (ids in species order, species s owning [offsets[s],

@@ -114,6 +114,7 @@ struct psc_lattice {
         EventArgs* ev = nullptr;       // allocated by the first stretch where the lattice's block has none
         bool ev_set = false;           // written, by the first stretch
         uint32_t* cell = nullptr;      // the cells, as ev
+        uint32_t version = 1;          // of what small_args writes: a step with every change of it
         bool barrier_set = false;      // the barrier word was zeroed once
         bool no_room = false;          // no memory for these: stretches are off until options are set
         int32_t* scratch = nullptr;    // 2 x scratch_n, for stretches that take a grid
@@ -123,6 +124,7 @@ struct psc_lattice {
         int cluster = 0, grid = 0;     // most blocks of a stretch: one cluster, a cooperative grid
         uint32_t general = 0, fo2 = 0;
         uint32_t products[kMaxSpecies] = {};
+        uint32_t closes[kMaxSpecies] = {};         // lists an event of the species may take entries off
     } small;
     // lattices without reactions (k_walk_run)
     bool walk_only = false;            // no reactions, no compartments

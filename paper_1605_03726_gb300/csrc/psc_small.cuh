@@ -783,23 +783,24 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_batch(const SmallArg
     }
 }
 
-int small_batch_blocks(int sm_count)
+int small_batch_blocks(int sm_count, int threads, bool births)
 {
     const void* f = (const void*)k_small_batch;
     const int smem = kBirthSortMax * (int)sizeof(unsigned long long);
     int per_sm = 0;
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kSmallThreads, smem) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, births ? smem : 0) != cudaSuccess)
         per_sm = 0;
     cudaGetLastError();
     return per_sm * sm_count;
 }
 
 cudaError_t launch_small_batch(const SmallArgs* args, const SmallStretch* stretch, const int32_t* group,
-                               const uint8_t* seq, int32_t* counts, int blocks, bool births, cudaStream_t st)
+                               const uint8_t* seq, int32_t* counts, int blocks, int threads, bool births,
+                               cudaStream_t st)
 {
     void* p[] = {&args, &stretch, &group, &seq, &counts};
-    return cudaLaunchCooperativeKernel((const void*)k_small_batch, dim3(blocks), dim3(kSmallThreads), p,
+    return cudaLaunchCooperativeKernel((const void*)k_small_batch, dim3(blocks), dim3(threads), p,
                                        births ? (size_t)kBirthSortMax * sizeof(unsigned long long) : 0, st);
 }
 

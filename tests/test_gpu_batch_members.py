@@ -163,3 +163,38 @@ def test_members_take_turns_where_their_cells_exceed_the_cache():
         assert np.array_equal(members[r].unwrapped(0)[0], solo.unwrapped(0)[0])
         solo.close()
     B.close()
+
+
+@pytest.mark.parametrize("members,n,births", [(153, 500, False), (310, 150, False), (310, 150, True)])
+def test_more_members_than_blocks(members, n, births):
+    # narrower blocks, two or four on an SM; options of a member changed on the way
+    import torch
+    stream = torch.cuda.Stream().cuda_stream
+
+    def member(r, stream):
+        L = psc.Lattice(20 + 2 * (r % 3), 20, 22, voxel_radius=1e-8, stream=stream)
+        L.set_options(claim_table=1, resort_period=-1)
+        a = L.add_species(1e-12, n)
+        b = L.add_species(0.8e-12, n // 2)
+        c = L.add_species(0.0, 5)
+        L.add_reaction([a, b], [c, b], 1e-19)
+        L.add_reaction([b], [a, b] if births else [a], 0.01 / TAU)
+        L.populate(r)
+        return L
+
+    B = psc.Batch(stream=stream)
+    Ls = [member(r, stream) for r in range(members)]
+    for L in Ls:
+        B.add(L)
+    for k in (1, 3, 60, 1):
+        B.run_events(k)
+        Ls[7].set_options(collect_stats=1)
+    for r in range(0, members, members // 9):
+        solo = member(r, None)
+        solo.run_events(65)
+        assert np.array_equal(Ls[r].grid(), solo.grid()) and np.array_equal(Ls[r].counts(), solo.counts())
+        for s in range(3):
+            assert np.array_equal(Ls[r].unwrapped(s)[0], solo.unwrapped(s)[0])
+        solo.close()
+    assert Ls[7].stats()["attempts"] > 0
+    B.close()
