@@ -1038,9 +1038,11 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
                                             (int64_t)UINT32_MAX - L->g);
     A.g = L->g;
     int64_t longest = 0, closed = 0;                 // lists of due species; lists that may be closed up
+    double spare = 0.0;                              // events that a cluster makes faster, less for longer lists
     do {
         A.seq[A.n_events++] = (uint8_t)s;
         longest = std::max(longest, L->est[s]);
+        spare += std::max(0.0, 1.0 - (double)L->est[s] / (double)kSmallCluster);
         for (int x : L->reconcile[s]) closed = std::max(closed, L->est[x]);
         L->sp[s].done++;
         L->g++;
@@ -1052,9 +1054,8 @@ static int small_stretch(psc_lattice* L, int s, double t, double t_end, int64_t 
     // closing up the lists would take longer than the cluster spares; then a block
     // per SM, of half the threads while they suffice
     // (a cluster's hardware barrier knows no phantoms)
-    const double spare = (double)A.n_events * std::max(0.0, 1.0 - (double)longest / (double)kSmallCluster);
     bool cluster = longest <= kSmallCluster && L->opt.barrier_phantom <= 0;
-    if (cluster && (double)closed > kSmallClosed * (1.0 + spare)) {
+    if (cluster && (double)closed > kSmallClosed + kSmallClosedEvent * spare) {
         rc = small_buffers(L, true);
         if (rc == PSC_E_NOMEM) L->sticky = sticky;   // (no scratch: in a cluster all the same)
         else if (rc) return rc;

@@ -296,12 +296,12 @@ constexpr double kSmallRun = 1.5e6, kSmallRunLarge = 1e6, kSmallRunDense = 3.0, 
 constexpr int64_t kSmallCluster = 16384;
 // There one block closes up a list, 1.2 us for 1000 entries; a grid does it together.
 // An event of few molecules is 2 us faster in a cluster: a stretch of few events
-// with longer lists to close up than this, and as much more for each event (less for
-// longer lists, which gain less), runs in a grid.  us per call of one event, in a
+// with lists to close up longer than kSmallClosed, and kSmallClosedEvent for each event
+// (less for longer due lists, which gain less), runs in a grid.  us per call of one event, in a
 // cluster / in a grid (launches per event phase): 2000 A meeting 2000 B on 64^3 25 / -
 // (33), 15,000 and 15,000 49 / 29 (34), 2000 and 200,000 immobile ones on 128^3 294 / 29
 // (33), 2000 and 4 million on 256^3 8470 / 37 (46).
-constexpr double kSmallClosed = 2048.0;
+constexpr double kSmallClosed = 2048.0, kSmallClosedEvent = 2500.0;
 struct SmallArgs {
     const EventArgs* ev;       // [nsp] templates on the device (event_args with g unset)
     const ModelDev* model;
