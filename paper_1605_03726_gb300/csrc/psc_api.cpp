@@ -2420,7 +2420,7 @@ static int device_positions(psc_lattice* L, int32_t s, int64_t n, bool unwrapped
 {
     const bool by_id = !L->live[s] && n == L->sp[s].n0;
     if (n <= 0 || (n > L->rs_max && !by_id)) return 1;
-    // the list passes' scratch, 32 bytes per entry of the longest list
+    // the list passes' scratch, 24 bytes per entry of the longest list (16 are used)
     int32_t* pos = L->tmp.vox;
     uint32_t* ids = reinterpret_cast<uint32_t*>(pos + 3 * n);
     const int blocks = event_blocks(L, n);

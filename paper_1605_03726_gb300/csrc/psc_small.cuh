@@ -25,7 +25,7 @@
 //     are closed up at the end of the stretch, or when one could run out of
 //     room.
 // Births need a pass of their own (ids in parent order) in events that have
-// any.
+// any: a rank for each among the parents, by all blocks (small_births).
 //
 // One block of 512 threads per SM: the events need about 110 registers (two
 // blocks per SM spilled: crowded 256^3 30.1 us per event against 25.3), and two
@@ -33,7 +33,7 @@
 //
 // Measured (us per event; before: claim, commit, list check and fill launches
 // replayed from CUDA graphs, or the molecule-list kernel for walkers): A + B -> C
-// of 2000 + 2000 molecules on 64^3 12.5 -> 4.2, a cascade of 22 species of up to
+// of 2000 + 2000 molecules on 64^3 12.5 -> 4.1, a cascade of 22 species of up to
 // 16,000 molecules on 200^3 10.5 -> 3.1, 30,000 ligands and 5000 receptors in a
 // cell on 128^3 19.8 -> 6.2, reversible A + B <-> C under 30 % crowding with 839,000
 // A on 256^3 40.0 -> 24.6, with 1.6M on 320^3 92 -> 48, with 3.2M on 400^3
@@ -41,7 +41,10 @@
 // the barrier that ends an event (the first 4.2 -> 4.5, the second 3.1 -> 3.7: every
 // thread's extra instructions cost more than the load they hide); molecules kept in
 // shared memory between the phases (crowded 256^3 26.1).  The order of a list makes
-// no difference here (26.3 sorted on 256^3), so these stretches have no re-sorts.
+// little difference: two species of 400,000 on 256^3 22.6 us per event as placed, 22.2
+// sorted, of 1.0M on 400^3, whose cells do not fit in the L2 cache, 81.0 and 82.6, 64 members
+// of 160^3 at 2 % 182 and 182; only the longest gain (3.2M on 400^3 243 and 204).  So these
+// stretches have no re-sorts.
 
 // Event arguments and model of the lattice, copied to shared memory once per
 // launch: after a barrier a load of them from global memory would go to L2.
