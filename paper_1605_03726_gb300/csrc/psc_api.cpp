@@ -1616,14 +1616,6 @@ static int populate(psc_lattice* L, uint64_t seed, bool spare)
         L->table_slots = (int64_t)1 << hb_max;
         for (int t = 0; t < 2; ++t) carve.add(&L->tables[t], ((size_t)1 << hb_max) * sizeof(uint64_t));
     }
-    // reactions on lattices of up to 2^22 voxels run in stretches: their templates and
-    // cells come with the block (16 MB at most), so that events allocate nothing
-    bool general = false;
-    for (int s = 0; s < L->nsp; ++s) general = general || L->general[s];
-    if (general && stretch && direct && L->opt.persistent > 0 && L->V <= (1ll << 22)) {
-        carve.add(&L->small.ev, sizeof(EventArgs) * (size_t)L->nsp);
-        carve.add(&L->small.cell, nwords * 128);
-    }
     for (int s = 0; s < L->nsp; ++s) {
         SpeciesList& l = M.lists[s];
         l.cap = L->cap[s] + (is_product[s] ? (int32_t)L->list_slack : 0);
@@ -1806,6 +1798,15 @@ static int populate(psc_lattice* L, uint64_t seed, bool spare)
         dev_free_one(L, labels_d);
     }
     if (N == 0 && (rc = cuda_fail(L, cudaStreamSynchronize(st)))) return rc;     // (else the placement waited)
+    // reactions on lattices of up to 2^22 voxels run in stretches: their templates and
+    // cells come with the lattice (16 MB at most), so that events allocate nothing
+    bool reacts = false;
+    for (int s = 0; s < L->nsp; ++s) reacts = reacts || L->general[s];
+    if (reacts && stretch && direct && L->opt.persistent > 0 && L->V <= (1ll << 22)) {
+        L->small.ev = (EventArgs*)dev_alloc(L, sizeof(EventArgs) * (size_t)L->nsp);
+        L->small.cell = (uint32_t*)dev_alloc(L, nwords * 128);
+        if (!L->small.ev || !L->small.cell) return PSC_E_NOMEM;
+    }
     L->g = 0;
     L->clock = 0.0;
     L->populated = true;

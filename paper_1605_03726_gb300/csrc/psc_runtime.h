@@ -111,7 +111,7 @@ struct psc_lattice {
     // stretches of events in one launch (k_small_run): per-species argument
     // templates on the device, a cell per voxel and the scratch of closing lists up
     struct SmallBuffers {
-        EventArgs* ev = nullptr;       // allocated by the first stretch where the lattice's block has none
+        EventArgs* ev = nullptr;       // allocated with the lattice, a large one's by the first stretch
         bool ev_set = false;           // written, by the first stretch
         uint32_t* cell = nullptr;      // the cells, as ev
         uint32_t version = 1;          // of what small_args writes: a step with every change of it
