@@ -33,6 +33,7 @@ struct Member {
 }  // namespace
 
 constexpr int kNarrow = 2;
+constexpr int kNarrowMost = 8;             // times stretch_blocks, at most
 constexpr int kNarrowThreads[kNarrow] = {kSmallThreads / 2, kSmallThreads / 4};
 
 struct psc_batch {
@@ -49,7 +50,8 @@ struct psc_batch {
     int32_t resort_period = -1;           // events of a member's species between Morton re-sorts (-1 never)
     // stretches of the members' events, one launch for many members
     int stretch_blocks = -1;              // most blocks of a launch (-1: not asked, 0: no stretches)
-    int narrow_blocks[kNarrow][2] = {};   // of fewer threads; without and with births
+    int narrow_blocks[kNarrow][2] = {{-1, -1}, {-1, -1}};       // of fewer threads; without and with births
+    int sm_count = 0;
     bool use_stretches = true;
     SmallArgs* args_d = nullptr;          // [kBatchMax], device: a member's, but for its events
     char* upload_d = nullptr;             // stretches, blocks' groups and events of a call
@@ -237,16 +239,11 @@ int stretch_launches(int total, int blocks, double bytes, double molecules)
 
 int stretch_buffers(psc_batch* B, psc_lattice* L)
 {
-    if (B->stretch_blocks < 0) {
-        B->stretch_blocks = small_batch_blocks(L->sm_count, kSmallThreads, true);
-        for (int w = 0; w < kNarrow; ++w)
-            for (int births = 0; births < 2; ++births)
-                B->narrow_blocks[w][births] = small_batch_blocks(L->sm_count, kNarrowThreads[w], births != 0);
-    }
+    if (B->stretch_blocks < 0) B->stretch_blocks = small_batch_blocks(L->sm_count, kSmallThreads, true);
+    B->sm_count = L->sm_count;
     if (B->stretch_blocks == 0 || B->args_d) return PSC_OK;
     if (cudaMalloc(&B->args_d, sizeof(SmallArgs) * kBatchMax) != cudaSuccess ||
-        cudaMalloc(&B->upload_d, upload_bytes(std::max({B->stretch_blocks, B->narrow_blocks[0][0],
-                                                        B->narrow_blocks[kNarrow - 1][0]}))) != cudaSuccess ||
+        cudaMalloc(&B->upload_d, upload_bytes(kNarrowMost * B->stretch_blocks)) != cudaSuccess ||
         cudaMalloc(&B->counts_d, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaMallocHost(&B->counts_h, sizeof(int32_t) * kBatchMax * kSmallCounts) != cudaSuccess ||
         cudaEventCreateWithFlags(&B->counts_ev, cudaEventDisableTiming) != cudaSuccess) {
@@ -285,12 +282,13 @@ int member_stretches(psc_batch* B, psc_lattice* L, int64_t room, int64_t* extra,
     return PSC_OK;
 }
 
-// A copy of the members' list lengths every so many events, and the age at
-// which the host waits for one.  (Waited for by every call, with two copies up
+// A copy of the members' list lengths every so many events; the host waits for it
+// when the call would take its age to that number (the groups of a long call follow
+// the lengths after the one before: served replicas whose lists fall from step to step
+// took 4 % longer with older ones).  Waited for by every call, with two copies up
 // and a memset in every launch, run_events(1) took 52 us of 64 A + B -> C members on 48^3
-// and 133 of 300 on 32^3; now 27 and 40; in launches
-// per event phase 38 and 55.)
-constexpr int64_t kCountsEvery = 64, kCountsWait = 256;
+// and 133 of 300 on 32^3; now 27 and 40; in launches per event phase 38 and 55.
+constexpr int64_t kCountsEvery = 64;
 
 // Up to n_events next events of every member that runs in stretches, up to
 // its t_stop and t_cap; the number of members that had any.
@@ -298,10 +296,8 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
 {
     *rc_out = PSC_OK;
     if (!B->use_stretches || B->stretch_blocks <= 0) return 0;
-    // list lengths after an earlier stretch: groups follow them.  They come in the
-    // background, and once they are kCountsWait events old the host waits for them
-    // (the device still has as many queued)
-    if (B->counts_pending && (B->counts_age >= kCountsWait || cudaEventQuery(B->counts_ev) == cudaSuccess)) {
+    // list lengths after an earlier stretch: groups follow them
+    if (B->counts_pending && (B->counts_age + n_events >= kCountsEvery || cudaEventQuery(B->counts_ev) == cudaSuccess)) {
         if (cudaEventSynchronize(B->counts_ev) != cudaSuccess) {
             *rc_out = PSC_E_CUDA;
             return 1;
@@ -385,9 +381,11 @@ int batch_stretch(psc_batch* B, double t_cap, int64_t n_events, int* rc_out)
     // more members than blocks: narrower blocks, several on an SM, as long as their
     // threads hold the molecules of an event (500 members of 400 molecules on 24^3, calls of
     // 1 / 64 events: 64 / 19.7 us per event in launches one after the other, 27 / 9.6 so)
-    for (int w = 0; w < kNarrow; ++w) {
-        const int narrow = B->narrow_blocks[w][births ? 1 : 0];
-        if (total <= B->stretch_blocks || narrow <= blocks_most || molecules > 2.0 * kNarrowThreads[w] * total ||
+    for (int w = 0; w < kNarrow && total > B->stretch_blocks; ++w) {
+        int& narrow = B->narrow_blocks[w][births ? 1 : 0];
+        if (narrow < 0)
+            narrow = std::min(small_batch_blocks(B->sm_count, kNarrowThreads[w], births), kNarrowMost * B->stretch_blocks);
+        if (narrow <= blocks_most || molecules > 2.0 * kNarrowThreads[w] * total ||
             (total + narrow - 1) / narrow >= launches)
             continue;
         blocks_most = narrow;
