@@ -416,9 +416,12 @@ int psc_set_allocator(psc_alloc_fn alloc, psc_free_fn release, void *ctx);
  * Batches: many lattices (replicas, parameter sweeps) advanced together.
  * A launch gives every member a group of blocks for a stretch of its events, at
  * its own pace (up to 512; the members' extra buffers take 4 bytes per voxel, and
- * with reactions 10 to 48 per molecule); members with persistent = -1, with kernel
+ * with reactions 10 to 48 per molecule); members whose voxels exceed the L2 cache
+ * together take turns.  Members with persistent = -1, with kernel
  * timing or without room for the buffers run in launches that cover the next
- * event (its own species and event index) of each.  Results of a member are
+ * event (its own species and event index) of each.  A member with an error (a wait
+ * that ran out, a list that overflowed) gets no further events once the batch has
+ * seen it, with the list lengths it copies every 64 events.  Results of a member are
  * bit-identical to running it alone (same seed, same model).
  *
  *   psc_batch_create   cuda_stream as for psc_lattice_create.
